@@ -523,6 +523,9 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
     p.order = alpha == 4 ? 2 : 1;
     p.planes = alpha == 4 ? 13 : 5;
     for (int d = 0; d <= 4; ++d) p.aC[d] = kappa * kappa + (double)d;
+    p.var64 = 1.0 / gamma;
+    p.aC2_in = p.aC[4] * p.aC[4];
+    p.flC_in = std::max(1e-20 * p.aC2_in, 2.2250738585072014e-308);
     p.var_f = (float)(1.0 / gamma);
     for (int d = 0; d <= 4; ++d) {
         p.aC_f[d] = (float)p.aC[d];
@@ -645,7 +648,7 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
     } else if (o.tile_x) {
         c->shape = {o.tile_x, o.tile_y};
     } else {
-        c->shape = p.prec ? gabp::FusedShape{32, 8} : gabp::FusedShape{64, 16};
+        c->shape = p.prec ? gabp::fused_choose_shape_f64(nx, ny) : gabp::FusedShape{64, 16};
     }
     c->edges = 5 * n - 2 * (int64_t)(nx + ny) + 4 * m;
     if (p.order == 2) {   // 13-slot cell factors: count the slots whose node exists

@@ -37,15 +37,61 @@ template <> __device__ __forceinline__ double pos_inf<double>() {
 
 // Reciprocal.  FP32: the hardware approximation rcp.approx.ftz.f32, within 1 ulp over the
 // range the callers use (they never pass 0, a denormal or an infinity: cavity precisions are
-// floored at a normal number, and V is at least var > 0 and at most about 5e20).  FP64: IEEE
-// division.
-template <typename T> __device__ __forceinline__ T recip(T x);
-template <> __device__ __forceinline__ float recip<float>(float x) {
+// floored at a normal number, and V is at least var > 0 and at most about 5e20).  FP64: below.
+__device__ __forceinline__ float recip(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-template <> __device__ __forceinline__ double recip<double>(double x) { return 1.0 / x; }
+
+// FP64 reciprocal without an FP64 operation.  FP64 is the scarce unit of this GPU (measured: one
+// warp instruction per 64 to 76 cycles and SM quarter, whatever its parallelism), while its integer
+// and FP32 units are nearly idle in the FP64 kernels, so the quotient of the 53-bit significands is
+// formed there, by Newton's method in mixed fixed point:
+//   x = 2^E m, M = 2^52 m;  m = mh + ml with mh its 24-bit rounding;
+//   r = the FP32 approximation of 1 / mh, e = 1 - m r (two exact-product FMAs, |e| <= 1.6 2^-23),
+//   R0 = 2^53 (r + r (e + e^2)), an integer within 2^-46 of the quotient, relatively;
+//   D = 2^105 - M R0, whose low 64 bits hold it (|D| <= 2^60);
+//   R = R0 + round(R0 D / 2^105): within 0.5 + 2^-14 of 2^53 / m, the IEEE quotient but for near ties.
+// 1 / x = 2^(-E - 53) R.  About 35 integer and FP32 instructions in the place of seven FP64 ones of
+// IEEE sequence.  Exponents outside 2^+-1000 (zero, denormal, huge, infinite, NaN) set `out` and leave
+// a meaningless value: the caller divides instead, once for all its reciprocals, so that several
+// of them interleave without a branch (a branch in each made five of them take 1,250 cycles).
+__device__ __forceinline__ double recip_fixed(double x, bool &out) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned ex = (hi >> 20) & 0x7ffu;
+    out |= ex - 23u >= 2000u;
+    const unsigned mhi = (hi & 0xfffffu) | 0x100000u;                 // M = mhi : lo
+    const int tl = (int)(lo << 3) >> 3;                               // M's low 29 bits, signed: ml = 2^-52 tl
+    const float mh = __uint_as_float(0x3f800000u + (((hi << 3) | (lo >> 29)) & 0x7fffffu) + ((lo >> 28) & 1u));
+    const float r = recip(mh);
+    const float e = __fmaf_rn(-0x1p-52f * __int2float_rn(tl), r, __fmaf_rn(-mh, r, 1.f));
+    const unsigned ri = __float2uint_rn(r * 0x1p24f);                 // exact: r in [0.5, 1] has 24 bits
+    const int ci = __float2int_rn(0x1p53f * r * __fmaf_rn(e, e, e));
+    const unsigned long long R0 = ((unsigned long long)ri << 29) + (unsigned long long)(long long)ci;
+    const unsigned rl = (unsigned)R0, rh = (unsigned)(R0 >> 32);
+    // bits 32..63 of M R0; D's upper half is its complement (the dropped carry is 2^-20 of a unit)
+    const int dh = (int)~(__umulhi(lo, rl) + lo * rh + mhi * rl);
+    const long long R = (long long)R0 + __float2int_rn(0x1p-20f * r * __int2float_rn(dh));
+    const unsigned long long bits = ((unsigned long long)(2044u - ex) << 52) + (unsigned long long)R;
+    return __longlong_as_double((long long)(bits | ((unsigned long long)(hi & 0x80000000u) << 32)));
+}
+
+// The reciprocal in the message formulas: FP32 recip(); FP64 recip_fixed() (FAST) or the division.
+template <bool FAST> __device__ __forceinline__ float recip_or(float x, bool &) { return recip(x); }
+template <bool FAST> __device__ __forceinline__ double recip_or(double x, bool &out) {
+    return FAST ? recip_fixed(x, out) : 1.0 / x;
+}
+
+// x == 0 and max(x, f) for f > 0 (f where x is NaN or negative).  FP64: on the bits, in the integer
+// unit (a positive double orders as its bits do).
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.f; }
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ float floor_at(float x, float f) { return fmaxf(x, f); }
+__device__ __forceinline__ double floor_at(double x, double f) {
+    const long long b = __double_as_longlong(x);
+    return b >= __double_as_longlong(f) && b <= 0x7ff0000000000000LL ? x : f;
+}
 
 // Explicitly rounded arithmetic for the message formulas: no multiply is contracted into a
 // fused multiply-add unless written as one, so every kernel (scalar or packed two-lane FP32)
@@ -60,24 +106,37 @@ __device__ __forceinline__ double fma_rn(double a, double b, double c) { return 
 // Two-term compensated sum (TwoSum accumulation, Knuth TAOCP vol. 2 4.2.2): hi + lo carries
 // the running sum to about twice the working precision.  Used for the belief sums so that
 // the cavity (belief minus one message) keeps its relative accuracy even when that message
-// dominates the belief.
+// dominates the belief.  FP64: the same exact error by Fast2Sum (Dekker 1971) on the operands
+// ordered by exponent, three additions instead of six (the ordering runs in the integer unit), and
+// no renormalisation, which the cavity (hi - own) + lo does not need: its error bound is the same.
 template <typename T> struct CompSum {
     T hi, lo;
-    __device__ __forceinline__ CompSum() : hi(T(0)), lo(T(0)) {}
     // start from a first term: identical to adding it to an empty sum (TwoSum(0, x) = (x, 0))
     __device__ __forceinline__ explicit CompSum(T first) : hi(first), lo(T(0)) {}
-    __device__ __forceinline__ void add(T x) {
-        T t = hi + x;
-        T z = t - hi;
-        T e = (hi - (t - z)) + (x - z);
+    // hi += x; returns the rounding error
+    __device__ __forceinline__ T step(T x) {
+        const T t = hi + x;
+        T e;
+        if constexpr (sizeof(T) == 8) {
+            const bool sw = (__double2hiint(x) & 0x7fffffff) > (__double2hiint(hi) & 0x7fffffff);
+            const T big = sw ? x : hi, small = sw ? hi : x;
+            e = small - (t - big);
+        } else {
+            const T z = t - hi;
+            e = (hi - (t - z)) + (x - z);
+        }
         hi = t;
-        lo += e;
+        return e;
     }
-    // renormalise so that hi = fl(hi + lo)
+    __device__ __forceinline__ void second(T x) { lo = step(x); }   // the second term: lo is still 0
+    __device__ __forceinline__ void add(T x) { lo += step(x); }
+    // renormalise so that hi = fl(hi + lo) (FP32)
     __device__ __forceinline__ void finish() {
-        T t = hi + lo;
-        lo = lo - (t - hi);
-        hi = t;
+        if constexpr (sizeof(T) == 4) {
+            T t = hi + lo;
+            lo = lo - (t - hi);
+            hi = t;
+        }
     }
 };
 
@@ -95,9 +154,9 @@ template <typename T>
 __device__ __forceinline__ void add_obs_pair(CompSum<T> &se, CompSum<T> &sl, const T *O, int lo, int mid,
                                              int hi, int cl, int cr) {
     for (int k = lo; k < hi; ++k) {
-        const int c = k < mid ? cl : cr;
-        se.add(O[8 * (int64_t)k + 2 * c]);
-        sl.add(O[8 * (int64_t)k + 2 * c + 1]);
+        const T2<T> q = *reinterpret_cast<const T2<T> *>(O + 8 * (int64_t)k + 2 * (k < mid ? cl : cr));
+        se.add(q.x);
+        sl.add(q.y);
     }
 }
 
@@ -121,20 +180,22 @@ __device__ __forceinline__ void cavity(const Belief<T> &b, T own_eta, T own_lam,
 // 1e-20 V, and nothing overflows.  (Far from the observations the precision recursion drives
 // some cavity precisions far below the FP32 range while their information stays finite;
 // treating them as carrying no information would drop that information.)
-template <typename T, int K>
-__device__ __forceinline__ void factor_messages(const T (&a)[K], T var, T r, const T (&lam)[K],
-                                                const T (&eta)[K], T (&L)[K], T (&E)[K]) {
+// FAST: returns false where a reciprocal was out of the fast form's range (FP64 only).
+template <typename T, int K, bool FAST>
+__device__ __forceinline__ bool factor_messages_as(const T (&a)[K], T var, T r, const T (&lam)[K], const T (&eta)[K],
+                                                   T (&L)[K], T (&E)[K]) {
+    bool out = false;
     T t[K], p[K];
 #pragma unroll
     for (int u = 0; u < K; ++u) {
-        if (a[u] == T(0)) {
+        if (is_zero(a[u])) {
             t[u] = T(0);
             p[u] = T(0);
         } else {
             const T a2 = mul_rn(a[u], a[u]);
-            // fmax returns the other operand for a NaN one: a NaN cavity precision is floored
-            const T fl = fmax(mul_rn(lam_floor_rel<T>(), a2), tiny_normal<T>());
-            const T rl = recip(fmax(lam[u], fl));
+            // a NaN cavity precision is floored
+            const T fl = floor_at(mul_rn(lam_floor_rel<T>(), a2), tiny_normal<T>());
+            const T rl = recip_or<FAST>(floor_at(lam[u], fl), out);
             t[u] = mul_rn(a2, rl);
             p[u] = mul_rn(a[u], mul_rn(eta[u], rl));
         }
@@ -152,18 +213,72 @@ __device__ __forceinline__ void factor_messages(const T (&a)[K], T var, T r, con
     for (int v = K - 1; v >= 0; --v) {
         const T V = add_rn(preV[v], sufV);
         const T M = add_rn(preM[v], sufM);
-        const T rV = recip(V);
+        const T rV = recip_or<FAST>(V, out);
         L[v] = mul_rn(mul_rn(a[v], a[v]), rV);
         E[v] = mul_rn(mul_rn(a[v], add_rn(r, -M)), rV);
         sufV = add_rn(sufV, t[v]);
         sufM = add_rn(sufM, p[v]);
     }
+    return !out;
+}
+template <typename T, int K>
+__device__ __forceinline__ void factor_messages(const T (&a)[K], T var, T r, const T (&lam)[K],
+                                                const T (&eta)[K], T (&L)[K], T (&E)[K]) {
+    if (!factor_messages_as<T, K, true>(a, var, r, lam, eta, L, E)) factor_messages_as<T, K, false>(a, var, r, lam, eta, L, E);
 }
 
 // Damped update m_t = beta m_{t-1} + (1 - beta) m_new, evaluated as the fused multiply-add
 // m_new + beta (m_{t-1} - m_new).
 template <typename T> __device__ __forceinline__ T damp(T old, T fresh, T beta) {
     return fma_rn(beta, add_rn(old, -fresh), fresh);
+}
+
+// Update of the factor of one cell with all four neighbours, FP64: the messages of
+// factor_messages for a = (aC, -1, -1, -1, -1) with the products by -1 and 1 and the sums with an
+// exact zero left out, then the damping.  a2 = aC^2 and flC = the floor of the centre's cavity
+// precision are rounded on the host; b are the beliefs of the slots' nodes, own the cell's
+// messages, out the damped new ones.  74 FP64 operations.  Returns false, out unset, where a
+// reciprocal is out of recip_fixed()'s range: the general form serves those cells.
+__device__ __forceinline__ bool cell_update_interior(double aC, double a2, double flC, double var, bool has_r, double r,
+                                                     const Belief<double> *const (&b)[5], const double2 (&own)[5],
+                                                     double beta, double2 (&out)[5]) {
+    double t[5], p[5];
+    bool oor = false;
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+        double eta, lam;
+        cavity(*b[u], own[u].x, own[u].y, eta, lam);
+        const double rl = recip_fixed(floor_at(lam, u == 0 ? flC : lam_floor_rel<double>()), oor);
+        t[u] = u == 0 ? mul_rn(a2, rl) : rl;
+        p[u] = u == 0 ? mul_rn(aC, mul_rn(eta, rl)) : -mul_rn(eta, rl);
+    }
+    double preV[5], preM[5];
+    preV[0] = var;
+    preV[1] = add_rn(var, t[0]);
+    preM[0] = 0.0;
+    preM[1] = p[0];
+#pragma unroll
+    for (int v = 2; v < 5; ++v) {
+        preV[v] = add_rn(preV[v - 1], t[v - 1]);
+        preM[v] = add_rn(preM[v - 1], p[v - 1]);
+    }
+    double sufV = 0.0, sufM = 0.0;
+#pragma unroll
+    for (int v = 4; v >= 0; --v) {
+        const double V = v == 4 ? preV[4] : add_rn(preV[v], sufV);
+        double M = v == 4 ? preM[4] : v == 0 ? sufM : add_rn(preM[v], sufM);
+        if (has_r) M = add_rn(M, -r);
+        const double rV = recip_fixed(V, oor);
+        const double L = v == 0 ? mul_rn(a2, rV) : rV;
+        const double E = v == 0 ? mul_rn(mul_rn(aC, -M), rV) : mul_rn(M, rV);
+        out[v].x = fma_rn(beta, add_rn(own[v].x, -E), E);
+        out[v].y = fma_rn(beta, add_rn(own[v].y, -L), L);
+        if (v > 0) {
+            sufV = v == 4 ? t[4] : add_rn(sufV, t[v]);
+            sufM = v == 4 ? p[4] : add_rn(sufM, p[v]);
+        }
+    }
+    return !oor;
 }
 
 // Number of existing 4-neighbours of node (i, j).

@@ -182,6 +182,169 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
     }
 }
 
+// ---- FP64 ----
+// FP64 arithmetic bounds this kernel (GB300: two lanes per clock and SM; an iteration's bytes would
+// take a twentieth of the time), so the work per cell is what it saves: no product by +-1 and no
+// sum with an exact zero on interior cells (cell_update_interior), Fast2Sum and three-operation
+// reciprocals, comparisons and floors in the integer unit, and both observation ranges of a node
+// in one loop, so that lanes with a term in either run together.  The messages are read straight
+// from global memory (the second reading, in the factor update, hits L1): staging them cost a pass
+// of index arithmetic and the shared memory that limited the resident blocks.  Tiles of TX columns
+// and a height chosen per grid (fused_choose_shape_f64), NT threads.  Measured per iteration, with
+// the staged kernel of 32 x 8 tiles, compensated sums of six additions and IEEE divisions before:
+// 64^2 36 -> 13.5 us, 512^2 197 -> 91 us.
+template <int TX, int NT>
+__global__ void __launch_bounds__(NT) k_fused_f64(const __grid_constant__ DevProblem p, int TY, int src, double beta) {
+    constexpr int BX = TX + 2;
+    const int BY = TY + 2;   // belief window (1-cell halo)
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Belief<double> *sb = reinterpret_cast<Belief<double> *>(smem_raw);            // [BY][BX]
+    int *rstart = reinterpret_cast<int *>(smem_raw + sizeof(Belief<double>) * BX * BY);   // [TY]
+    int *rpre = rstart + TY;                                                              // [TY + 1]
+
+    const int nx = p.nx, ny = p.ny, px = p.px;
+    const int64_t pn = p.pn;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const double2 *__restrict__ P = (const double2 *)p.P[src];
+    double2 *__restrict__ Q = (double2 *)p.P[src ^ 1];
+    const double *__restrict__ O = (const double *)p.O[src];
+    double *__restrict__ OQ = (double *)p.O[src ^ 1];
+    const int *__restrict__ optr = p.optr;
+
+    // observation ranges of the tile's base rows (the last warp; a prefix sum by shuffles)
+    if (p.m > 0 && threadIdx.x >= NT - 32) {
+        const int r = threadIdx.x - (NT - 32), gy = y0 + r;
+        int lo = 0, cnt = 0;
+        if (r < TY && gy < ny) {
+            lo = optr[(int64_t)gy * nx + x0];
+            cnt = optr[(int64_t)gy * nx + min(x0 + TX, nx)] - lo;
+        }
+        int inc = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (r >= o) inc += v;
+        }
+        if (r < TY) {
+            rstart[r] = lo;
+            rpre[r] = inc - cnt;
+        }
+        if (r == TY - 1) rpre[TY] = inc;
+    }
+
+    // 1. compensated beliefs over the tile plus a 1-cell halo
+#pragma unroll 1
+    for (int q = threadIdx.x; q < BX * BY; q += NT) {
+        const int ly = q / BX, lx = q - ly * BX;
+        const int gx = x0 - 1 + lx, gy = y0 - 1 + ly;
+        if (gx < 0 || gx >= nx || gy < 0 || gy >= ny) continue;
+        const int64_t v = (int64_t)gy * px + gx;
+        const double2 zero = make_double2(0.0, 0.0);
+        const double2 mC = P[DIR_C * pn + v];
+        const double2 mE = gx > 0 ? P[DIR_E * pn + v - 1] : zero;
+        const double2 mW = gx < nx - 1 ? P[DIR_W * pn + v + 1] : zero;
+        const double2 mN = gy > 0 ? P[DIR_N * pn + v - px] : zero;
+        const double2 mS = gy < ny - 1 ? P[DIR_S * pn + v + px] : zero;
+        int lo1 = 0, mid1 = 0, hi1 = 0, lo2 = 0, mid2 = 0, hi2 = 0;
+        if (p.m > 0) {
+            const int *o = optr + (int64_t)gy * nx + gx;
+            mid1 = o[0];
+            hi1 = o[1];
+            lo1 = gx > 0 ? o[-1] : mid1;
+            if (gy > 0) {
+                mid2 = o[-nx];
+                hi2 = o[1 - nx];
+                lo2 = gx > 0 ? o[-nx - 1] : mid2;
+            }
+        }
+        CompSum<double> se(mC.x), sl(mC.y);   // a missing neighbour adds an exact zero
+        se.second(mE.x); sl.second(mE.y);
+        se.add(mW.x); sl.add(mW.y);
+        se.add(mN.x); sl.add(mN.y);
+        se.add(mS.x); sl.add(mS.y);
+        // the observation messages of both ranges in their order, the next one loaded ahead
+        const int n1 = hi1 - lo1, nt = n1 + hi2 - lo2;
+        auto term = [&](int t) {
+            const int k = t < n1 ? lo1 + t : lo2 + t - n1;
+            const int cr = t < n1 ? (k < mid1 ? 1 : 0) : (k < mid2 ? 3 : 2);
+            return *reinterpret_cast<const double2 *>(O + 8 * (int64_t)k + 2 * cr);
+        };
+        double2 nx_t = nt > 0 ? term(0) : zero;
+        for (int t = 0; t < nt; ++t) {
+            const double2 cu = nx_t;
+            if (t + 1 < nt) nx_t = term(t + 1);
+            se.add(cu.x);
+            sl.add(cu.y);
+        }
+        se.finish();
+        sl.finish();
+        Belief<double> b;
+        b.ehi = se.hi; b.elo = se.lo; b.lhi = sl.hi; b.llo = sl.lo;
+        sb[q] = b;
+    }
+    __syncthreads();
+
+    // 2. prior cell factors of the tile
+    const double *__restrict__ tgt = (const double *)p.ptgt;
+#pragma unroll 1
+    for (int q = threadIdx.x; q < TX * TY; q += NT) {
+        const int ty = q / TX, tx = q - ty * TX;
+        const int gx = x0 + tx, gy = y0 + ty;
+        if (gx >= nx || gy >= ny) continue;
+        const int64_t c = (int64_t)gy * px + gx;
+        double2 own[5], out[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) own[u] = P[u * pn + c];
+        const Belief<double> *w = sb + (ty + 1) * BX + tx + 1;
+        const Belief<double> *const bs[5] = {w, w - 1, w + 1, w - BX, w + BX};
+        cell_update_f64(p, gy, gx, tgt ? tgt[(int64_t)gy * nx + gx] : 0.0, bs, own, beta, out);
+#pragma unroll
+        for (int u = 0; u < 5; ++u) Q[u * pn + c] = out[u];
+    }
+
+    // 3. observation factors whose base cell lies in the tile, last threads first (the first ones
+    // may still hold a cell of the loop above)
+    if (p.m > 0) {
+        const int total = rpre[TY];
+        const double *W = (const double *)p.ow;
+        const double *YV = (const double *)p.ovar;
+        for (int q = NT - 1 - threadIdx.x; q < total; q += NT) {
+            int r = 0;
+            while (r + 1 < TY && rpre[r + 1] <= q) ++r;
+            const int64_t k = rstart[r] + (q - rpre[r]);
+            const int lx = p.obase[k] - (y0 + r) * nx - x0 + 1;   // belief-window column
+            const Belief<double> *w = sb + (r + 1) * BX + lx;
+            const Belief<double> *const bs[4] = {w, w + 1, w + BX, w + BX + 1};
+            double a[4], lam[4], eta[4];
+            double2 own[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a[u] = W[4 * k + u];
+                own[u] = *reinterpret_cast<const double2 *>(O + 8 * k + 2 * u);
+                cavity(*bs[u], own[u].x, own[u].y, eta[u], lam[u]);
+            }
+            double L[4], E[4];
+            factor_messages<double, 4>(a, YV[2 * k + 1], YV[2 * k], lam, eta, L, E);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                *reinterpret_cast<double2 *>(OQ + 8 * k + 2 * u) =
+                    make_double2(damp(own[u].x, E[u], beta), damp(own[u].y, L[u], beta));
+        }
+    }
+}
+
+constexpr int F64_MAX_TY = 32;   // a warp holds the tile's row ranges
+
+template <int TX, int NT>
+cudaError_t launch_f64(const DevProblem &p, int ty, int src, double beta, cudaStream_t st) {
+    static_assert(NT >= 32, "one warp at least");
+    const size_t bytes = sizeof(Belief<double>) * (TX + 2) * (ty + 2) + sizeof(int) * (2 * ty + 1);
+    if (ty < 1 || ty > F64_MAX_TY || bytes > 48 * 1024) return cudaErrorInvalidValue;
+    const dim3 grid((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + ty - 1) / ty));
+    k_fused_f64<TX, NT><<<grid, NT, bytes, st>>>(p, ty, src, beta);
+    return cudaGetLastError();
+}
+
 template <typename T, int TX, int TY>
 cudaError_t launch_shape(const DevProblem &p, int src, double beta, cudaStream_t st) {
     using LY = FusedLayout<T, TX, TY>;
@@ -197,10 +360,9 @@ cudaError_t launch_shape(const DevProblem &p, int src, double beta, cudaStream_t
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t dispatch(const DevProblem &p, int src, double beta, FusedShape s, cudaStream_t st) {
+cudaError_t dispatch_f32(const DevProblem &p, int src, double beta, FusedShape s, cudaStream_t st) {
 #define GABP_SHAPE(X, Y) \
-    if (s.tx == X && s.ty == Y) return launch_shape<T, X, Y>(p, src, beta, st);
+    if (s.tx == X && s.ty == Y) return launch_shape<float, X, Y>(p, src, beta, st);
     GABP_SHAPE(32, 8)
     GABP_SHAPE(32, 16)
     GABP_SHAPE(64, 8)
@@ -211,6 +373,16 @@ cudaError_t dispatch(const DevProblem &p, int src, double beta, FusedShape s, cu
     return cudaErrorInvalidValue;
 }
 
+cudaError_t dispatch_f64(const DevProblem &p, int src, double beta, FusedShape s, cudaStream_t st) {
+    switch (s.tx) {
+        case 128: return launch_f64<128, 256>(p, s.ty, src, beta, st);
+        case 64: return launch_f64<64, 256>(p, s.ty, src, beta, st);
+        case 32: return launch_f64<32, 128>(p, s.ty, src, beta, st);
+        case 16: return launch_f64<16, 128>(p, s.ty, src, beta, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
 }  // namespace
 
 bool fused_shape_supported(int tx, int ty) {
@@ -218,14 +390,25 @@ bool fused_shape_supported(int tx, int ty) {
            (tx == 128 && ty == 8);
 }
 
-size_t fused_smem_bytes(int prec, FusedShape s) {
-    const size_t t2 = prec ? 16 : 8, bel = prec ? 32 : 16;
-    return t2 * 5 * (s.tx + 4) * (s.ty + 4) + bel * (s.tx + 2) * (s.ty + 2) + sizeof(int) * 2 * (s.ty + 1);
+// Tiles of 16 columns: of 8, 16 and 32 the fastest or within 3 % of it from 64^2 to 1024^2.  Their
+// height is the shortest of 4, 8 and 14 rows that gives an SM at most four tiles: short tiles
+// spread a small grid over the chip (128^2: 16.3 us with 16 x 4 against 33.0 us with 16 x 14 tiles,
+// 180^2: 24.8 against 29.6), tall ones recompute fewer halo beliefs (256^2: 37.7 against 36.1 us,
+// 1024^2: 345 against 286 us).
+FusedShape fused_choose_shape_f64(int nx, int ny) {
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        nsm = 152;
+    }
+    for (int ty : {4, 8})
+        if ((int64_t)((nx + 15) / 16) * ((ny + ty - 1) / ty) <= 4 * (int64_t)nsm) return {16, ty};
+    return {16, 14};
 }
 
 cudaError_t launch_fused_iteration(const DevProblem &p, int src, double beta, FusedShape shape,
                                    cudaStream_t st) {
-    return p.prec ? dispatch<double>(p, src, beta, shape, st) : dispatch<float>(p, src, beta, shape, st);
+    return p.prec ? dispatch_f64(p, src, beta, shape, st) : dispatch_f32(p, src, beta, shape, st);
 }
 
 }  // namespace gabp

@@ -6,6 +6,8 @@
 
 #include <string>
 
+#include "gabp_device.cuh"
+
 namespace gabp {
 
 // Device-resident description of one problem instance.  All pointers are device pointers.
@@ -16,6 +18,9 @@ struct DevProblem {
     int prec;            // 0 = FP32, 1 = FP64
     double gamma;        // prior scale (factor precision of every cell factor)
     double aC[5];        // kappa^2 + deg for deg = 0..4 (FP64)
+    double var64;        // 1 / gamma, rounded once on the host
+    double aC2_in;       // aC[4]^2: the centre coefficient of a cell with all four neighbours, squared
+    double flC_in;       // floor of that slot's cavity precision: max(1e-20 aC2_in, the smallest normal)
     float var_f;         // (float)(1 / gamma), rounded once on the host
     float aC_f[5];       // (float)aC[d]
     float aC_lo[5];      // aC[d] - aC_f[d] rounded: aC[d] as a double-float pair (aC_f, aC_lo)
@@ -69,10 +74,35 @@ __host__ __device__ __forceinline__ int64_t plane_at(const DevProblem &p, int i,
 // instructions in the FP32 kernels); FP64 kernels read the FP64 values.
 template <typename T> __device__ __forceinline__ T prior_var(const DevProblem &p);
 template <> __device__ __forceinline__ float prior_var<float>(const DevProblem &p) { return p.var_f; }
-template <> __device__ __forceinline__ double prior_var<double>(const DevProblem &p) { return 1.0 / p.gamma; }
+template <> __device__ __forceinline__ double prior_var<double>(const DevProblem &p) { return p.var64; }
 template <typename T> __device__ __forceinline__ T cell_coef(const DevProblem &p, int deg);
 template <> __device__ __forceinline__ float cell_coef<float>(const DevProblem &p, int deg) { return p.aC_f[deg]; }
 template <> __device__ __forceinline__ double cell_coef<double>(const DevProblem &p, int deg) { return p.aC[deg]; }
+
+// FP64 update of the factor of cell (i, j) with target r: beliefs b of its slots' nodes (a slot
+// without a node is not read), own messages, the damped messages into out (0, 0 in slots without
+// a node).  Shared by the split and the fused kernel, so that their messages are the same bits.
+__device__ __forceinline__ void cell_update_f64(const DevProblem &p, int i, int j, double r, const Belief<double> *const (&b)[5],
+                                                const double2 (&own)[5], double beta, double2 (&out)[5]) {
+    const int nx = p.nx, ny = p.ny;
+    if (i > 0 && i < ny - 1 && j > 0 && j < nx - 1 &&
+        cell_update_interior(p.aC[4], p.aC2_in, p.flC_in, p.var64, p.ptgt != nullptr, r, b, own, beta, out))
+        return;
+    const bool has[5] = {true, j > 0, j < nx - 1, i > 0, i < ny - 1};
+    double a[5], lam[5], eta[5], L[5], E[5];
+    a[0] = p.aC[grid_degree(i, j, nx, ny)];
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+        if (u > 0) a[u] = has[u] ? -1.0 : 0.0;
+        lam[u] = 1.0;
+        eta[u] = 0.0;
+        if (has[u]) cavity(*b[u], own[u].x, own[u].y, eta[u], lam[u]);
+    }
+    factor_messages<double, 5>(a, p.var64, r, lam, eta, L, E);
+#pragma unroll
+    for (int u = 0; u < 5; ++u)
+        out[u] = has[u] ? make_double2(damp(own[u].x, E[u], beta), damp(own[u].y, L[u], beta)) : make_double2(0.0, 0.0);
+}
 
 constexpr int RES_BLOCKS = 1024;   // fixed partition of the deterministic residual reduction
 
@@ -168,7 +198,8 @@ struct FusedShape {
 bool fused_shape_supported(int tx, int ty);
 cudaError_t launch_fused_iteration(const DevProblem &p, int src, double beta, FusedShape shape,
                                    cudaStream_t st);
-size_t fused_smem_bytes(int prec, FusedShape shape);
+// the FP64 tile shape for an nx x ny grid
+FusedShape fused_choose_shape_f64(int nx, int ny);
 
 // ---- warp-synchronous column sweep, FP32 (gabp_sweep.cu); tile 30 columns x h rows ----
 bool sweep_shape_supported(int h);

@@ -92,10 +92,25 @@ template <typename T> __global__ void k_prior(DevProblem p, int src, T beta) {
     const int64_t pn = p.pn, pc = plane_at(p, i, j);
     const T2<T> *P = (const T2<T> *)p.P[src];
     T2<T> *Q = (T2<T> *)p.P[src ^ 1];
+    const int64_t node[5] = {c, c - 1, c + 1, c - nx, c + nx};
+    if constexpr (sizeof(T) == 8) {   // the update the fused FP64 kernel uses
+        const bool has[5] = {true, j > 0, j < nx - 1, i > 0, i < ny - 1};
+        Belief<double> bl[5];
+        double2 own[5], out[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+            own[u] = P[u * pn + pc];
+            if (has[u]) bl[u] = load_belief<double>(p, node[u]);
+        }
+        const Belief<double> *const bs[5] = {&bl[0], &bl[1], &bl[2], &bl[3], &bl[4]};
+        cell_update_f64(p, i, j, p.ptgt ? ((const double *)p.ptgt)[c] : 0.0, bs, own, beta, out);
+#pragma unroll
+        for (int u = 0; u < 5; ++u) Q[u * pn + pc] = out[u];
+        return;
+    }
     const int deg = grid_degree(i, j, nx, ny);
     const T a[5] = {cell_coef<T>(p, deg), j > 0 ? T(-1) : T(0), j < nx - 1 ? T(-1) : T(0),
                     i > 0 ? T(-1) : T(0), i < ny - 1 ? T(-1) : T(0)};
-    const int64_t node[5] = {c, c - 1, c + 1, c - nx, c + nx};
     T2<T> own[5];
     T lam[5], eta[5];
 #pragma unroll

@@ -1,0 +1,63 @@
+"""GPU: which kernel and tile serve a grid under GABP_KERNEL_AUTO, against the split kernels (the
+plain form of the iteration), bit for bit, at the sizes where the choice changes."""
+import numpy as np
+import pytest
+
+import gabp_synth
+from gpu_common import ensure_built, solver
+
+pytestmark = pytest.mark.gpu
+
+SPLIT = 2
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    ensure_built()
+
+
+def _problem(nx, ny, seed=5):
+    return gabp_synth.make_problem(nx, ny, 0.05, seed, n_tracks=4, per_track=max(nx, ny), n_uniform=max(nx * ny // 15, 2),
+                                   sigma=(0.02, 0.1))
+
+
+@pytest.mark.parametrize("shape, tile", [((2, 2), 4), ((16, 4), 4), ((17, 5), 4), ((63, 61), 4), ((256, 152), 4),
+                                         ((257, 153), 8), ((256, 300), 8), ((273, 421), 14)])
+def test_fp64_auto_tiles_match_split(shape, tile):
+    p = _problem(*shape)
+    bufs = []
+    for kernel in (SPLIT, 0):
+        with solver(p, "fp64", kernel=kernel) as s:
+            if kernel == 0:
+                st = s.stats()
+                assert (st["tile_x"], st["tile_y"]) == (16, tile)
+            s.iterate(23, 0.3)
+            bufs.append(s.get_messages())
+    assert np.array_equal(bufs[0], bufs[1])
+
+
+def test_fp64_interior_update_with_a_prior_mean_matches_split():
+    p = _problem(45, 38)
+    fb = np.random.default_rng(1).standard_normal(p.n)
+    bufs = []
+    for kernel in (SPLIT, 0):
+        with solver(p, "fp64", kernel=kernel) as s:
+            s.set_prior_mean(fb)
+            s.iterate(15, 0.5)
+            bufs.append(s.get_messages())
+    assert np.array_equal(bufs[0], bufs[1])
+
+
+@pytest.mark.parametrize("gamma", [3e-303, 1e-150, 1e150, 1e303])
+def test_fp64_reciprocals_out_of_the_fast_range(orc, gamma):
+    """Scales whose precisions leave 2^+-1000 take the divisions: the marginals are the oracle's."""
+    p = gabp_synth.make_problem(20, 18, 0.3, 2, n_uniform=60)
+    fl = orc.build_factors(p.nx, p.ny, p.kappa, p.obs_x, p.obs_y, p.y, p.noise_var, gamma)
+    with np.errstate(all="ignore"):
+        mu_o, var_o, _ = orc.gabp(fl, 0.5, 12)
+    with solver(p, "fp64", gamma=gamma) as s:
+        s.iterate(12, 0.5)
+        mu, var = s.marginals()
+    ok = np.isfinite(mu_o) & np.isfinite(var_o)
+    np.testing.assert_allclose(mu[ok], mu_o[ok], rtol=1e-10, atol=1e-10 * np.max(np.abs(mu_o[ok])))
+    np.testing.assert_allclose(var[ok], var_o[ok], rtol=1e-10)
