@@ -66,9 +66,11 @@ extern "C" {
 #define GABP_INIT_PAPER 1    /* Lambda = 1e-8, eta = 0 (Alg. 1 / Alg. 2 initialisation) */
 
 /* iteration kernel (gabp_options.kernel) */
-#define GABP_KERNEL_AUTO 0   /* FP32: GABP_KERNEL_TMA if nx is a multiple of 4, else
-                                GABP_KERNEL_SWEEP; FP64: GABP_KERNEL_FUSED.  The alpha = 4
-                                prior: GABP_KERNEL_FUSED (FP32), GABP_KERNEL_SPLIT (FP64) */
+#define GABP_KERNEL_AUTO 0   /* FP32: GABP_KERNEL_TMA if nx is a multiple of 4 or the grid has 4096
+                                nodes or more (on plane rows padded to an even pitch where nx is
+                                odd), else GABP_KERNEL_SWEEP; FP64: GABP_KERNEL_FUSED.  The
+                                alpha = 4 prior: GABP_KERNEL_FUSED (FP32), GABP_KERNEL_SPLIT
+                                (FP64) */
 #define GABP_KERNEL_FUSED 1  /* one fused kernel per iteration (beliefs + all factors) */
 #define GABP_KERNEL_SPLIT 2  /* three kernels per iteration: beliefs, prior factors, obs factors */
 #define GABP_KERNEL_TMA 3    /* the fused kernel as persistent blocks fed by TMA tensor loads;

@@ -79,6 +79,12 @@ thread_local std::string t_create_err;
 // padded by one cell (DevProblem::px), so that the batched TMA kernel copies them as tensors
 thread_local bool t_pad_odd_planes = false;
 
+// AUTO runs FP32 contexts whose width is not a multiple of 4 on the TMA kernel too, on plane rows
+// padded to an even pitch and a copy of the observation index padded to a multiple of 4 ints (the
+// layout of batch members), from this many nodes on; smaller ones keep the column sweep.
+// 361 x 181: 116 -> 7 us per iteration; 1601 x 1201: 130 -> 42 us.
+constexpr int64_t TMA_PADDED_MIN_NODES = 4096;
+
 struct DeviceGuard {
     int prev = -1;
     bool ok = true;
@@ -431,6 +437,10 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
     if (o.kernel < GABP_KERNEL_AUTO || o.kernel > GABP_KERNEL_SWEEP) return fail(c, GABP_ERR_ARG, "bad kernel");
     if (!(o.tol > 0.0) || o.check_every < 1 || o.max_iters < 1) return fail(c, GABP_ERR_ARG, "bad tol/check_every/max_iters");
     if (o.tile_run < 0 || o.tile_run > 8) return fail(c, GABP_ERR_ARG, "tile_run must be 0..8");
+    // AUTO on a width that is not a multiple of 4: the TMA kernel on padded rows (options that ask
+    // for a sweep tile keep the sweep kernel)
+    const bool pad_tma = o.kernel == GABP_KERNEL_AUTO && o.precision == GABP_FP32 && alpha == 2 && nx % 4 != 0 && nx >= 5 &&
+                         (int64_t)nx * ny >= TMA_PADDED_MIN_NODES && !o.tile_x && !o.tile_y;
     if (alpha == 4) {
         // FP32: the fused tile kernel (AUTO or FUSED, tiles 28 x 4 or 28 x 8) or the split kernels;
         // FP64: the split kernels
@@ -442,10 +452,11 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
         if ((o.tile_x || o.tile_y) && !(fused && o.tile_x == 28 && gabp::fused_l2_shape_supported(o.tile_y)))
             return fail(c, GABP_ERR_ARG, "unsupported tile shape for the alpha = 4 prior (fused kernel: 28 x 4 or 28 x 8)");
     } else {
-        // the kernel AUTO resolves to: the sweep for FP32, the plain fused kernel for FP64
+        // the kernel AUTO resolves to: the TMA kernel or the sweep for FP32, the plain fused kernel
+        // for FP64
         const int k = o.kernel != GABP_KERNEL_AUTO
                           ? o.kernel
-                          : (o.precision == GABP_FP32 ? (nx % 4 == 0 && nx >= 4 ? GABP_KERNEL_TMA : GABP_KERNEL_SWEEP)
+                          : (o.precision == GABP_FP32 ? ((nx % 4 == 0 && nx >= 4) || pad_tma ? GABP_KERNEL_TMA : GABP_KERNEL_SWEEP)
                                                       : GABP_KERNEL_FUSED);
         const bool tiled = o.tile_x || o.tile_y;
         if (tiled && (k == GABP_KERNEL_FUSED || k == GABP_KERNEL_SPLIT) && !gabp::fused_shape_supported(o.tile_x, o.tile_y))
@@ -512,7 +523,7 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
     };
     DevProblem &p = c->p;
     p.nx = nx;
-    p.px = (t_pad_odd_planes && nx % 2 && alpha == 2) ? nx + 1 : nx;
+    p.px = ((t_pad_odd_planes || pad_tma) && nx % 2 && alpha == 2) ? nx + 1 : nx;
     p.pn = (int64_t)p.px * ny;
     p.ny = ny;
     p.n = n;
@@ -618,12 +629,21 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
         if (e != cudaSuccess) return cuda_fail(c, e, "observation upload/sort/precompute");
     }
     CK(gabp::launch_obs_pointers(p, c->stream), "observation pointers");
+    const int opitch = (nx + 3) & ~3;   // padded TMA contexts: rows of the index copy
+    int *optr_pad = nullptr;
+    if (pad_tma) {
+        if ((rc = dalloc(c, &q, sizeof(int) * (size_t)opitch * ny, "alloc padded index"))) return rc;
+        optr_pad = (int *)q;
+        CK(cudaMemcpy2DAsync(optr_pad, sizeof(int) * (size_t)opitch, p.optr, sizeof(int) * (size_t)nx, sizeof(int) * (size_t)nx,
+                             ny, cudaMemcpyDeviceToDevice, c->stream),
+           "padded index copy");
+    }
     CK(gabp::launch_rhs_norm(p, c->stream), "rhs norm");
     if ((rc = init_messages(c))) return rc;
     CK(cudaStreamSynchronize(c->stream), "create sync");
 
     // iteration kernel and tile shape
-    const bool tma_ok = gabp::tma_problem_supported(p);
+    const bool tma_ok = gabp::tma_problem_supported(p) || pad_tma;
     if (o.kernel == GABP_KERNEL_TMA && !tma_ok)
         return fail(c, GABP_ERR_ARG, "the TMA kernel needs FP32 messages and nx a multiple of 4");
     if (o.kernel == GABP_KERNEL_SWEEP && p.prec != 0)
@@ -637,7 +657,8 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
         c->shape = o.tile_y ? gabp::FusedShape{30, o.tile_y} : gabp::FusedShape{30, 64};
     } else if (c->kernel == GABP_KERNEL_TMA) {
         c->shape = o.tile_x ? gabp::FusedShape{o.tile_x, o.tile_y} : gabp::FusedShape{30, 14};
-        CK(gabp::make_tma_maps(p, c->shape.tx, c->shape.ty, c->maps), "tensor map encode");
+        CK(gabp::make_tma_maps(p, c->shape.tx, c->shape.ty, c->maps, gabp::TMA_MAP_PLANES | gabp::TMA_MAP_OPTR, optr_pad, opitch),
+           "tensor map encode");
         c->maps.run = o.tile_run ? o.tile_run : gabp::tma_choose_run(p, c->shape.ty);
     } else if (p.order == 2) {
         c->shape = {0, 0};
@@ -936,11 +957,15 @@ int64_t gabp_message_bytes(const gabp_ctx *c) {
 
 int gabp_get_messages(gabp_ctx *c, void *buf) {
     if (!c || !buf) return c ? fail(c, GABP_ERR_ARG, "buffer must not be NULL") : GABP_ERR_ARG;
-    if (c->p.px != c->p.nx) return fail(c, GABP_ERR_STATE, "padded message layout");   // batch members only
     DeviceGuard g(c->dev);
-    const size_t T = tsize(c);
-    const size_t pb = 2 * (size_t)c->p.planes * (size_t)c->p.n * T, ob = 8 * (size_t)c->p.m * T;
-    CK(cudaMemcpyAsync(buf, c->p.P[c->cur], pb, cudaMemcpyDefault, c->stream), "copy messages");
+    // the buffer's plane rows are nx cells long, the context's px (padding cells stay behind)
+    const size_t cell = 2 * tsize(c), row = (size_t)c->p.nx * cell, rows = (size_t)c->p.planes * c->p.ny;
+    const size_t pb = row * rows, ob = 4 * (size_t)c->p.m * cell;
+    if (c->p.px == c->p.nx)
+        CK(cudaMemcpyAsync(buf, c->p.P[c->cur], pb, cudaMemcpyDefault, c->stream), "copy messages");
+    else
+        CK(cudaMemcpy2DAsync(buf, row, c->p.P[c->cur], (size_t)c->p.px * cell, row, rows, cudaMemcpyDefault, c->stream),
+           "copy messages");
     if (ob) CK(cudaMemcpyAsync((char *)buf + pb, c->p.O[c->cur], ob, cudaMemcpyDefault, c->stream), "copy messages");
     CK(cudaStreamSynchronize(c->stream), "messages sync");
     return GABP_OK;
@@ -948,11 +973,14 @@ int gabp_get_messages(gabp_ctx *c, void *buf) {
 
 int gabp_set_messages(gabp_ctx *c, const void *buf) {
     if (!c || !buf) return c ? fail(c, GABP_ERR_ARG, "buffer must not be NULL") : GABP_ERR_ARG;
-    if (c->p.px != c->p.nx) return fail(c, GABP_ERR_STATE, "padded message layout");   // batch members only
     DeviceGuard g(c->dev);
-    const size_t T = tsize(c);
-    const size_t pb = 2 * (size_t)c->p.planes * (size_t)c->p.n * T, ob = 8 * (size_t)c->p.m * T;
-    CK(cudaMemcpyAsync(c->p.P[0], buf, pb, cudaMemcpyDefault, c->stream), "copy messages");
+    const size_t cell = 2 * tsize(c), row = (size_t)c->p.nx * cell, rows = (size_t)c->p.planes * c->p.ny;
+    const size_t pb = row * rows, ob = 4 * (size_t)c->p.m * cell;
+    if (c->p.px == c->p.nx)
+        CK(cudaMemcpyAsync(c->p.P[0], buf, pb, cudaMemcpyDefault, c->stream), "copy messages");
+    else
+        CK(cudaMemcpy2DAsync(c->p.P[0], (size_t)c->p.px * cell, buf, row, row, rows, cudaMemcpyDefault, c->stream),
+           "copy messages");
     if (ob) CK(cudaMemcpyAsync(c->p.O[0], (const char *)buf + pb, ob, cudaMemcpyDefault, c->stream), "copy messages");
     CK(cudaStreamSynchronize(c->stream), "messages sync");
     c->cur = 0;

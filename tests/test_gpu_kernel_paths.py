@@ -61,3 +61,39 @@ def test_fp64_reciprocals_out_of_the_fast_range(orc, gamma):
     ok = np.isfinite(mu_o) & np.isfinite(var_o)
     np.testing.assert_allclose(mu[ok], mu_o[ok], rtol=1e-10, atol=1e-10 * np.max(np.abs(mu_o[ok])))
     np.testing.assert_allclose(var[ok], var_o[ok], rtol=1e-10)
+
+
+@pytest.mark.parametrize("shape", [(5, 820), (61, 68), (62, 67), (63, 66), (90, 46), (91, 46), (1021, 7), (331, 209)])
+def test_fp32_padded_rows_match_split(shape):
+    """Widths that are not a multiple of 4, from 4096 nodes on: the TMA kernel on padded plane rows.
+    Messages, checkpoints (whose layout has no padding), message change, warm start, residual and
+    marginals are those of the split kernels."""
+    p = _problem(*shape)
+    got = []
+    for kernel in (SPLIT, 0):
+        with solver(p, "fp32", kernel=kernel) as s:
+            assert s.stats()["kernel"] == (SPLIT if kernel else 3)
+            s.iterate(23, 0.3)
+            a = s.get_messages()
+            change, res = s.message_change(), s.residual()
+            s.iterate(4, 0.3)
+            s.set_messages(a)
+            s.iterate(4, 0.3)
+            b = s.get_messages()
+            mean, var = s.marginals()
+            s.warm_start(mean, 1.0 / var)
+            s.iterate(3, 0.3)
+            got.append((a, b, s.get_messages(), mean, var, np.array([change, res])))
+    for x, y in zip(*got):
+        # the message change adds the planes in another order of threads (the padded layout)
+        np.testing.assert_allclose(x, y, rtol=1e-5) if x.size == 2 else np.testing.assert_array_equal(x, y)
+
+
+def test_fp32_small_or_tiled_odd_grids_keep_the_sweep():
+    for (nx, ny), opts in [((63, 65), {}), ((91, 70), dict(tile_x=30, tile_y=32)), ((4, 2), {})]:
+        p = _problem(nx, ny)
+        with solver(p, "fp32", **opts) as s:
+            assert s.stats()["kernel"] == (3 if nx == 4 else 4)
+    from paper_2404_12968_gb300 import GabpError
+    with pytest.raises(GabpError, match="multiple of 4"):
+        solver(_problem(91, 70), "fp32", kernel=3)   # asked for by name: as before
