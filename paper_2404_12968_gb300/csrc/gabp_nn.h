@@ -39,7 +39,9 @@ struct TcConvArgs {
     const __nv_bfloat16 *wpk;     // packed weights (tc_pack_weights)
     const float *bias;            // [Cout]
     __nv_bfloat16 *out;           // [B][H][W][Cout], or NULL
-    __nv_bfloat16 *pool_out;      // 2x2 average of out, [B][H/2][W/2][Cout], or NULL
+    const __nv_bfloat16 *mask;    // [B][H][W][Cout]: out is 0 where mask <= 0 (the ReLU's backward), or NULL
+    __nv_bfloat16 *pool_out;      // pool_scale x the 2x2 sums of out, [B][H/2][W/2][Cout], or NULL
+    float pool_scale;             // 0.25: the average (forward); 1: the sum (backward of the upsampling)
     const __nv_bfloat16 *up_skip; // [B][2H][2W][Cout] (with up_out)
     __nv_bfloat16 *up_out;        // nearest-upsampled out + up_skip, [B][2H][2W][Cout], or NULL
     const float *head_w;          // [2][Cout] FP32 head (Cout = 32), or NULL
@@ -82,18 +84,21 @@ cudaError_t bias_grad(const __nv_bfloat16 *g, int64_t P, int C, float *db, float
 cudaError_t flip_transpose(const __nv_bfloat16 *w, int Cout, int T, int Cin, __nv_bfloat16 *wt, cudaStream_t st);
 cudaError_t relu_bwd(const __nv_bfloat16 *y, const __nv_bfloat16 *dy, __nv_bfloat16 *dx, int64_t n, cudaStream_t st);
 cudaError_t pool(const __nv_bfloat16 *x, int B, int H, int W, int C, __nv_bfloat16 *y, cudaStream_t st);
-cudaError_t pool_bwd_add(const __nv_bfloat16 *dy, int B, int H, int W, int C, __nv_bfloat16 *dx, cudaStream_t st);
+// backward of the pooling, added to the skip gradient, then of the ReLU: dx = y > 0 ? g + dy / 4 : 0
+// (dy at half resolution, each sum rounded to BF16); C a multiple of 8
+cudaError_t pool_relu_bwd(const __nv_bfloat16 *dy, const __nv_bfloat16 *g, const __nv_bfloat16 *y, int B, int H, int W,
+                          int C, __nv_bfloat16 *dx, cudaStream_t st);
 cudaError_t up_add(const __nv_bfloat16 *r, const __nv_bfloat16 *s, int B, int H, int W, int C, __nv_bfloat16 *y,
                    cudaStream_t st);
 cudaError_t down_sum(const __nv_bfloat16 *dy, int B, int H, int W, int C, __nv_bfloat16 *dr, cudaStream_t st);
-cudaError_t add_into(const __nv_bfloat16 *a, __nv_bfloat16 *b, int64_t n, cudaStream_t st);
 cudaError_t head(const __nv_bfloat16 *x, int64_t P, int C, const float *w, const float *b, float *out,
                  cudaStream_t st);
 cudaError_t loss(const float *out, const float *target, int64_t P, float *dout, float *part, int parts,
                  cudaStream_t st);
-// dx (BF16) and the head's weight/bias gradients dwb[2C + 2] (part: ceil(P/1024) * (2C+2) floats)
-cudaError_t head_bwd(const float *dout, const __nv_bfloat16 *x, int64_t P, int C, const float *w,
-                     __nv_bfloat16 *dx, float *part, float *dwb, cudaStream_t st);
+// backward of the head (32 channels) and of the ReLU in front of it: dx = x > 0 ? sum_j dout_j w[j] : 0
+// (BF16), and the head's weight/bias gradients dwb[66] (part: at most part_cap floats, 66 or more)
+cudaError_t head_relu_bwd(const float *dout, const __nv_bfloat16 *x, int64_t P, const float *w, __nv_bfloat16 *dx,
+                          float *part, int64_t part_cap, float *dwb, cudaStream_t st);
 cudaError_t adam(float *w, float *m, float *v, const float *g, int64_t n, float lr, float b1, float b2, float eps,
                  int step, __nv_bfloat16 *w16, cudaStream_t st);
 cudaError_t to_bf16(const float *x, __nv_bfloat16 *y, int64_t n, cudaStream_t st);

@@ -310,9 +310,19 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
                     if (a.relu) f = fmaxf(f, 0.f);
                     v[j] = __float2bfloat16(f);
                 }
+                if (a.mask && valid) {   // the ReLU's backward: zero where its output was not positive
+                    uint4 mq[2];
+                    const uint4 *ms = reinterpret_cast<const uint4 *>(a.mask + pix * a.Cout + co0 + c);
+                    mq[0] = ms[0];
+                    mq[1] = ms[1];
+                    const __nv_bfloat16 *mh = reinterpret_cast<const __nv_bfloat16 *>(mq);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (!(__bfloat162float(mh[j]) > 0.f)) v[j] = __float2bfloat16(0.f);
+                }
                 if (a.out && valid) store16_bf16(a.out + pix * a.Cout + co0 + c, v);
                 if (a.pool_out) {
-                    // 2x2 average: (y, x), (y, x+1), (y+1, x), (y+1, x+1) are lanes +0, +1, +8, +9
+                    // 2x2 sum, scaled: (y, x), (y, x+1), (y+1, x), (y+1, x+1) are lanes +0, +1, +8, +9
                     __nv_bfloat16 pv[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
@@ -320,7 +330,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
                         const float f1 = __shfl_down_sync(0xffffffffu, f, 1);
                         const float f8 = __shfl_down_sync(0xffffffffu, f, 8);
                         const float f9 = __shfl_down_sync(0xffffffffu, f, 9);
-                        pv[j] = __float2bfloat16(0.25f * (((f + f1) + f8) + f9));
+                        pv[j] = __float2bfloat16(a.pool_scale * (((f + f1) + f8) + f9));
                     }
                     if (valid && !(xx & 1) && !(yy & 1)) {
                         const int64_t q = ((int64_t)b * (a.H / 2) + gy / 2) * (a.W / 2) + gx / 2;

@@ -161,9 +161,7 @@ int ensure_shape(gabp_wsnet *net, int B, int H, int W, bool grads) {
             const int64_t c32 = 32 * count;
             need = c32 > need ? c32 : need;
         }
-        const int64_t hp = ((P0 + 1023) / 1024) * (2 * HEAD_C + 2);
-        need = need > hp ? need : hp;
-        need = need > 4096 ? need : 4096;
+        need = need > 4096 ? need : 4096;   // the loss and the head's sums at the least
         WK(cudaMalloc(&q, sizeof(float) * need), "alloc partials");
         net->act_allocs.push_back(q);
         net->part = (float *)q;
@@ -215,6 +213,7 @@ int forward_tc(gabp_wsnet *net) {
         a.bias = net->w + net->boff[l];
         a.out = out ? out->p : nullptr;
         a.pool_out = pool ? pool->p : nullptr;
+        a.pool_scale = 0.25f;
         a.up_skip = up_skip ? up_skip->p : nullptr;
         a.up_out = up ? up->p : nullptr;
         if (head) {
@@ -292,8 +291,12 @@ int forward(gabp_wsnet *net) {
 }
 
 // gradient of layer l given the gradient g (after the activation's backward) at its output;
-// writes dW, db into net->g and, if din, the gradient w.r.t. its input
-int conv_bwd(gabp_wsnet *net, int l, const Buf &g, const Buf &in, Buf *din, int h, int w) {
+// writes dW, db into net->g and, if din, the gradient w.r.t. its input, with the backward of the
+// ReLU that made that input if relu (its output), and the 2x2 sums of it into down if down (the
+// backward of the upsampling).  On the tensor-core kernels both are part of the convolution's
+// epilogue.
+int conv_bwd(gabp_wsnet *net, int l, const Buf &g, const Buf &in, Buf *din, int h, int w, const Buf *relu = nullptr,
+             Buf *down = nullptr) {
     const int B = net->B;
     cudaStream_t st = net->stream;
     const LayerSpec &s = SPECS[l];
@@ -335,6 +338,9 @@ int conv_bwd(gabp_wsnet *net, int l, const Buf &g, const Buf &in, Buf *din, int 
         a.wpk = net->wtpk;
         a.bias = net->zbias;
         a.out = din->p;
+        a.mask = relu ? relu->p : nullptr;
+        a.pool_out = down ? down->p : nullptr;
+        a.pool_scale = 1.f;
         a.err = net->derr;
         a.B = B;
         a.H = h;
@@ -357,6 +363,8 @@ int conv_bwd(gabp_wsnet *net, int l, const Buf &g, const Buf &in, Buf *din, int 
         a.Cout = s.cin;
         a.T = s.taps;
         WK(gabp::nn::conv(a, st), "conv backward data");
+        if (relu) WK(gabp::nn::relu_bwd(relu->p, din->p, din->p, (int64_t)B * h * w * s.cin, st), "relu bwd");
+        if (down) WK(gabp::nn::down_sum(din->p, B, h, w, s.cin, down->p, st), "down");
     }
     return GABP_OK;
 }
@@ -367,47 +375,29 @@ int backward(gabp_wsnet *net) {
     cudaStream_t st = net->stream;
     int rc;
     Buf &ga = net->ga, &gb = net->gb;
-    // head
-    WK(gabp::nn::head_bwd(net->dout, net->d0.p, P0, HEAD_C, net->w + net->head_off, ga.p, net->part,
-                          net->g + net->head_off, st),
+    // head and the ReLU before it
+    WK(gabp::nn::head_relu_bwd(net->dout, net->d0.p, P0, net->w + net->head_off, gb.p, net->part, net->part_n,
+                               net->g + net->head_off, st),
        "head backward");
-    // dec0
-    WK(gabp::nn::relu_bwd(net->d0.p, ga.p, gb.p, P0 * 32, st), "relu bwd");
-    if ((rc = conv_bwd(net, 13, gb, net->u0, &net->gs0, H, W))) return rc;        // gs0 = du0
-    WK(gabp::nn::down_sum(net->gs0.p, B, H, W, 32, net->gr.p, st), "down");        // gr = dr0
-    if ((rc = conv_bwd(net, 12, net->gr, net->d1, &ga, H / 2, W / 2))) return rc;  // ga = dd1
-    // dec1
-    WK(gabp::nn::relu_bwd(net->d1.p, ga.p, gb.p, P0 / 4 * 64, st), "relu bwd");
-    if ((rc = conv_bwd(net, 11, gb, net->u1, &net->gs1, H / 2, W / 2))) return rc;  // gs1 = du1
-    WK(gabp::nn::down_sum(net->gs1.p, B, H / 2, W / 2, 64, net->gr.p, st), "down"); // gr = dr1
-    if ((rc = conv_bwd(net, 10, net->gr, net->d2, &ga, H / 4, W / 4))) return rc;   // ga = dd2
-    // dec2
-    WK(gabp::nn::relu_bwd(net->d2.p, ga.p, gb.p, P0 / 16 * 128, st), "relu bwd");
-    if ((rc = conv_bwd(net, 9, gb, net->u2, &net->gs2, H / 4, W / 4))) return rc;   // gs2 = du2
-    WK(gabp::nn::down_sum(net->gs2.p, B, H / 4, W / 4, 128, net->gr.p, st), "down"); // gr = dr2
-    if ((rc = conv_bwd(net, 8, net->gr, net->b3, &ga, H / 8, W / 8))) return rc;     // ga = db3
-    // enc3
-    WK(gabp::nn::relu_bwd(net->b3.p, ga.p, gb.p, P0 / 64 * 256, st), "relu bwd");
-    if ((rc = conv_bwd(net, 7, gb, net->a3, &ga, H / 8, W / 8))) return rc;          // ga = da3
-    WK(gabp::nn::relu_bwd(net->a3.p, ga.p, gb.p, P0 / 64 * 256, st), "relu bwd");
-    if ((rc = conv_bwd(net, 6, gb, net->p2, &ga, H / 8, W / 8))) return rc;          // ga = dp2
-    WK(gabp::nn::pool_bwd_add(ga.p, B, H / 4, W / 4, 128, net->gs2.p, st), "pool bwd");
-    // enc2
-    WK(gabp::nn::relu_bwd(net->s2.p, net->gs2.p, gb.p, P0 / 16 * 128, st), "relu bwd");
-    if ((rc = conv_bwd(net, 5, gb, net->a2, &ga, H / 4, W / 4))) return rc;          // ga = da2
-    WK(gabp::nn::relu_bwd(net->a2.p, ga.p, gb.p, P0 / 16 * 128, st), "relu bwd");
-    if ((rc = conv_bwd(net, 4, gb, net->p1, &ga, H / 4, W / 4))) return rc;          // ga = dp1
-    WK(gabp::nn::pool_bwd_add(ga.p, B, H / 2, W / 2, 64, net->gs1.p, st), "pool bwd");
-    // enc1
-    WK(gabp::nn::relu_bwd(net->s1.p, net->gs1.p, gb.p, P0 / 4 * 64, st), "relu bwd");
-    if ((rc = conv_bwd(net, 3, gb, net->a1, &ga, H / 2, W / 2))) return rc;          // ga = da1
-    WK(gabp::nn::relu_bwd(net->a1.p, ga.p, gb.p, P0 / 4 * 64, st), "relu bwd");
-    if ((rc = conv_bwd(net, 2, gb, net->p0, &ga, H / 2, W / 2))) return rc;          // ga = dp0
-    WK(gabp::nn::pool_bwd_add(ga.p, B, H, W, 32, net->gs0.p, st), "pool bwd");
-    // enc0
-    WK(gabp::nn::relu_bwd(net->s0.p, net->gs0.p, gb.p, P0 * 32, st), "relu bwd");
-    if ((rc = conv_bwd(net, 1, gb, net->a0, &ga, H, W))) return rc;                  // ga = da0
-    WK(gabp::nn::relu_bwd(net->a0.p, ga.p, gb.p, P0 * 32, st), "relu bwd");
+    // the decoder; gs = the skip gradients, gr = the gradients of the 1x1 reductions (a convolution
+    // reads its gradient from one of ga, gb and writes the other)
+    if ((rc = conv_bwd(net, 13, gb, net->u0, &net->gs0, H, W, nullptr, &net->gr))) return rc;          // du0, dr0
+    if ((rc = conv_bwd(net, 12, net->gr, net->d1, &gb, H / 2, W / 2, &net->d1))) return rc;             // dd1
+    if ((rc = conv_bwd(net, 11, gb, net->u1, &net->gs1, H / 2, W / 2, nullptr, &net->gr))) return rc;  // du1, dr1
+    if ((rc = conv_bwd(net, 10, net->gr, net->d2, &gb, H / 4, W / 4, &net->d2))) return rc;             // dd2
+    if ((rc = conv_bwd(net, 9, gb, net->u2, &net->gs2, H / 4, W / 4, nullptr, &net->gr))) return rc;   // du2, dr2
+    if ((rc = conv_bwd(net, 8, net->gr, net->b3, &gb, H / 8, W / 8, &net->b3))) return rc;              // db3
+    // the encoder
+    if ((rc = conv_bwd(net, 7, gb, net->a3, &ga, H / 8, W / 8, &net->a3))) return rc;                   // da3
+    if ((rc = conv_bwd(net, 6, ga, net->p2, &gb, H / 8, W / 8))) return rc;                             // dp2
+    WK(gabp::nn::pool_relu_bwd(gb.p, net->gs2.p, net->s2.p, B, H / 4, W / 4, 128, ga.p, st), "pool bwd");   // ds2
+    if ((rc = conv_bwd(net, 5, ga, net->a2, &gb, H / 4, W / 4, &net->a2))) return rc;                   // da2
+    if ((rc = conv_bwd(net, 4, gb, net->p1, &ga, H / 4, W / 4))) return rc;                             // dp1
+    WK(gabp::nn::pool_relu_bwd(ga.p, net->gs1.p, net->s1.p, B, H / 2, W / 2, 64, gb.p, st), "pool bwd");    // ds1
+    if ((rc = conv_bwd(net, 3, gb, net->a1, &ga, H / 2, W / 2, &net->a1))) return rc;                   // da1
+    if ((rc = conv_bwd(net, 2, ga, net->p0, &gb, H / 2, W / 2))) return rc;                             // dp0
+    WK(gabp::nn::pool_relu_bwd(gb.p, net->gs0.p, net->s0.p, B, H, W, 32, ga.p, st), "pool bwd");            // ds0
+    if ((rc = conv_bwd(net, 1, ga, net->a0, &gb, H, W, &net->a0))) return rc;                           // da0
     if ((rc = conv_bwd(net, 0, gb, net->x, nullptr, H, W))) return rc;
     return GABP_OK;
 }
