@@ -127,6 +127,15 @@ __device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t a, uint64_t b, ui
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
+// One lane of the (converged) warp.  The MMA loops run on the whole warp with warp-uniform
+// descriptors and only the instruction itself on the elected lane: issued from a loop of one
+// divergent lane, with the descriptors formed per MMA, an MMA takes 71 cycles however small it is;
+// this way 40 (M = 128, N = 32: the shared-memory reads of its operands) to 128 (N = 256).
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -163,7 +172,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
     // full[S], empty[S], acc_full[2], acc_empty[2], weights
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * S + 5);
     volatile int *fail = reinterpret_cast<volatile int *>(tslot + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t sbase = saddr(smem);
     auto full = [&](int s) { return saddr(&bars[s]); };
     auto empty = [&](int s) { return saddr(&bars[S + s]); };
@@ -237,46 +246,44 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
         }
     } else if (warp == 5) {
         // ---- MMA issuer ----
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc<N>();
-            int64_t it = 0;
-            int lt = 0;
-            if (resident && !mbar_wait(wbar, 0)) *fail = 1;
-            for (int64_t tile = blockIdx.x; tile < ntiles && !*fail; tile += gridDim.x, ++lt) {
-                const int acc = lt & 1;
-                if (!mbar_wait(acce(acc), (((uint32_t)lt >> 1) & 1) ^ 1)) {
-                    *fail = 1;
-                    break;
-                }
+        const uint32_t idesc = instr_desc<N>();
+        const bool one = elect_lane();
+        const uint64_t ad0 = smem_desc(0, CHUNK_PITCH, HALO_X * 16), bd0 = smem_desc(0, N * 16, 128);
+        uint32_t it = 0;
+        int lt = 0;
+        bool ok = !resident || mbar_wait(wbar, 0);
+        if (__any_sync(0xffffffffu, !ok)) *fail = 1;
+        __syncwarp();
+        for (int64_t tile = blockIdx.x; tile < ntiles && !*fail; tile += gridDim.x, ++lt) {
+            const int acc = lt & 1;
+            ok = mbar_wait(acce(acc), (((uint32_t)lt >> 1) & 1) ^ 1);
+            if (__any_sync(0xffffffffu, !ok)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t d = tmem + (uint32_t)(acc * N);
+            int kb = 0;
+            for (; kb < nkb; ++kb, ++it) {
+                const uint32_t s = it % (uint32_t)S;
+                ok = mbar_wait(full(s), (it / (uint32_t)S) & 1);
+                if (__any_sync(0xffffffffu, !ok)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d = tmem + (uint32_t)(acc * N);
-                bool ok = true;
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = (int)(it % S);
-                    if (!mbar_wait(full(s), (uint32_t)(it / S) & 1)) {
-                        ok = false;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t st = ring + (uint32_t)s * STAGE;
-                    const uint32_t wsl = resident ? sbase + (uint32_t)kb * WBYTES : st + HALO_BYTES;
+                const uint32_t st = ring + s * STAGE;
+                const uint64_t ad = ad0 + (st >> 4), bd = bd0 + ((resident ? sbase + (uint32_t)kb * WBYTES : st + HALO_BYTES) >> 4);
+                if (one) {
 #pragma unroll
                     for (int t = 0; t < T; ++t) {
                         const int dy = T == 9 ? t / 3 - 1 : 0, dx = T == 9 ? t % 3 - 1 : 0;
-                        const uint64_t ad =
-                            smem_desc(st + (uint32_t)(((dy + 1) * HALO_X + (dx + 1)) * 16), CHUNK_PITCH, HALO_X * 16);
-                        const uint64_t bd = smem_desc(wsl + (uint32_t)(t * 2 * N * 16), N * 16, 128);
-                        umma(d, ad, bd, idesc, (kb > 0 || t > 0) ? 1u : 0u);
+                        umma(d, ad + (uint64_t)((dy + 1) * HALO_X + (dx + 1)), bd + (uint64_t)(t * 2 * N), idesc,
+                             (kb > 0 || t > 0) ? 1u : 0u);
                     }
                     umma_commit(empty(s));   // the stage is free once these MMAs have read it
                 }
-                if (!ok) {
-                    *fail = 1;
-                    break;
-                }
-                umma_commit(accf(acc));   // accumulator complete
+                __syncwarp();
             }
+            if (kb < nkb) break;   // a wait ran out
+            if (one) umma_commit(accf(acc));   // accumulator complete
+            __syncwarp();
         }
+        if (__any_sync(0xffffffffu, !ok)) *fail = 1;
     } else {
         // ---- epilogue: warps 0-3, TMEM lanes 32 w .. 32 w + 31 = tile pixels ----
         const int m = 32 * warp + lane;
@@ -407,7 +414,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)S * STAGE);   // full[S], empty[S], acc
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * S + 1);
     volatile int *fail = reinterpret_cast<volatile int *>(tslot + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t sbase = saddr(smem);
     auto full = [&](int s) { return saddr(&bars[s]); };
     auto empty = [&](int s) { return saddr(&bars[S + s]); };
@@ -481,32 +488,34 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
         }
     } else if (warp == 5) {
         // ---- MMA issuer: one MMA (K = 16) per tile row and tap ----
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc_mn(N);
-            bool ok = true;
-            for (int i = 0; i < nk && !*fail; ++i) {
-                const int s = i % S;
-                if (!mbar_wait(full(s), (uint32_t)(i / S) & 1)) {
-                    ok = false;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t st = sbase + (uint32_t)s * STAGE;
+        const uint32_t idesc = instr_desc_mn(N);
+        const bool one = elect_lane();
+        const uint64_t ad0 = smem_desc(0, 128u, AG), bd0 = smem_desc(0, 128u, BG);
+        bool ok = true;
+        for (int i = 0; i < nk && !*fail; ++i) {
+            const uint32_t s = (uint32_t)i % (uint32_t)S;
+            ok = mbar_wait(full(s), ((uint32_t)i / (uint32_t)S) & 1);
+            if (__any_sync(0xffffffffu, !ok)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t st = sbase + s * STAGE;
+            const uint64_t ad = ad0 + (st >> 4), bd = bd0 + ((st + ABYTES) >> 4);
+            if (one) {
                 for (int j = 0; j < ntap; ++j) {
-                    const int t = t0 + j;
-                    const int dy = a.T == 9 ? t / 3 - 1 : 0, dx = a.T == 9 ? t % 3 - 1 : 0;
-                    for (int kk = 0; kk < KY; ++kk) {
-                        const uint64_t ad = smem_desc(st + (uint32_t)kk * 256u, 128u, AG);
-                        const uint64_t bd =
-                            smem_desc(st + ABYTES + (uint32_t)(((kk + h + dy) * HX + h + dx) * 16), 128u, BG);
-                        umma(tmem + (uint32_t)(j * N), ad, bd, idesc, (i > 0 || kk > 0) ? 1u : 0u);
-                    }
+                    const int t = t0 + j, dy = h ? t / 3 - 1 : 0, dx = h ? t % 3 - 1 : 0;
+                    const uint64_t bt = bd + (uint64_t)((h + dy) * HX + h + dx);
+                    const uint32_t d = tmem + (uint32_t)(j * N);
+                    for (int k4 = 0; k4 < KY; k4 += 4)   // KY is 4 or 8
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            umma(d, ad + (uint64_t)((k4 + q) * 16), bt + (uint64_t)((k4 + q) * HX), idesc,
+                                 (i > 0 || k4 + q > 0) ? 1u : 0u);
                 }
                 umma_commit(empty(s));   // the stage is free once these MMAs have read it
             }
-            if (!ok) *fail = 1;
-            umma_commit(accb);   // also after a failure, so that the epilogue does not wait out
+            __syncwarp();
         }
+        if (__any_sync(0xffffffffu, !ok)) *fail = 1;
+        if (one) umma_commit(accb);   // also after a failure, so that the epilogue does not wait out
     } else {
         // ---- epilogue: warps 0-3, TMEM lane 32 w + lane = output channel 128 mb + 32 w + lane ----
         const bool ok = mbar_wait(accb, 0);
@@ -696,7 +705,9 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
     const int64_t per_chunk_blocks = (int64_t)a.ngroups * a.nbm * a.nbn;
     const int64_t count = (int64_t)a.Cout * a.T * a.Cin;
     const int resident = a.tpc * a.N <= 256 && stage * a.stages <= 100u * 1024u ? 2 : 1;
-    int64_t chunks = ((int64_t)resident * nsm + per_chunk_blocks - 1) / per_chunk_blocks;
+    // (rounded down: one block more than the SMs hold is a second round for all)
+    int64_t chunks = (int64_t)resident * nsm / per_chunk_blocks;
+    if (chunks < 1) chunks = 1;
     if (chunks > a.ktiles) chunks = a.ktiles;
     if (chunks * count > a.part_cap) chunks = a.part_cap / count;
     if (chunks < 1) return cudaErrorInvalidValue;
