@@ -71,7 +71,7 @@ struct TcWgradArgs {
     int *err;                   // device flag, set if a bounded wait ran out
     int B, H, W, Cin, Cout, T;
     // set by tc_wgrad
-    int N, nbn, nbm, chunks, stages, ky, ga, tpc, ngroups;
+    int M, N, nbn, nbm, chunks, stages, ky, ga, tpc, ngroups;
     int64_t ktiles, tiles_x, tiles_y, per_chunk;
 };
 cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st);
