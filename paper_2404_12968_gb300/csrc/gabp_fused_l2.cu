@@ -129,9 +129,9 @@ __device__ __forceinline__ Belief2 node_belief_l2(const float2 *P, const float *
         if (INTERIOR || (ci >= 0 && ci < ny && cj >= 0 && cj < nx))
             in[d] = P[d * pn + v - ((int64_t)l2_dy(d) * nx + l2_dx(d))];
     }
-    CompSum2 s(in[0]);
+    CompSum2 s(in[0], in[1]);   // a missing neighbour adds an exact zero
 #pragma unroll
-    for (int d = 1; d < L2_SLOTS; ++d) {
+    for (int d = 2; d < L2_SLOTS; ++d) {
         const int ci = gy - l2_dy(d), cj = gx - l2_dx(d);
         if (INTERIOR || (ci >= 0 && ci < ny && cj >= 0 && cj < nx)) s.add(in[d]);
     }

@@ -63,14 +63,17 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // Compensated (eta, Lambda) belief sums: TwoSum accumulation of both components at once.
 struct CompSum2 {
     float2 hi, lo;
-    __device__ __forceinline__ explicit CompSum2(float2 first) : hi(first), lo(f2(0.f, 0.f)) {}
-    __device__ __forceinline__ void add(float2 x) {
+    // the first two terms (adding the first error to a zero lo would leave it as it is: a TwoSum
+    // error is never -0)
+    __device__ __forceinline__ CompSum2(float2 first, float2 x) : hi(first) { lo = step(x); }
+    __device__ __forceinline__ float2 step(float2 x) {   // hi += x; returns the rounding error
         const float2 t = add2(hi, x);
         const float2 z = sub2(t, hi);
         const float2 e = add2(sub2(hi, sub2(t, z)), sub2(x, z));
         hi = t;
-        lo = add2(lo, e);
+        return e;
     }
+    __device__ __forceinline__ void add(float2 x) { lo = add2(lo, step(x)); }
     __device__ __forceinline__ void finish() {
         const float2 t = add2(hi, lo);
         lo = sub2(lo, sub2(t, hi));
@@ -90,8 +93,7 @@ __device__ __forceinline__ float2 cavity2(const Belief2 &b, float2 own) { return
 // observation index (the order every kernel uses): corner cl for [lo, mid), cr for [mid, hi).
 __device__ __forceinline__ void add_obs_pair2(CompSum2 &s, const float *O, int lo, int mid, int hi, int cl, int cr) {
     for (int k = lo; k < hi; ++k) {
-        const int c = k < mid ? cl : cr;
-        s.add(*reinterpret_cast<const float2 *>(O + 8 * (int64_t)k + 2 * c));
+        s.add(reinterpret_cast<const float2 *>(O)[4u * (unsigned)k + (unsigned)(k < mid ? cl : cr)]);
     }
 }
 
