@@ -205,10 +205,10 @@ __global__ void __launch_bounds__(NT) k_fused_f64(const __grid_constant__ DevPro
     const int nx = p.nx, ny = p.ny, px = p.px;
     const int64_t pn = p.pn;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const double2 *__restrict__ P = (const double2 *)p.P[src];
-    double2 *__restrict__ Q = (double2 *)p.P[src ^ 1];
-    const double *__restrict__ O = (const double *)p.O[src];
-    double *__restrict__ OQ = (double *)p.O[src ^ 1];
+    const double2 *P = (const double2 *)p.P[src];
+    double2 *Q = (double2 *)p.P[src ^ 1];
+    const double *O = (const double *)p.O[src];
+    double *OQ = (double *)p.O[src ^ 1];
     const int *__restrict__ optr = p.optr;
 
     // observation ranges of the tile's base rows (the last warp; a prefix sum by shuffles)
@@ -231,6 +231,9 @@ __global__ void __launch_bounds__(NT) k_fused_f64(const __grid_constant__ DevPro
         }
         if (r == TY - 1) rpre[TY] = inc;
     }
+
+    pdl_wait();   // the ranges above are static; the messages are the previous iteration's
+    pdl_trigger();
 
     // 1. compensated beliefs over the tile plus a 1-cell halo
 #pragma unroll 1
@@ -333,6 +336,22 @@ __global__ void __launch_bounds__(NT) k_fused_f64(const __grid_constant__ DevPro
     }
 }
 
+// SMs of the current device (looked up once per device)
+int sm_count() {
+    static int dev_cached = -1, nsm = 152;
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev != dev_cached) {
+        int v = 0;
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0) {
+            nsm = v;
+            dev_cached = dev;
+        } else {
+            cudaGetLastError();
+        }
+    }
+    return nsm;
+}
+
 constexpr int F64_MAX_TY = 32;   // a warp holds the tile's row ranges
 
 template <int TX, int NT>
@@ -341,8 +360,9 @@ cudaError_t launch_f64(const DevProblem &p, int ty, int src, double beta, cudaSt
     const size_t bytes = sizeof(Belief<double>) * (TX + 2) * (ty + 2) + sizeof(int) * (2 * ty + 1);
     if (ty < 1 || ty > F64_MAX_TY || bytes > 48 * 1024) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + ty - 1) / ty));
-    k_fused_f64<TX, NT><<<grid, NT, bytes, st>>>(p, ty, src, beta);
-    return cudaGetLastError();
+    // overlapped launches for grids of at most one block per SM (64^2: 13.5 -> 12.8 us); with more, the
+    // next launch's blocks fill the slots unevenly (256^2: 36 -> 38 us)
+    return launch_pdl((int64_t)grid.x * grid.y <= sm_count(), k_fused_f64<TX, NT>, grid, NT, bytes, st, p, ty, src, beta);
 }
 
 template <typename T, int TX, int TY>
@@ -396,11 +416,7 @@ bool fused_shape_supported(int tx, int ty) {
 // 180^2: 24.8 against 29.6), tall ones recompute fewer halo beliefs (256^2: 37.7 against 36.1 us,
 // 1024^2: 345 against 286 us).
 FusedShape fused_choose_shape_f64(int nx, int ny) {
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        nsm = 152;
-    }
+    const int nsm = sm_count();
     for (int ty : {4, 8})
         if ((int64_t)((nx + 15) / 16) * ((ny + ty - 1) / ty) <= 4 * (int64_t)nsm) return {16, ty};
     return {16, 14};

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + LY::bar_off);
     int *flag = reinterpret_cast<int *>(smem + LY::ints_off) + 2 * LY::NI;
 
-    const int ntiles = BATCH ? *ba.nitems : 0;   // BATCH: work items
+    const int ntiles = BATCH ? *ba.nitems : 0;   // BATCH: work items (uploaded before the launches)
     const int G = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float2 beta2 = f2(beta, beta);
@@ -206,6 +206,8 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
         *flag = 0;
     }
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
     if (BATCH ? ba.debug_stall : p.debug_stall) {
         // failure-detection test: wait on a barrier that nothing arrives on, before any copy is
         // issued; the bounded wait runs out, the block raises the error flag and returns
@@ -319,17 +321,16 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
                     lo2 = gx > 0 ? wptr(gx - 1, gy - 1) : mid2;
                     hi2 = last ? mid2 : wptr(gx + 1, gy - 1);
                     const float2 *O2 = reinterpret_cast<const float2 *>(O);   // (eta, Lambda) of k, corner c at 4 k + c
-                    if (lo1 < hi1) first1 = O2[4 * (int64_t)lo1 + (lo1 < mid1 ? 1 : 0)];
-                    if (lo2 < hi2) first2 = O2[4 * (int64_t)lo2 + (lo2 < mid2 ? 3 : 2)];
+                    if (lo1 < hi1) first1 = O2[4u * (unsigned)lo1 + (lo1 < mid1 ? 1u : 0u)];
+                    if (lo2 < hi2) first2 = O2[4u * (unsigned)lo2 + (lo2 < mid2 ? 3u : 2u)];
                     any2 = __any_sync(__activemask(), lo1 + 1 < hi1 || lo2 + 1 < hi2);
                     if (any2) {
-                        if (lo1 + 1 < hi1) second1 = O2[4 * (int64_t)(lo1 + 1) + (lo1 + 1 < mid1 ? 1 : 0)];
-                        if (lo2 + 1 < hi2) second2 = O2[4 * (int64_t)(lo2 + 1) + (lo2 + 1 < mid2 ? 3 : 2)];
+                        if (lo1 + 1 < hi1) second1 = O2[4u * (unsigned)(lo1 + 1) + (lo1 + 1 < mid1 ? 1u : 0u)];
+                        if (lo2 + 1 < hi2) second2 = O2[4u * (unsigned)(lo2 + 1) + (lo2 + 1 < mid2 ? 3u : 2u)];
                     }
                 }
-                CompSum2 s(sm[(DIR_C * RY + ry) * RX + rx]);
                 // zero-filled outside the grid: the boundary terms add exact zeros
-                s.add(sm[(DIR_E * RY + ry) * RX + rx - 1]);
+                CompSum2 s(sm[(DIR_C * RY + ry) * RX + rx], sm[(DIR_E * RY + ry) * RX + rx - 1]);
                 s.add(sm[(DIR_W * RY + ry) * RX + rx + 1]);
                 s.add(sm[(DIR_N * RY + ry - 1) * RX + rx]);
                 s.add(sm[(DIR_S * RY + ry + 1) * RX + rx]);
@@ -496,9 +497,8 @@ cudaError_t launch_cfg(const DevProblem &p, const TmaMaps &maps, int src, double
     tr.step_x = grid % tr.ntx;
     tr.step_b = grid / tr.ntx;
     const TmaBatchArgs none{};
-    k_fused_tma<TY, S, RW, false><<<grid, LY::TNT, LY::bytes, st>>>(maps.planes[src], maps.optr, p, none, tr, src,
-                                                                     (float)beta);
-    return cudaGetLastError();
+    return launch_pdl(true, k_fused_tma<TY, S, RW, false>, dim3((unsigned)grid), LY::TNT, LY::bytes, st, maps.planes[src], maps.optr, p,
+                      none, tr, src, (float)beta);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
@@ -601,8 +601,8 @@ cudaError_t launch_batch_cfg(const TmaBatchArgs &ba, const DevProblem &first, in
     CUtensorMap unused;
     std::memset(&unused, 0, sizeof unused);
     const TileRuns none{1, 1, 1, 0, 0};
-    k_fused_tma<TY, 2, 1, true><<<grid, LY::TNT, LY::bytes, st>>>(unused, unused, first, ba, none, src, (float)beta);
-    return cudaGetLastError();
+    return launch_pdl(true, k_fused_tma<TY, 2, 1, true>, dim3((unsigned)grid), LY::TNT, LY::bytes, st, unused, unused, first, ba, none,
+                      src, (float)beta);
 }
 
 bool tma_batch_shape_supported(int ty) { return ty == 14 || ty == 22 || ty == 30; }

@@ -119,13 +119,15 @@ __global__ void k_pw_zero(T *m, int64_t count) {
 // node's reads are in flight at once without a register each, and one latency is paid per node.
 // (Loaded into registers, bounded to 40 for six resident blocks of 256 threads, the own messages and
 // coefficients were read one direction after the other, and the spills missed L1.)  Slots
-// are private to the thread, so no barrier is needed.  Per iteration: 64^2 8.6 -> 6.2 us, 512^2 22.5 ->
-// 14.2 us, 1024^2 71 -> 61 us, 4096^2 887 -> 883 us (there 4.7 TB/s of DRAM traffic, the algorithmic
-// bytes); FP64 512^2 311 -> 242 us (bound by FP64 arithmetic).
-constexpr int PW_NT = 128;   // threads per block
+// are private to the thread, so no barrier is needed.  The order of the copies matters to DRAM:
+// coefficients, incoming, own messages 0.70 ms at 4096^2; own before incoming messages 0.84 ms; own
+// messages and coefficients in turn 0.88 ms.  Per iteration, before and after: 64^2 8.6 -> 3.4 us,
+// 512^2 22.5 -> 11.3 us, 1024^2 71 -> 47 us, 4096^2 887 -> 703 us (5.9 TB/s); FP64 512^2 311 -> 206 us
+// (bound by FP64 arithmetic; 247 us with blocks of 128).
 template <typename T> struct PwSlots {
-    T2<T> in[ND][PW_NT], old[ND][PW_NT];
-    T q[ND][PW_NT];
+    static constexpr int NT = sizeof(T) == 4 ? 128 : 64;   // threads per block
+    T2<T> in[ND][NT], old[ND][NT];
+    T q[ND][NT];
 };
 
 template <int BYTES> __device__ __forceinline__ void copy_async(void *dst, const void *src) {
@@ -160,16 +162,24 @@ __device__ __forceinline__ float2 pair_add(float2 a, float2 b) { return make_flo
 __device__ __forceinline__ double2 pair_add(double2 a, double2 b) { return make_double2(add_rn(a.x, b.x), add_rn(a.y, b.y)); }
 
 template <typename T>
-__global__ void __launch_bounds__(PW_NT) k_pw_iter(int nx, int ny, int64_t n, const T *__restrict__ Pd, const T *__restrict__ hv,
-                                                   const T *__restrict__ Pn, const T2<T> *__restrict__ src, T2<T> *__restrict__ dst,
+__global__ void __launch_bounds__(PwSlots<T>::NT) k_pw_iter(int nx, int ny, int64_t n, const T *__restrict__ Pd, const T *__restrict__ hv,
+                                                   const T *__restrict__ Pn, const T2<T> *src, T2<T> *dst,
                                                    T c, T inv_c, T eta) {
     extern __shared__ __align__(16) unsigned char pw_smem[];
     PwSlots<T> &S = *reinterpret_cast<PwSlots<T> *>(pw_smem);
     const int t = threadIdx.x;
-    const int64_t v = blockIdx.x * (int64_t)PW_NT + t;
-    if (v >= n) return;
+    const int64_t v = blockIdx.x * (int64_t)PwSlots<T>::NT + t;
+    if (v >= n) {
+        pdl_wait();
+        return;
+    }
     const int i = (int)((unsigned)v / (unsigned)nx), j = (int)((unsigned)v - (unsigned)i * (unsigned)nx);   // n <= 2^30
     const bool interior = i >= 2 && i < ny - 2 && j >= 2 && j < nx - 2;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) copy_async<sizeof(T)>(&S.q[d][t], Pn + (int64_t)d * n + v);
+    const T2<T> node = {Pd[v], hv[v]};
+    pdl_wait();   // the coefficients are static; the messages are the previous iteration's
+    pdl_trigger();
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
         // incoming from the neighbour at -off_d: plane d there
@@ -180,11 +190,7 @@ __global__ void __launch_bounds__(PW_NT) k_pw_iter(int nx, int ny, int64_t n, co
             S.in[d][t] = T2<T>{T(0), T(0)};
     }
 #pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        copy_async<sizeof(T2<T>)>(&S.old[d][t], src + (int64_t)d * n + v);
-        copy_async<sizeof(T)>(&S.q[d][t], Pn + (int64_t)d * n + v);
-    }
-    const T2<T> node = {Pd[v], hv[v]};
+    for (int d = 0; d < ND; ++d) copy_async<sizeof(T2<T>)>(&S.old[d][t], src + (int64_t)d * n + v);
     const T cm1 = add_rn(c, T(-1)), keep = add_rn(T(1), -eta);
     asm volatile("cp.async.wait_all;" ::: "memory");
     // leave-one-out sums of the incoming messages, in direction order: suffix sums kept, the prefix
@@ -269,10 +275,9 @@ cudaError_t pw_launch(const DevProblem &p, const void *Pd, const void *hv, const
         if (e != cudaSuccess) return e;
         configured_dev = dev;
     }
-    const unsigned blocks = (unsigned)((p.n + PW_NT - 1) / PW_NT);
-    k_pw_iter<T><<<blocks, PW_NT, sizeof(PwSlots<T>), st>>>(p.nx, p.ny, p.n, (const T *)Pd, (const T *)hv, (const T *)Pn,
-                                                            (const T2<T> *)src, (T2<T> *)dst, (T)c, (T)(1.0 / c), (T)eta);
-    return cudaGetLastError();
+    const unsigned blocks = (unsigned)((p.n + PwSlots<T>::NT - 1) / PwSlots<T>::NT);
+    return launch_pdl(true, k_pw_iter<T>, dim3(blocks), PwSlots<T>::NT, sizeof(PwSlots<T>), st, p.nx, p.ny, p.n, (const T *)Pd, (const T *)hv,
+                      (const T *)Pn, (const T2<T> *)src, (T2<T> *)dst, (T)c, (T)(1.0 / c), (T)eta);
 }
 }  // namespace
 
