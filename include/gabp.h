@@ -110,7 +110,7 @@ typedef struct {
     int tile_x;       /* fused-kernel tile width in cells; 0 = the default / autotuned shape */
     int tile_y;       /* fused-kernel tile height in cells; 0 = the default / autotuned shape.
                          GABP_KERNEL_FUSED: 32x8, 32x16, 32x32, 64x8, 64x16, 128x8 (the FP64
-                         default: 16x4, 16x8 or 16x14 by the grid's size);
+                         default: 8x4, 16x4, 16x8 or 16x14 by the grid's size);
                          GABP_KERNEL_TMA: 30x14, 30x22, 30x30;
                          GABP_KERNEL_SWEEP: 30x16, 30x32, 30x64, 30x128;
                          GABP_KERNEL_FUSED with alpha = 4: 28x4, 28x8 */

@@ -336,6 +336,211 @@ __global__ void __launch_bounds__(NT) k_fused_f64(const __grid_constant__ DevPro
     }
 }
 
+// The same iteration for small grids, where a tile's chain of FP64 instructions is what takes the time
+// (each holds its SM quarter for 64 cycles or more, however few lanes are active): the chain is cut by
+// giving more warps a part of it.  Tiles of 8 x 4 cells, 8 warps:
+//   beliefs: warps 0, 1 sum the window nodes' eta messages, warps 2, 3 their Lambda messages;
+//   cell factors: warp u (0..4) owns slot u of the tile's 32 cells.  It forms the slot's terms
+//     t_u = a_u^2 / lam_u and p_u = a_u eta_u / lam_u, the warps exchange them through shared memory,
+//     and each adds the other four slots' in the order of factor_messages (21 FP64 instructions per
+//     warp against 74 in one);
+//   observation factors: warps 5..7, four lanes per factor, one per corner.
+// Messages are bit-identical to the other kernels' (but for the sign of a zero at damping 0).
+constexpr int WX = 8, WY = 4, WNT = 256, WBX = WX + 2, WNODES = WBX * (WY + 2);
+
+__device__ __forceinline__ void bar_cells() { asm volatile("bar.sync 1, 160;" ::: "memory"); }   // warps 0..4
+
+__global__ void __launch_bounds__(WNT) k_fused_f64_wide(const __grid_constant__ DevProblem p, int src, double beta) {
+    __shared__ double sb[4][WNODES];        // eta_hi, eta_lo, lam_hi, lam_lo of the window's nodes
+    __shared__ double2 stp[5][32];          // (t, p) of the cells' slots
+    __shared__ int rstart[WY], rpre[WY + 1];
+    const int nx = p.nx, ny = p.ny, px = p.px, tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int64_t pn = p.pn;
+    const int x0 = blockIdx.x * WX, y0 = blockIdx.y * WY;
+    const double2 *P = (const double2 *)p.P[src];
+    double2 *Q = (double2 *)p.P[src ^ 1];
+    const double *O = (const double *)p.O[src];
+    double *OQ = (double *)p.O[src ^ 1];
+    const int *__restrict__ optr = p.optr;
+
+    // observation ranges of the tile's base rows (one lane each)
+    if (warp == 4 && p.m > 0) {
+        const int gy = y0 + lane;
+        int lo = 0, cnt = 0;
+        if (lane < WY && gy < ny) {
+            lo = optr[(int64_t)gy * nx + x0];
+            cnt = optr[(int64_t)gy * nx + min(x0 + WX, nx)] - lo;
+        }
+        int inc = cnt;
+#pragma unroll
+        for (int o = 1; o < WY; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (lane < WY) {
+            rstart[lane] = lo;
+            rpre[lane] = inc - cnt;
+        }
+        if (lane == WY - 1) rpre[WY] = inc;
+    }
+    // the window node of this thread and its observation ranges (static), then the messages
+    const int node = (warp & 1) * 32 + lane, comp = warp >> 1;   // warps 0..3
+    const int ly = node / WBX, lx = node - ly * WBX, gx = x0 - 1 + lx, gy = y0 - 1 + ly;
+    const bool mine = warp < 4 && node < WNODES && gx >= 0 && gx < nx && gy >= 0 && gy < ny;
+    int lo1 = 0, mid1 = 0, hi1 = 0, lo2 = 0, mid2 = 0, hi2 = 0;
+    if (mine && p.m > 0) {
+        const int *o = optr + (int64_t)gy * nx + gx;
+        mid1 = o[0];
+        hi1 = o[1];
+        lo1 = gx > 0 ? o[-1] : mid1;
+        if (gy > 0) {
+            mid2 = o[-nx];
+            hi2 = o[1 - nx];
+            lo2 = gx > 0 ? o[-nx - 1] : mid2;
+        }
+    }
+    pdl_wait();
+    pdl_trigger();
+    // the cell of this lane (warps 0..4): its own message on the warp's slot
+    const int cty = lane / WX, ctx = lane - cty * WX, cx = x0 + ctx, cy = y0 + cty;
+    const int u = warp;   // slot: C, W, E, S, N
+    const bool cell = u < 5 && cx < nx && cy < ny;
+    const bool has = cell && (u == 0 || (u == 1 && cx > 0) || (u == 2 && cx < nx - 1) || (u == 3 && cy > 0) ||
+                              (u == 4 && cy < ny - 1));
+    const int64_t pc = (int64_t)cy * px + cx;
+    double2 own = make_double2(0.0, 0.0);
+    if (has) own = P[u * pn + pc];
+
+    // 1. compensated beliefs, one component per thread
+    if (mine) {
+        const int64_t v = (int64_t)gy * px + gx;
+        auto at = [&](int d, int64_t i) { return reinterpret_cast<const double *>(P + d * pn + i)[comp]; };
+        const double mC = at(DIR_C, v);
+        const double mE = gx > 0 ? at(DIR_E, v - 1) : 0.0, mW = gx < nx - 1 ? at(DIR_W, v + 1) : 0.0;
+        const double mN = gy > 0 ? at(DIR_N, v - px) : 0.0, mS = gy < ny - 1 ? at(DIR_S, v + px) : 0.0;
+        const int n1 = hi1 - lo1, nt = n1 + hi2 - lo2;
+        auto term = [&](int t) {   // the observation messages of both ranges in their order
+            const int k = t < n1 ? lo1 + t : lo2 + t - n1;
+            const int cr = t < n1 ? (k < mid1 ? 1 : 0) : (k < mid2 ? 3 : 2);
+            return O[8 * (int64_t)k + 2 * cr + comp];
+        };
+        double next = nt > 0 ? term(0) : 0.0;
+        CompSum<double> s(mC);
+        s.second(mE);
+        s.add(mW);
+        s.add(mN);
+        s.add(mS);
+        for (int t = 0; t < nt; ++t) {
+            const double cu = next;
+            if (t + 1 < nt) next = term(t + 1);
+            s.add(cu);
+        }
+        s.finish();
+        sb[2 * comp][node] = s.hi;
+        sb[2 * comp + 1][node] = s.lo;
+    }
+    __syncthreads();
+
+    if (warp < 5) {
+        // 2. cell factors: slot u of 32 cells
+        const int w = (cty + 1) * WBX + ctx + 1 + (u == 1 ? -1 : u == 2 ? 1 : u == 3 ? -WBX : u == 4 ? WBX : 0);
+        const double aC = cell ? p.aC[grid_degree(cy, cx, nx, ny)] : 1.0;
+        const double a2 = u == 0 ? mul_rn(aC, aC) : 1.0;
+        bool out = false;
+        double2 tp = make_double2(0.0, 0.0);
+        if (has) {
+            const double lam = (sb[2][w] - own.y) + sb[3][w], eta = (sb[0][w] - own.x) + sb[1][w];
+            double fl = lam_floor_rel<double>();
+            if (u == 0) fl = floor_at(mul_rn(fl, a2), tiny_normal<double>());
+            const double x = floor_at(lam, fl);
+            double rl = recip_fixed(x, out);
+            if (out) rl = 1.0 / x;
+            tp.x = u == 0 ? mul_rn(a2, rl) : rl;
+            tp.y = u == 0 ? mul_rn(aC, mul_rn(eta, rl)) : -mul_rn(eta, rl);
+        }
+        stp[u][lane] = tp;
+        bar_cells();
+        // the other slots' terms: those before u from the left, those after it from the right
+        double V = p.var64, M = 0.0, sV = 0.0, sM = 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (q < u) {
+                const double2 o = stp[q][lane];
+                V = add_rn(V, o.x);
+                M = q == 0 ? o.y : add_rn(M, o.y);
+            }
+#pragma unroll
+        for (int q = 4; q > 0; --q)
+            if (q > u) {
+                const double2 o = stp[q][lane];
+                sV = q == 4 ? o.x : add_rn(sV, o.x);
+                sM = q == 4 ? o.y : add_rn(sM, o.y);
+            }
+        if (u < 4) {
+            V = add_rn(V, sV);
+            M = u == 0 ? sM : add_rn(M, sM);
+        }
+        if (p.ptgt && cell) M = add_rn(M, -((const double *)p.ptgt)[(int64_t)cy * nx + cx]);
+        out = false;
+        double rV = recip_fixed(V, out);
+        if (out) rV = 1.0 / V;
+        const double L = u == 0 ? mul_rn(a2, rV) : rV;
+        const double E = u == 0 ? mul_rn(mul_rn(aC, -M), rV) : mul_rn(M, rV);
+        if (cell) Q[u * pn + pc] = has ? make_double2(damp(own.x, E, beta), damp(own.y, L, beta)) : make_double2(0.0, 0.0);
+    } else if (p.m > 0) {
+        // 3. observation factors based in the tile: lane = (factor, corner)
+        const int total = rpre[WY], c = lane & 3;
+        const double *W = (const double *)p.ow;
+        const double *YV = (const double *)p.ovar;
+        for (int q0 = 8 * (warp - 5); q0 < total; q0 += 24) {
+            const int q = q0 + (lane >> 2);
+            const bool on = q < total;
+            const int qq = on ? q : total - 1;
+            int r = 0;
+#pragma unroll
+            for (int t = 1; t < WY; ++t)
+                if (rpre[t] <= qq) r = t;
+            const int64_t k = rstart[r] + (qq - rpre[r]);
+            const int w = (r + 1 + (c >> 1)) * WBX + p.obase[k] - (y0 + r) * nx - x0 + 1 + (c & 1);
+            const double a = W[4 * k + c], y = YV[2 * k], var = YV[2 * k + 1];
+            const double2 o = *reinterpret_cast<const double2 *>(O + 8 * k + 2 * c);
+            const double lam = (sb[2][w] - o.y) + sb[3][w], eta = (sb[0][w] - o.x) + sb[1][w];
+            const double a2 = mul_rn(a, a);
+            const double x = floor_at(lam, floor_at(mul_rn(lam_floor_rel<double>(), a2), tiny_normal<double>()));
+            bool out = false;
+            double rl = recip_fixed(x, out);
+            if (out) rl = 1.0 / x;
+            double t = mul_rn(a2, rl), pp = mul_rn(a, mul_rn(eta, rl));
+            if (is_zero(a)) t = pp = 0.0;
+            double V = var, M = 0.0, sV = 0.0, sM = 0.0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {   // slots before this one, in order
+                const double tj = __shfl_sync(0xffffffffu, t, j, 4), pj = __shfl_sync(0xffffffffu, pp, j, 4);
+                if (j < 3) {
+                    const double nV = add_rn(V, tj), nM = add_rn(M, pj);
+                    if (j < c) V = nV, M = nM;
+                }
+            }
+#pragma unroll
+            for (int j = 3; j >= 0; --j) {   // slots after it, from the last
+                const double tj = __shfl_sync(0xffffffffu, t, j, 4), pj = __shfl_sync(0xffffffffu, pp, j, 4);
+                if (j > 0) {
+                    const double nV = add_rn(sV, tj), nM = add_rn(sM, pj);
+                    if (j > c) sV = nV, sM = nM;
+                }
+            }
+            V = add_rn(V, sV);
+            M = add_rn(M, sM);
+            out = false;
+            double rV = recip_fixed(V, out);
+            if (out) rV = 1.0 / V;
+            const double L = mul_rn(a2, rV), E = mul_rn(mul_rn(a, add_rn(y, -M)), rV);
+            if (on) *reinterpret_cast<double2 *>(OQ + 8 * k + 2 * c) = make_double2(damp(o.x, E, beta), damp(o.y, L, beta));
+        }
+    }
+}
+
 // SMs of the current device (looked up once per device)
 int sm_count() {
     static int dev_cached = -1, nsm = 152;
@@ -398,6 +603,11 @@ cudaError_t dispatch_f64(const DevProblem &p, int src, double beta, FusedShape s
         case 128: return launch_f64<128, 256>(p, s.ty, src, beta, st);
         case 64: return launch_f64<64, 256>(p, s.ty, src, beta, st);
         case 32: return launch_f64<32, 128>(p, s.ty, src, beta, st);
+        case 8: {
+            const dim3 grid((unsigned)((p.nx + WX - 1) / WX), (unsigned)((p.ny + WY - 1) / WY));
+            return launch_pdl(s.ty == WY && grid.y <= 65535 ? (int64_t)grid.x * grid.y <= sm_count() : false, k_fused_f64_wide, grid,
+                              WNT, 0, st, p, src, beta);
+        }
         case 16: return launch_f64<16, 128>(p, s.ty, src, beta, st);
     }
     return cudaErrorInvalidValue;
@@ -410,13 +620,15 @@ bool fused_shape_supported(int tx, int ty) {
            (tx == 128 && ty == 8);
 }
 
-// Tiles of 16 columns: of 8, 16 and 32 the fastest or within 3 % of it from 64^2 to 1024^2.  Their
-// height is the shortest of 4, 8 and 14 rows that gives an SM at most four tiles: short tiles
-// spread a small grid over the chip (128^2: 16.3 us with 16 x 4 against 33.0 us with 16 x 14 tiles,
-// 180^2: 24.8 against 29.6), tall ones recompute fewer halo beliefs (256^2: 37.7 against 36.1 us,
-// 1024^2: 345 against 286 us).
+// Small grids: the 8 x 4 tiles of k_fused_f64_wide while an SM gets at most three of them (64^2 13.2 ->
+// 6.8 us, 96^2 12.8 -> 11.1 us, 110^2 17.4 -> 14.6 us, 128^2 16.8 -> 17.2 us).  Else tiles of 16 columns,
+// of 8, 16 and 32 the fastest or within 3 % of it up to 1024^2; their height is the shortest of 4, 8
+// and 14 rows that gives an SM at most four tiles: short tiles spread a small grid over the chip
+// (128^2: 16.3 us with 16 x 4 against 33.0 us with 16 x 14 tiles, 180^2: 24.8 against 29.6), tall ones
+// recompute fewer halo beliefs (256^2: 37.7 against 36.1 us, 1024^2: 345 against 286 us).
 FusedShape fused_choose_shape_f64(int nx, int ny) {
     const int nsm = sm_count();
+    if ((int64_t)((nx + WX - 1) / WX) * ((ny + WY - 1) / WY) <= 3 * (int64_t)nsm) return {WX, WY};
     for (int ty : {4, 8})
         if ((int64_t)((nx + 15) / 16) * ((ny + ty - 1) / ty) <= 4 * (int64_t)nsm) return {16, ty};
     return {16, 14};

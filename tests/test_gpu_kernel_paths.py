@@ -21,8 +21,10 @@ def _problem(nx, ny, seed=5):
                                    sigma=(0.02, 0.1))
 
 
-@pytest.mark.parametrize("shape, tile", [((2, 2), 4), ((16, 4), 4), ((17, 5), 4), ((63, 61), 4), ((256, 152), 4),
-                                         ((257, 153), 8), ((256, 300), 8), ((273, 421), 14)])
+@pytest.mark.parametrize("shape, tile", [((2, 2), (8, 4)), ((8, 4), (8, 4)), ((9, 5), (8, 4)), ((64, 3), (8, 4)),
+                                         ((63, 61), (8, 4)), ((120, 120), (8, 4)), ((120, 121), (16, 4)),
+                                         ((256, 152), (16, 4)), ((257, 153), (16, 8)), ((256, 300), (16, 8)),
+                                         ((273, 421), (16, 14))])
 def test_fp64_auto_tiles_match_split(shape, tile):
     p = _problem(*shape)
     bufs = []
@@ -30,14 +32,15 @@ def test_fp64_auto_tiles_match_split(shape, tile):
         with solver(p, "fp64", kernel=kernel) as s:
             if kernel == 0:
                 st = s.stats()
-                assert (st["tile_x"], st["tile_y"]) == (16, tile)
+                assert (st["tile_x"], st["tile_y"]) == tile
             s.iterate(23, 0.3)
             bufs.append(s.get_messages())
     assert np.array_equal(bufs[0], bufs[1])
 
 
-def test_fp64_interior_update_with_a_prior_mean_matches_split():
-    p = _problem(45, 38)
+@pytest.mark.parametrize("shape", [(45, 38), (145, 138)])
+def test_fp64_interior_update_with_a_prior_mean_matches_split(shape):
+    p = _problem(*shape)
     fb = np.random.default_rng(1).standard_normal(p.n)
     bufs = []
     for kernel in (SPLIT, 0):
