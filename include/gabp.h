@@ -111,7 +111,8 @@ typedef struct {
     int tile_y;       /* fused-kernel tile height in cells; 0 = the default / autotuned shape.
                          GABP_KERNEL_FUSED: 32x8, 32x16, 32x32, 64x8, 64x16, 128x8 (the FP64
                          default: 8x4, 16x4, 16x8 or 16x14 by the grid's size);
-                         GABP_KERNEL_TMA: 30x14, 30x22, 30x30;
+                         GABP_KERNEL_TMA: 30x14, 30x22, 30x30 (the default: 30x14, or 30x2 or
+                         30x6 on small or densely observed grids);
                          GABP_KERNEL_SWEEP: 30x16, 30x32, 30x64, 30x128;
                          GABP_KERNEL_FUSED with alpha = 4: 28x4, 28x8 */
     double tol;       /* relative-residual target of gabp_iterate(n < 0); default 1e-5 */

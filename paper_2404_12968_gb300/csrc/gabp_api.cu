@@ -656,7 +656,7 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
     if (c->kernel == GABP_KERNEL_SWEEP) {
         c->shape = o.tile_y ? gabp::FusedShape{30, o.tile_y} : gabp::FusedShape{30, 64};
     } else if (c->kernel == GABP_KERNEL_TMA) {
-        c->shape = o.tile_x ? gabp::FusedShape{o.tile_x, o.tile_y} : gabp::FusedShape{30, 14};
+        c->shape = o.tile_x ? gabp::FusedShape{o.tile_x, o.tile_y} : gabp::FusedShape{30, gabp::tma_choose_height(p)};
         CK(gabp::make_tma_maps(p, c->shape.tx, c->shape.ty, c->maps, gabp::TMA_MAP_PLANES | gabp::TMA_MAP_OPTR, optr_pad, opitch),
            "tensor map encode");
         c->maps.run = o.tile_run ? o.tile_run : gabp::tma_choose_run(p, c->shape.ty);

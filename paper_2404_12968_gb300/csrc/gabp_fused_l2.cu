@@ -319,6 +319,7 @@ template <int TY> cudaError_t launch_l2_cfg(const DevProblem &p, int run, int sr
     cudaError_t e = l2_persistent_grid<TY>(grid);
     if (e != cudaSuccess) return e;
     TileRuns tr;
+    tr.slices = 1;
     tr.ntx = (p.nx + LTX - 1) / LTX;
     tr.nty = (p.ny + TY - 1) / TY;
     tr.run = run;

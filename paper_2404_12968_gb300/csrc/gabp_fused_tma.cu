@@ -153,8 +153,12 @@ template <int TY, int S, int RW> struct TileLayout {
 
 // BATCH: the tiles of several problems (TmaBatchArgs) instead of one; the per-tile work is the
 // same, on the problem that owns the tile.
-template <int TY, int S, int RW, bool BATCH>
-__global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, RW>::MINB)
+// DENSE (one problem): short tiles for small grids and for many observations per cell, as on the
+// coarse grids of a multigrid hierarchy.  The belief sums keep OBS_AHEAD messages in flight, and
+// tr.slices blocks share a tile: each forms the beliefs, slice 0 updates the cells, and the
+// observation factors are dealt to all of them.  The rule and the figures are at tma_choose_height.
+template <int TY, int S, int RW, bool BATCH, bool DENSE = false>
+__global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, DENSE ? 1 : TileLayout<TY, S, RW>::MINB)
     k_fused_tma(const __grid_constant__ CUtensorMap mplanes, const __grid_constant__ CUtensorMap moptr,
                 const __grid_constant__ DevProblem p, const __grid_constant__ TmaBatchArgs ba, const TileRuns tr,
                 int src, float beta) {
@@ -219,6 +223,7 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
         if (*flag) return;
     }
     TileWalk wk{0, 0, 0, 0};   // single problem: this block's tile
+    const int slice = DENSE ? blockIdx.x % tr.slices : 0;
     if constexpr (BATCH) {
         for (int s = 0; s < S; ++s) {
             const int t = blockIdx.x + s * G;
@@ -226,7 +231,7 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
             fill(s, t);
         }
     } else {
-        wk.start(blockIdx.x, tr);
+        wk.start(DENSE ? blockIdx.x / tr.slices : blockIdx.x, tr);
         if (tid == 0) {
             TileWalk w = wk;
             for (int s = 0; s < S && w.len > 0; ++s, w.next(tr)) issue(s, w.cx, w.ty(tr));
@@ -320,6 +325,8 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
                     mid2 = wptr(gx, gy - 1);
                     lo2 = gx > 0 ? wptr(gx - 1, gy - 1) : mid2;
                     hi2 = last ? mid2 : wptr(gx + 1, gy - 1);
+                }
+                if (!DENSE && m > 0) {
                     const float2 *O2 = reinterpret_cast<const float2 *>(O);   // (eta, Lambda) of k, corner c at 4 k + c
                     if (lo1 < hi1) first1 = O2[4u * (unsigned)lo1 + (lo1 < mid1 ? 1u : 0u)];
                     if (lo2 < hi2) first2 = O2[4u * (unsigned)lo2 + (lo2 < mid2 ? 3u : 2u)];
@@ -334,7 +341,9 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
                 s.add(sm[(DIR_W * RY + ry) * RX + rx + 1]);
                 s.add(sm[(DIR_N * RY + ry - 1) * RX + rx]);
                 s.add(sm[(DIR_S * RY + ry + 1) * RX + rx]);
-                if (m > 0) {
+                if (DENSE) {
+                    add_obs_dense(s, O, lo1, mid1, hi1, lo2, mid2, hi2);
+                } else if (m > 0) {
                     s.add(first1);
                     if (any2) {
                         s.add(second1);
@@ -377,7 +386,7 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
         }
 
         // ---- B: cell factors of the tile, then the observation factors based in it ----
-        for (int ty = warp; ty < TY; ty += TW) {
+        for (int ty = DENSE && slice > 0 ? TY : warp; ty < TY; ty += TW) {
             const int tx = lane, gx = x0 + tx, gy = y0 + ty;
             if (tx >= TTX || gx >= nx || gy >= ny) continue;
             const int64_t c = (int64_t)gy * nx + gx, pc = (int64_t)gy * cur.px + gx;
@@ -417,7 +426,8 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
             const float *YV = (const float *)cur.ovar;
             const int *ob = cur.obase;
             // observation factors go first to the two warps with one cell row fewer
-            for (int q = (tid + TNT - 32 * (TW - 2)) % TNT; q < total; q += TNT) {
+            for (int q = (tid + TNT - 32 * (TW - 2)) % TNT + (DENSE ? slice * TNT : 0); q < total;
+                 q += DENSE ? tr.slices * TNT : TNT) {
                 int lo = 0, hi = TY - 1;   // last row r with rpre[r] <= q
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
@@ -453,8 +463,8 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, TileLayout<TY, S, 
     }
 }
 
-// persistent grid of k_fused_tma<TY, S, RW, BATCH>: SMs x resident blocks (set up once per device)
-template <int TY, int S, int RW, bool BATCH> cudaError_t persistent_grid(int &grid) {
+// persistent grid of k_fused_tma<...>: SMs x resident blocks (set up once per device)
+template <int TY, int S, int RW, bool BATCH, bool DENSE = false> cudaError_t persistent_grid(int &grid) {
     using LY = TileLayout<TY, S, RW>;
     static int grid_cache = 0;
     static int configured_dev = -1;
@@ -462,13 +472,13 @@ template <int TY, int S, int RW, bool BATCH> cudaError_t persistent_grid(int &gr
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_fused_tma<TY, S, RW, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_fused_tma<TY, S, RW, BATCH, DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)LY::bytes);
         if (e != cudaSuccess) return e;
         int nsm = 0, per_sm = 0;
         e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_tma<TY, S, RW, BATCH>, LY::TNT, LY::bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_tma<TY, S, RW, BATCH, DENSE>, LY::TNT, LY::bytes);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         grid_cache = nsm * per_sm;
@@ -478,7 +488,7 @@ template <int TY, int S, int RW, bool BATCH> cudaError_t persistent_grid(int &gr
     return cudaSuccess;
 }
 
-template <int TY, int S, int RW>
+template <int TY, int S, int RW, bool DENSE = false>
 cudaError_t launch_cfg(const DevProblem &p, const TmaMaps &maps, int src, double beta, cudaStream_t st) {
     using LY = TileLayout<TY, S, RW>;
     // the tensor maps' boxes must have been encoded for this tile height (the smem layout and
@@ -486,18 +496,25 @@ cudaError_t launch_cfg(const DevProblem &p, const TmaMaps &maps, int src, double
     if (maps.tx != TTX || maps.ty != TY) return cudaErrorInvalidValue;
     if (maps.run < 1) return cudaErrorInvalidValue;
     int grid = 0;
-    cudaError_t e = persistent_grid<TY, S, RW, false>(grid);
+    cudaError_t e = persistent_grid<TY, S, RW, false, DENSE>(grid);
     if (e != cudaSuccess) return e;
     TileRuns tr;
+    tr.slices = 1;
     tr.run = maps.run;
     tr.ntx = (p.nx + TTX - 1) / TTX;
     tr.nty = (p.ny + TY - 1) / TY;
     const int64_t runs = (int64_t)tr.ntx * ((tr.nty + tr.run - 1) / tr.run);
+    const int slots = grid;
     if (runs < grid) grid = (int)runs;
     tr.step_x = grid % tr.ntx;
     tr.step_b = grid / tr.ntx;
+    if (DENSE && runs <= slots / 2) {   // each block has one run: enough blocks for one round of observations
+        const int64_t rounds = (p.m + runs * LY::TNT - 1) / (runs * LY::TNT), most = slots / runs;
+        tr.slices = (int)(rounds < 1 ? 1 : rounds < most ? rounds : most);
+        grid *= tr.slices;
+    }
     const TmaBatchArgs none{};
-    return launch_pdl(true, k_fused_tma<TY, S, RW, false>, dim3((unsigned)grid), LY::TNT, LY::bytes, st, maps.planes[src], maps.optr, p,
+    return launch_pdl(true, k_fused_tma<TY, S, RW, false, DENSE>, dim3((unsigned)grid), LY::TNT, LY::bytes, st, maps.planes[src], maps.optr, p,
                       none, tr, src, (float)beta);
 }
 
@@ -528,7 +545,7 @@ bool tma_problem_supported(const DevProblem &p) { return p.prec == 0 && p.nx % 4
 cudaError_t make_tma_maps(const DevProblem &p, int tx, int ty, TmaMaps &maps, int parts, const int *optr,
                           int optr_pitch) {
     maps.valid = false;
-    if (!tma_shape_supported(tx, ty)) return cudaErrorInvalidValue;
+    if (!tma_shape_supported(tx, ty) && !(tx == TTX && (ty == 2 || ty == 6))) return cudaErrorInvalidValue;
     auto enc = encoder();
     if (!enc) return cudaErrorNotSupported;
     for (int b = 0; b < 2 && (parts & TMA_MAP_PLANES); ++b) {
@@ -583,6 +600,24 @@ template <int TY> int choose_run(int nx, int ny) {
 }
 }  // namespace
 
+// Short tiles spread a small grid over the SMs and, where nodes have many observations, over the L1
+// caches that their gathers are bound by: 30 x 2 while an SM gets at most one such tile (64^2 with a
+// tenth of an observation per cell 4.1 -> 3.6 us, with 6.4 per cell 19.0 -> 7.0 us, 32^2 with 26 per
+// cell 70 -> 19 us), else 30 x 6 by the same line (128^2: 4.1 -> 4.1, with 1.6 per cell 7.5 -> 5.1 us)
+// or above two observations per cell (512^2: 2 per cell 26.2 -> 25.4 us, 4 per cell 70 -> 44 us; with
+// one per cell 17.3 -> 20.4 us).
+int tma_choose_height(const DevProblem &p) {
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 14;
+    }
+    const int64_t ntx = (p.nx + TTX - 1) / TTX;
+    if (ntx * ((p.ny + 1) / 2) <= nsm) return 2;
+    if (ntx * ((p.ny + 5) / 6) <= nsm || p.m > 2 * p.n) return 6;
+    return 14;
+}
+
 int tma_choose_run(const DevProblem &p, int ty) {
     if (ty == 14) return choose_run<14>(p.nx, p.ny);
     if (ty == 22) return choose_run<22>(p.nx, p.ny);
@@ -600,7 +635,7 @@ cudaError_t launch_batch_cfg(const TmaBatchArgs &ba, const DevProblem &first, in
     if (max_tiles < grid) grid = max_tiles;
     CUtensorMap unused;
     std::memset(&unused, 0, sizeof unused);
-    const TileRuns none{1, 1, 1, 0, 0};
+    const TileRuns none{1, 1, 1, 0, 0, 1};
     return launch_pdl(true, k_fused_tma<TY, 2, 1, true>, dim3((unsigned)grid), LY::TNT, LY::bytes, st, unused, unused, first, ba, none,
                       src, (float)beta);
 }
@@ -640,6 +675,8 @@ size_t tma_smem_bytes(int tx, int ty) {
 cudaError_t launch_tma_iteration(const DevProblem &p, const TmaMaps &maps, int src, double beta,
                                  cudaStream_t st) {
     if (!maps.valid) return cudaErrorInvalidValue;
+    if (maps.ty == 2) return launch_cfg<2, 2, 1, true>(p, maps, src, beta, st);
+    if (maps.ty == 6) return launch_cfg<6, 2, 1, true>(p, maps, src, beta, st);
     if (maps.ty == 14) return launch_cfg<14, 2, 1>(p, maps, src, beta, st);
     if (maps.ty == 22) return launch_cfg<22, 2, 1>(p, maps, src, beta, st);
     if (maps.ty == 30) return launch_cfg<30, 2, 1>(p, maps, src, beta, st);

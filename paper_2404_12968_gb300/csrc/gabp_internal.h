@@ -251,6 +251,9 @@ size_t tma_smem_bytes(int tx, int ty);
 // Tiles per run for a problem on 30 x ty tiles: the length in 1..4 that balances the
 // persistent blocks best (longest on ties).
 int tma_choose_run(const DevProblem &p, int ty);
+// Tile height of a problem whose options leave it open: 14, or 2 or 6 (the dense kernel; not
+// selectable) for problems with many observations per cell.
+int tma_choose_height(const DevProblem &p);
 cudaError_t launch_tma_iteration(const DevProblem &p, const TmaMaps &maps, int src, double beta,
                                  cudaStream_t st);
 

@@ -16,6 +16,7 @@ namespace tiles {
 // the G blocks; step_x = G % ntx and step_b = G / ntx advance a block to its next run.
 struct TileRuns {
     int run, ntx, nty, step_x, step_b;
+    int slices;   // blocks that share a tile (the dense TMA kernel; 1 elsewhere)
 };
 
 // A block's position on its schedule: run (cx, band), tile r of len in that run; len = 0 once
@@ -95,6 +96,30 @@ __device__ __forceinline__ void add_obs_pair2(CompSum2 &s, const float *O, int l
     for (int k = lo; k < hi; ++k) {
         s.add(reinterpret_cast<const float2 *>(O)[4u * (unsigned)k + (unsigned)(k < mid ? cl : cr)]);
     }
+}
+
+// The same for both base rows of a node (corners 1, 0, then 3, 2) where nodes have many
+// observations: the loads of the next OBS_AHEAD messages run while these are added, so that a
+// latency is paid per OBS_AHEAD messages instead of per message.
+constexpr int OBS_AHEAD = 16;
+__device__ __forceinline__ void add_obs_dense(CompSum2 &s, const float *O, int lo1, int mid1, int hi1, int lo2, int mid2,
+                                              int hi2) {
+    const int n1 = hi1 - lo1, nt = n1 + hi2 - lo2;
+    auto load = [&](int t) {
+        const int k = t < n1 ? lo1 + t : lo2 + t - n1;
+        const unsigned c = t < n1 ? (k < mid1 ? 1u : 0u) : (k < mid2 ? 3u : 2u);
+        return t < nt ? reinterpret_cast<const float2 *>(O)[4u * (unsigned)k + c] : f2(0.f, 0.f);
+    };
+    float2 buf[OBS_AHEAD];
+#pragma unroll
+    for (int q = 0; q < OBS_AHEAD; ++q) buf[q] = load(q);
+    for (int t = 0; t < nt; t += OBS_AHEAD)
+#pragma unroll
+        for (int q = 0; q < OBS_AHEAD; ++q) {
+            const float2 x = buf[q];
+            buf[q] = load(t + q + OBS_AHEAD);
+            if (t + q < nt) s.add(x);
+        }
 }
 
 // Factor-to-variable messages of a rank-1 factor with K slots on (eta, Lambda) pairs: the

@@ -100,3 +100,27 @@ def test_fp32_small_or_tiled_odd_grids_keep_the_sweep():
     from paper_2404_12968_gb300 import GabpError
     with pytest.raises(GabpError, match="multiple of 4"):
         solver(_problem(91, 70), "fp32", kernel=3)   # asked for by name: as before
+
+
+@pytest.mark.parametrize("shape, per_cell, tile", [((4, 2), 9, 2), ((32, 32), 25, 2), ((60, 59), 3, 2), ((90, 100), 1, 2), ((90, 101), 1, 6),
+                                                   ((91, 102), 5, 6), ((130, 67), 2, 6), ((301, 160), 3, 6),
+                                                   ((300, 300), 1, 14)])
+def test_fp32_short_tiles_match_split(shape, per_cell, tile):
+    """The short TMA tiles of small and of densely observed grids (tiles shared by several blocks, the
+    belief sums of many observations per node) against the split kernels."""
+    nx, ny = shape
+    rng = np.random.default_rng(11)
+    m = per_cell * nx * ny + 1
+    # half of the observations on one corner cell of every fourth column: long, uneven ranges
+    xy = rng.uniform(0, 1, (m, 2)) * np.array([nx - 1.0, ny - 1.0])
+    xy[::2, 0] = np.minimum(np.floor(xy[::2, 0] / 4) * 4, nx - 2) + 0.5
+    y, nv = rng.standard_normal(m), rng.uniform(0.01, 0.1, m)
+    from paper_2404_12968_gb300 import Solver
+    bufs = []
+    for kernel in (SPLIT, 0):
+        with Solver(nx=nx, ny=ny, kappa=0.2, obs_xy=xy, y=y, noise_var=nv, precision="fp32", kernel=kernel) as s:
+            if kernel == 0 and nx % 4 == 0 or nx * ny >= 4096:
+                assert kernel or (s.stats()["kernel"], s.stats()["tile_y"]) == (3, tile)
+            s.iterate(23, 0.5)
+            bufs.append(s.get_messages())
+    assert np.array_equal(bufs[0], bufs[1])
