@@ -177,12 +177,16 @@ cudaError_t launch_iteration(gabp_ctx *c, int src, double beta, cudaStream_t st)
     return gabp::launch_fused_iteration(c->p, src, beta, c->shape, st);
 }
 
-// A kernel's bounded wait gave up: report it (and clear the flag).
-int check_device_error(gabp_ctx *c) {
-    int h = 0;
-    CK(cudaMemcpyAsync(&h, c->p.err, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "error flag copy");
-    CK(cudaStreamSynchronize(c->stream), "error flag sync");
-    if (h) {
+constexpr int NSCAL = 4;   // doubles at p.scal in front of the error flag
+
+// Copy p.scal[first ..] and the error flag behind it to the pinned mirror and wait for the stream: the
+// one synchronisation of a call that has launched iterations.  A kernel's bounded wait that gave up
+// is reported (and the flag cleared).
+int sync_scalars(gabp_ctx *c, int first, const char *what) {
+    CK(cudaMemcpyAsync(c->hscal + first, c->p.scal + first, (NSCAL + 1 - first) * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
+       what);
+    CK(cudaStreamSynchronize(c->stream), what);
+    if (*(const int *)(c->hscal + NSCAL)) {
         CK(cudaMemsetAsync(c->p.err, 0, sizeof(int), c->stream), "error flag reset");
         CK(cudaStreamSynchronize(c->stream), "error flag sync");
         return fail(c, GABP_ERR_TIMEOUT, "a bounded wait inside the iteration kernel gave up");
@@ -244,9 +248,7 @@ int run_iterations(gabp_ctx *c, int64_t count, double beta) {
 
 int compute_residual(gabp_ctx *c, double *out) {
     CK(gabp::launch_residual(c->p, c->cur, c->stream), "residual kernels");
-    CK(cudaMemcpyAsync(c->hscal, c->p.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-       "residual copy");
-    CK(cudaStreamSynchronize(c->stream), "residual sync");
+    if (int rc = sync_scalars(c, 0, "residual sync")) return rc;
     const double r2 = c->hscal[0], b2 = c->hscal[1];
     *out = b2 > 0.0 ? std::sqrt(r2) / std::sqrt(b2) : std::sqrt(r2);
     c->last_res = *out;
@@ -257,9 +259,7 @@ int compute_residual(gabp_ctx *c, double *out) {
 // |m_t - m_{t-1}|, the quantity of the early-stopping rule (App. B)
 int compute_msg_change(gabp_ctx *c, double *out) {
     CK(gabp::launch_msg_change(c->p, c->cur, c->p.scal + 2, c->stream), "message change kernels");
-    CK(cudaMemcpyAsync(c->hscal + 2, c->p.scal + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-       "message change copy");
-    CK(cudaStreamSynchronize(c->stream), "message change sync");
+    if (int rc = sync_scalars(c, 2, "message change sync")) return rc;
     *out = c->hscal[2] / (2.0 * (double)c->edges);
     return GABP_OK;
 }
@@ -589,15 +589,15 @@ int create_impl(gabp_ctx *c, gabp_grid grid, double kappa_h, const gabp_prior *p
     p.e64 = (double *)q;
     if ((rc = dalloc(c, &q, gabp::RES_BLOCKS * sizeof(double), "alloc partial sums"))) return rc;
     p.part = (double *)q;
-    if ((rc = dalloc(c, &q, 4 * sizeof(double), "alloc scalars"))) return rc;   // |r|^2, |b|^2, message change
+    // |r|^2, |b|^2, message change (rank-1, pairwise), then the error flag: one copy brings a result
+    // and the flag to the host
+    if ((rc = dalloc(c, &q, (NSCAL + 1) * sizeof(double), "alloc scalars"))) return rc;
     p.scal = (double *)q;
-    if ((rc = dalloc(c, &q, sizeof(int), "alloc error flag"))) return rc;
-    p.err = (int *)q;
-    CK(cudaMemsetAsync(p.err, 0, sizeof(int), c->stream), "memset");
+    p.err = (int *)(p.scal + NSCAL);
     if ((rc = dalloc(c, &q, 2 * (size_t)n * sizeof(double), "alloc staging"))) return rc;
     c->stage = (double *)q;
-    CK(cudaMallocHost((void **)&c->hscal, 4 * sizeof(double)), "alloc pinned scalars");
-    CK(cudaMemsetAsync(p.scal, 0, 4 * sizeof(double), c->stream), "memset");
+    CK(cudaMallocHost((void **)&c->hscal, (NSCAL + 1) * sizeof(double)), "alloc pinned scalars");
+    CK(cudaMemsetAsync(p.scal, 0, (NSCAL + 1) * sizeof(double), c->stream), "memset");
 
     // upload the caller's observations as they are, then on the GPU: base cells, the stable
     // sort by base cell (sorted raw data kept in c->dsorted: x, y pairs, values, variances),
@@ -770,8 +770,7 @@ int gabp_iterate(gabp_ctx *c, int n_iters, double damping) {
         const int64_t iters0 = c->iters;
         int rc = run_iterations(c, n_iters, damping);
         if (rc) return rc;
-        CK(cudaStreamSynchronize(c->stream), "iterate sync");
-        rc = check_device_error(c);
+        rc = sync_scalars(c, NSCAL, "iterate sync");
         if (rc) {   // a kernel gave up: point back at the messages the call started from
             c->cur = cur0;
             c->iters = iters0;
@@ -791,9 +790,7 @@ int gabp_iterate(gabp_ctx *c, int n_iters, double damping) {
             return fail(c, GABP_ERR_TIMEOUT, "max_iters reached with residual " + std::to_string(res));
         int64_t chunk = c->opt.check_every;
         if (done + chunk > c->opt.max_iters) chunk = c->opt.max_iters - done;
-        rc = run_iterations(c, chunk, damping);
-        if (rc) return rc;
-        if ((rc = check_device_error(c))) return rc;
+        if ((rc = run_iterations(c, chunk, damping))) return rc;   // checked with the next residual
         done += chunk;
     }
 }
@@ -818,7 +815,7 @@ int gabp_iterate_early_stop(gabp_ctx *c, int max_iters, double damping, double t
     if (stopped_at) *stopped_at = 0;
     // iterations 1 and 2 of this call; the change of iteration 2 is the reference
     int rc = run_iterations(c, 2, damping);
-    if (rc || (rc = check_device_error(c))) return rc;
+    if (rc) return rc;
     double ref = 0.0, d = 0.0;
     if ((rc = compute_msg_change(c, &ref))) return rc;
     if (!std::isfinite(ref)) return fail(c, GABP_ERR_DIVERGED, "message change is not finite");
@@ -827,8 +824,7 @@ int gabp_iterate_early_stop(gabp_ctx *c, int max_iters, double damping, double t
         if (t >= max_iters) return fail(c, GABP_ERR_TIMEOUT, "max_iters reached before the early-stopping rule held");
         int64_t chunk = check_every;
         if (t + chunk > max_iters) chunk = max_iters - t;
-        rc = run_iterations(c, (int)chunk, damping);
-        if (rc || (rc = check_device_error(c))) return rc;
+        if ((rc = run_iterations(c, (int)chunk, damping))) return rc;   // checked with the message change
         t += chunk;
         if ((rc = compute_msg_change(c, &d))) return rc;
         if (!std::isfinite(d)) return fail(c, GABP_ERR_DIVERGED, "message change is not finite");
@@ -1233,13 +1229,10 @@ int batch_set_height(gabp_batch *b, int H) {
     return GABP_OK;
 }
 
-// A bounded wait of the batched TMA kernel gave up: report it (and clear the flag).
-int batch_check_error(gabp_batch *b) {
-    if (b->kernel != GABP_KERNEL_TMA) return GABP_OK;
-    int h = 0;
-    BK(cudaMemcpyAsync(&h, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream), "error flag copy");
-    BK(cudaStreamSynchronize(b->stream), "error flag sync");
-    if (h) {
+// A bounded wait of the batched TMA kernel gave up: report it (and clear the flag).  The flag is
+// behind the residuals in the pinned mirror (copied by the caller before its synchronisation).
+int batch_take_error(gabp_batch *b) {
+    if (*(const int *)(b->h_scal + 2 * b->inst.size())) {
         BK(cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream), "error flag reset");
         BK(cudaStreamSynchronize(b->stream), "error flag sync");
         return bfail(b, GABP_ERR_TIMEOUT, "a bounded wait inside the batched iteration kernel gave up");
@@ -1317,6 +1310,8 @@ int batch_residuals(gabp_batch *b) {
                 le = cudaMemcpyAsync(b->h_scal + 2 * i, b->inst[i]->p.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                                      b->cap);
         }
+        if (le == cudaSuccess)
+            le = cudaMemcpyAsync(b->h_scal + 2 * count, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->cap);
         cudaError_t ee = cudaStreamEndCapture(b->cap, &g);
         if (le != cudaSuccess) {
             if (g) cudaGraphDestroy(g);
@@ -1332,7 +1327,7 @@ int batch_residuals(gabp_batch *b) {
     }
     BK(cudaGraphLaunch(b->g_res, b->stream), "residual graph launch");
     BK(cudaStreamSynchronize(b->stream), "residual sync");
-    if (int rc = batch_check_error(b)) return rc;
+    if (int rc = batch_take_error(b)) return rc;
     if (b->cur != 0) {   // only the parity-0 graph is kept
         cudaGraphExecDestroy(b->g_res);
         b->g_res = nullptr;
@@ -1487,7 +1482,7 @@ int batch_create_impl(gabp_batch *b, int count, const gabp_problem *problems) {
     BK(cudaMalloc((void **)&b->d_prefix, sizeof(int) * (count + 1)), "alloc strip offsets");
     BK(cudaMalloc((void **)&b->d_active, sizeof(int) * count), "alloc active flags");
     BK(cudaMallocHost((void **)&b->h_active, sizeof(int) * count), "alloc pinned flags");
-    BK(cudaMallocHost((void **)&b->h_scal, 2 * sizeof(double) * count), "alloc pinned scalars");
+    BK(cudaMallocHost((void **)&b->h_scal, sizeof(double) * (2 * (size_t)count + 1)), "alloc pinned scalars");
     std::vector<gabp::DevProblem> table(count);
     for (int i = 0; i < count; ++i) {
         table[i] = b->inst[i]->p;
@@ -1570,8 +1565,9 @@ int gabp_batch_iterate(gabp_batch *b, int n_iters, double damping) {
         if (rc) return rc;
         rc = batch_run(b, n_iters, damping);
         if (rc) return rc;
+        BK(cudaMemcpyAsync(b->h_scal + 2 * count, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream), "error flag copy");
         BK(cudaStreamSynchronize(b->stream), "iterate sync");
-        return batch_check_error(b);
+        return batch_take_error(b);
     }
     int rc;
     if (b->cur == 1) {   // checks run at parity 0
@@ -1707,7 +1703,9 @@ struct gabp_mg {
     gabp_ctx *target = nullptr;
     int levels = 0;
     std::vector<gabp_ctx *> lv;   // lv[k] = level k (k >= 1); lv[0] unused (the target)
-    double *mu[2] = {nullptr, nullptr}, *q[2] = {nullptr, nullptr};   // marginal buffers (target size)
+    double *buf = nullptr;    // marginal buffers, four of the target's size, from the contexts' pool
+    bool pooled = false;
+    double *mu[2] = {nullptr, nullptr}, *q[2] = {nullptr, nullptr};
     std::string err;
 };
 
@@ -1732,9 +1730,12 @@ void mg_free(gabp_mg *g) {
         if (c) gabp_destroy(c);
     g->lv.clear();
     for (int i = 0; i < 2; ++i) {
-        if (g->mu[i]) cudaFree(g->mu[i]);
-        if (g->q[i]) cudaFree(g->q[i]);
         g->mu[i] = g->q[i] = nullptr;
+    }
+    if (g->buf) {
+        if (g->pooled) cudaFreeAsync(g->buf, g->target->stream);   // every call has waited for its kernels
+        else cudaFree(g->buf);
+        g->buf = nullptr;
     }
 }
 
@@ -1813,11 +1814,20 @@ int gabp_mg_create(gabp_mg **out, gabp_ctx *ctx, int levels) {
         rc = gabp_create(&g->lv[(size_t)k], gk, ctx->kappa * s, &pk, m, xy.data(), ctx->hy.data(), ctx->hvar.data(), &ok);
         if (rc) fail(ctx, rc, "multigrid level " + std::to_string(k) + ": " + gabp_create_error());
     }
-    for (int i = 0; i < 2 && rc == GABP_OK; ++i) {
-        const size_t bytes = (size_t)ctx->p.n * sizeof(double);
-        if (cudaMalloc((void **)&g->mu[i], bytes) != cudaSuccess || cudaMalloc((void **)&g->q[i], bytes) != cudaSuccess) {
+    if (rc == GABP_OK) {
+        const size_t n = (size_t)ctx->p.n, bytes = 4 * n * sizeof(double);
+        cudaMemPool_t pool = context_pool(ctx->dev);
+        g->pooled = pool != nullptr;
+        if ((pool ? cudaMallocFromPoolAsync((void **)&g->buf, bytes, pool, ctx->stream) : cudaMalloc((void **)&g->buf, bytes)) !=
+            cudaSuccess) {
             cudaGetLastError();
+            g->buf = nullptr;
             rc = fail(ctx, GABP_ERR_OOM, "multigrid buffers");
+        } else {
+            for (int i = 0; i < 2; ++i) {
+                g->mu[i] = g->buf + 2 * i * n;
+                g->q[i] = g->mu[i] + n;
+            }
         }
     }
     if (rc) {
