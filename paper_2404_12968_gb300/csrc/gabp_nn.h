@@ -61,8 +61,8 @@ int64_t wgrad_chunks(const WgradArgs &a);
 cudaError_t conv_wgrad(WgradArgs a, float *dw, cudaStream_t st);
 // Weight gradient on the tcgen05 tensor cores (gabp_nn_tc.cu): dw[co][t][ci] = sum over the
 // pixels p of g[p][co] in[p + d_t][ci] (zero outside the image), as partial sums over pixel
-// chunks in part (at most part_cap floats) reduced into dw in chunk order.  Cin a multiple
-// of 16 (at most 256 per block of N), any Cout (blocks of 128; rows past Cout are zero).
+// chunks in part (at most part_cap floats) reduced into dw in chunk order.  Cin 16 or a multiple
+// of 32 (at most 256 per block of N), Cout a multiple of 32 (blocks of 64 or 128).
 struct TcWgradArgs {
     const __nv_bfloat16 *g;     // [B][H][W][Cout]
     const __nv_bfloat16 *in;    // [B][H][W][Cin]
@@ -71,7 +71,7 @@ struct TcWgradArgs {
     int *err;                   // device flag, set if a bounded wait ran out
     int B, H, W, Cin, Cout, T;
     // set by tc_wgrad
-    int M, N, nbn, nbm, chunks, stages, ky, ga, tpc, ngroups;
+    int M, N, nbn, nbm, chunks, stages, ky, ga, cbx, tpc, ngroups;
     int64_t ktiles, tiles_x, tiles_y, per_chunk;
 };
 cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st);

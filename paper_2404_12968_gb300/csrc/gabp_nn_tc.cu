@@ -5,12 +5,13 @@
 // M = pixels, N = output channels, K = taps x input channels.  A block computes tiles of
 // 16 x 8 output pixels (M = 128, GEMM row m = 8 y + x) times N output channels:
 //
-//   * the input tile plus a one-pixel halo, 18 x 10 pixels, is loaded by TMA once per block of
-//     16 input channels, as two [18][10][8] BF16 chunks (zero fill outside the image is the
-//     convolution's zero padding).  Every tap (dy, dx) is then the same shared-memory matrix at
-//     another start address: start + ((dy + 1) * 10 + (dx + 1)) * 16 bytes, 16 bytes between
-//     the 8 pixels of a row, 160 bytes between pixel rows, one chunk pitch between the two
-//     8-channel halves of K.  No input pixel is copied more than once per channel block.
+//   * the input tile plus a one-pixel halo (3x3 taps), 18 x 10 pixels, is loaded by TMA once per
+//     block of CB = 32 or 16 input channels, as rows of one pixel's channels swizzled over 64 or 32
+//     bytes (zero fill outside the image is the convolution's zero padding).  Every tap (dy, dx) is
+//     then the same shared-memory matrix at another start address, (dy + 1) * 10 + (dx + 1) pixels
+//     on: the swizzle is a function of the address, so it follows.  No input pixel is copied more
+//     than once per channel block.  (Unswizzled, the operand's core matrices are 16 bytes wide, the
+//     copies had rows of 16 bytes and a pixel's channel block took two of them.)
 //   * the weights of that channel block are a prepacked [tap][8-channel half][N][8] BF16 slab
 //     (one bulk copy), the K-major canonical layout of the MMA's B operand.
 //   * one MMA per tap (K = 16) accumulates into one of two TMEM accumulators of N FP32
@@ -25,11 +26,10 @@
 //
 // The weight gradient of training, dw[co][t][ci] = sum_p g[p][co] in[p + d_t][ci], is a GEMM
 // with M = output channels, N = input channels and K = pixels, per tap (k_tc_wgrad).  Both
-// operands come straight from the NHWC tensors: 8 channels of one pixel are 16 contiguous
-// bytes, so a tile of 64 pixels (16 x 4) x 8 channels is one MN-major core-matrix column
-// (8 pixels = 128 bytes per core matrix along K), loaded by one 5-D TMA copy per operand
-// (channel-in-group, x, y, image, channel group) with zero fill outside the image for the tap
-// shift.  One accumulator of N FP32 columns per block covers a chunk of pixel tiles; the
+// operands come straight from the NHWC tensors as MN-major matrices: a pixel's 32 channels are 64
+// contiguous bytes, a row of a swizzle atom, and a tile of pixels is loaded by one 5-D TMA copy per
+// operand (channel in block, x, y, image, channel block) with zero fill outside the image for the tap
+// shift.  One accumulator of N FP32 columns per tap and block covers a chunk of pixel tiles; the
 // epilogue writes it to a partial-sum buffer that a second kernel reduces in chunk order.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -45,10 +45,12 @@ namespace {
 
 constexpr int TC_THREADS = 192;
 constexpr int TILE_Y = 16, TILE_X = 8;          // output pixels per tile (M = 128)
-constexpr int HALO_Y = TILE_Y + 2, HALO_X = TILE_X + 2;
-constexpr uint32_t CHUNK_BYTES = HALO_Y * HALO_X * 16;   // one 8-channel halo chunk (2880 B)
-constexpr uint32_t CHUNK_PITCH = 2944;                   // chunk pitch in shared memory (128-aligned)
-constexpr uint32_t HALO_BYTES = 2 * CHUNK_PITCH;          // 16 channels
+// the staged input of T taps and CB channels: pixels, bytes copied, stage bytes (a multiple of 1024,
+// so that every stage starts a swizzle pattern)
+template <int T, int CB> struct InTile {
+    static constexpr int X = TILE_X + (T == 9 ? 2 : 0), Y = TILE_Y + (T == 9 ? 2 : 0);
+    static constexpr uint32_t ROW = CB * 2, BYTES = X * Y * ROW, PITCH = (BYTES + 1023) & ~1023u;
+};
 
 __device__ __forceinline__ uint32_t saddr(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
@@ -99,6 +101,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
 }
+// the same with a 64-byte (CB = 32) or 32-byte (CB = 16) swizzle
+template <int CB> __device__ __forceinline__ uint64_t smem_desc_sw(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+    return smem_desc(addr, lbo, sbo) | ((uint64_t)(CB == 32 ? 4 : 6) << 61);
+}
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3, int c4,
                                             uint32_t bar) {
     asm volatile(
@@ -148,26 +154,37 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void store16_bf16(__nv_bfloat16 *dst, const __nv_bfloat16 (&v)[16]) {
-    uint4 q[2];
-    __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(q);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) h[j] = v[j];
-    reinterpret_cast<uint4 *>(dst)[0] = q[0];
-    reinterpret_cast<uint4 *>(dst)[1] = q[1];
+// BF16 pairs in one register (low half first)
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&p);
+}
+__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+__device__ __forceinline__ uint32_t relu_bf16(uint32_t v) {   // max(., 0); rounding and max commute
+    const __nv_bfloat162 m = __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&v), __nv_bfloat162(__float2bfloat16(0.f), __float2bfloat16(0.f)));
+    return *reinterpret_cast<const uint32_t *>(&m);
+}
+__device__ __forceinline__ uint32_t positive_mask(uint32_t v) {   // all ones in the halves above zero
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&v), __nv_bfloat162(__float2bfloat16(0.f), __float2bfloat16(0.f)));
+}
+__device__ __forceinline__ void store16_bf16(__nv_bfloat16 *dst, const uint32_t (&v)[8]) {
+    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4 *>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
 }
 
-template <int N, int T>
-__global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ CUtensorMap in_map, TcConvArgs a) {
-    constexpr uint32_t WBYTES = (uint32_t)T * 32 * N;          // weight slab of one channel block
+template <int N, int T, int CB>
+__global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant__ CUtensorMap in_map, TcConvArgs a) {
+    using IN = InTile<T, CB>;
+    constexpr uint32_t WBYTES = (uint32_t)T * 2 * CB * N;      // weight slab of one channel block
     extern __shared__ __align__(1024) unsigned char smem[];
     const int S = a.stages;
-    const int nkb = a.Cin / 16;
+    const int nkb = a.Cin / CB;
     // resident weights: all nkb slabs stay in shared memory and the ring carries halos only;
     // otherwise every stage carries a halo and its weight slab
     const bool resident = a.resident != 0;
     const uint32_t wres = resident ? (uint32_t)nkb * WBYTES : 0u;   // resident weight bytes
-    const uint32_t STAGE = resident ? HALO_BYTES : HALO_BYTES + WBYTES;   // multiples of 128
+    const uint32_t STAGE = resident ? IN::PITCH : IN::PITCH + WBYTES;   // multiples of 1024
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + wres + (size_t)S * STAGE);
     // full[S], empty[S], acc_full[2], acc_empty[2], weights
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * S + 5);
@@ -206,12 +223,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
 
     const int64_t ntiles = a.ntiles;
     auto tile_coords = [&](int64_t tile, int &b, int &y0, int &x0, int &nb) {
-        nb = (int)(tile % a.nblocks);
-        int64_t r = tile / a.nblocks;
-        const int tx = (int)(r % a.tiles_x);
-        r /= a.tiles_x;
-        const int ty = (int)(r % a.tiles_y);
-        b = (int)(r / a.tiles_y);
+        uint32_t r = (uint32_t)tile / (uint32_t)a.nblocks;   // fewer than 2^31 tiles (checked on the host)
+        nb = (int)((uint32_t)tile - r * (uint32_t)a.nblocks);
+        const uint32_t q = r / (uint32_t)a.tiles_x;
+        const int tx = (int)(r - q * (uint32_t)a.tiles_x);
+        b = (int)(q / (uint32_t)a.tiles_y);
+        const int ty = (int)(q - (uint32_t)b * (uint32_t)a.tiles_y);
         y0 = ty * TILE_Y;
         x0 = tx * TILE_X;
     };
@@ -236,11 +253,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
                         break;
                     }
                     const uint32_t st = ring + (uint32_t)s * STAGE;
-                    mbar_expect_tx(full(s), 2 * CHUNK_BYTES + (resident ? 0u : WBYTES));
-                    tma_load_4d(st, &in_map, 16 * kb, x0 - 1, y0 - 1, b, full(s));
-                    tma_load_4d(st + CHUNK_PITCH, &in_map, 16 * kb + 8, x0 - 1, y0 - 1, b, full(s));
+                    mbar_expect_tx(full(s), IN::BYTES + (resident ? 0u : WBYTES));
+                    tma_load_4d(st, &in_map, CB * kb, x0 - (T == 9), y0 - (T == 9), b, full(s));
                     if (!resident)
-                        bulk_load(st + HALO_BYTES, a.wpk + ((int64_t)nb * nkb + kb) * (WBYTES / 2), WBYTES, full(s));
+                        bulk_load(st + IN::PITCH, a.wpk + ((int64_t)nb * nkb + kb) * (WBYTES / 2), WBYTES, full(s));
                 }
             }
         }
@@ -248,7 +264,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
         // ---- MMA issuer ----
         const uint32_t idesc = instr_desc<N>();
         const bool one = elect_lane();
-        const uint64_t ad0 = smem_desc(0, CHUNK_PITCH, HALO_X * 16), bd0 = smem_desc(0, N * 16, 128);
+        const uint64_t ad0 = smem_desc_sw<CB>(0, 16, IN::X * IN::ROW), bd0 = smem_desc(0, N * 16, 128);
         uint32_t it = 0;
         int lt = 0;
         bool ok = !resident || mbar_wait(wbar, 0);
@@ -267,14 +283,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
                 if (__any_sync(0xffffffffu, !ok)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t st = ring + s * STAGE;
-                const uint64_t ad = ad0 + (st >> 4), bd = bd0 + ((resident ? sbase + (uint32_t)kb * WBYTES : st + HALO_BYTES) >> 4);
+                const uint64_t ad = ad0 + (st >> 4), bd = bd0 + ((resident ? sbase + (uint32_t)kb * WBYTES : st + IN::PITCH) >> 4);
                 if (one) {
 #pragma unroll
-                    for (int t = 0; t < T; ++t) {
-                        const int dy = T == 9 ? t / 3 - 1 : 0, dx = T == 9 ? t % 3 - 1 : 0;
-                        umma(d, ad + (uint64_t)((dy + 1) * HALO_X + (dx + 1)), bd + (uint64_t)(t * 2 * N), idesc,
-                             (kb > 0 || t > 0) ? 1u : 0u);
-                    }
+                    for (int j = 0; j < CB / 16; ++j)   // 16 channels: one MMA per tap
+#pragma unroll
+                        for (int t = 0; t < T; ++t)
+                            umma(d, ad + (uint64_t)((t / 3 * IN::X + t % 3) * (int)(IN::ROW / 16) + 2 * j),
+                                 bd + (uint64_t)((j * T + t) * 2 * N), idesc, (kb > 0 || j > 0 || t > 0) ? 1u : 0u);
                     umma_commit(empty(s));   // the stage is free once these MMAs have read it
                 }
                 __syncwarp();
@@ -308,36 +324,35 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
             }
 #pragma unroll 1
             for (int c = 0; c < N; c += 16) {
-                uint32_t r[16];
+                uint32_t r[16], v[8];   // 16 channels: FP32 sums, BF16 pairs
                 tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * N + c), r);
-                __nv_bfloat16 v[16];
+                const float4 *bias4 = reinterpret_cast<const float4 *>(a.bias + co0 + c);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    float f = __uint_as_float(r[j]) + a.bias[co0 + c + j];
-                    if (a.relu) f = fmaxf(f, 0.f);
-                    v[j] = __float2bfloat16(f);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 bv = bias4[j];
+                    v[2 * j] = pack_bf16(__uint_as_float(r[4 * j]) + bv.x, __uint_as_float(r[4 * j + 1]) + bv.y);
+                    v[2 * j + 1] = pack_bf16(__uint_as_float(r[4 * j + 2]) + bv.z, __uint_as_float(r[4 * j + 3]) + bv.w);
                 }
-                if (a.mask && valid) {   // the ReLU's backward: zero where its output was not positive
-                    uint4 mq[2];
-                    const uint4 *ms = reinterpret_cast<const uint4 *>(a.mask + pix * a.Cout + co0 + c);
-                    mq[0] = ms[0];
-                    mq[1] = ms[1];
-                    const __nv_bfloat16 *mh = reinterpret_cast<const __nv_bfloat16 *>(mq);
+                if (a.relu)
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (!(__bfloat162float(mh[j]) > 0.f)) v[j] = __float2bfloat16(0.f);
+                    for (int j = 0; j < 8; ++j) v[j] = relu_bf16(v[j]);
+                if (a.mask && valid) {   // the ReLU's backward: zero where its output was not positive
+                    const uint4 *ms = reinterpret_cast<const uint4 *>(a.mask + pix * a.Cout + co0 + c);
+                    const uint4 m0 = ms[0], m1 = ms[1];
+                    const uint32_t mk[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] &= positive_mask(mk[j]);
                 }
                 if (a.out && valid) store16_bf16(a.out + pix * a.Cout + co0 + c, v);
                 if (a.pool_out) {
                     // 2x2 sum, scaled: (y, x), (y, x+1), (y+1, x), (y+1, x+1) are lanes +0, +1, +8, +9
-                    __nv_bfloat16 pv[16];
+                    uint32_t pv[8];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float f = __bfloat162float(v[j]);
-                        const float f1 = __shfl_down_sync(0xffffffffu, f, 1);
-                        const float f8 = __shfl_down_sync(0xffffffffu, f, 8);
-                        const float f9 = __shfl_down_sync(0xffffffffu, f, 9);
-                        pv[j] = __float2bfloat16(a.pool_scale * (((f + f1) + f8) + f9));
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t v1 = __shfl_down_sync(0xffffffffu, v[j], 1), v8 = __shfl_down_sync(0xffffffffu, v[j], 8);
+                        const uint32_t v9 = __shfl_down_sync(0xffffffffu, v[j], 9);
+                        pv[j] = pack_bf16(a.pool_scale * (((bf_lo(v[j]) + bf_lo(v1)) + bf_lo(v8)) + bf_lo(v9)),
+                                          a.pool_scale * (((bf_hi(v[j]) + bf_hi(v1)) + bf_hi(v8)) + bf_hi(v9)));
                     }
                     if (valid && !(xx & 1) && !(yy & 1)) {
                         const int64_t q = ((int64_t)b * (a.H / 2) + gy / 2) * (a.W / 2) + gx / 2;
@@ -350,21 +365,20 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
                     for (int q = 0; q < 4; ++q) {
                         const int fy = 2 * gy + (q >> 1), fx = 2 * gx + (q & 1);
                         const int64_t fp = ((int64_t)b * (2 * a.H) + fy) * (2 * a.W) + fx;
-                        const __nv_bfloat16 *sk = a.up_skip + fp * a.Cout + co0 + c;
-                        uint4 sq[2];
-                        sq[0] = reinterpret_cast<const uint4 *>(sk)[0];
-                        sq[1] = reinterpret_cast<const uint4 *>(sk)[1];
-                        const __nv_bfloat16 *sh = reinterpret_cast<const __nv_bfloat16 *>(sq);
-                        __nv_bfloat16 u[16];
+                        const uint4 *sk = reinterpret_cast<const uint4 *>(a.up_skip + fp * a.Cout + co0 + c);
+                        const uint4 s0 = sk[0], s1 = sk[1];
+                        const uint32_t sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+                        uint32_t u[8];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) u[j] = __float2bfloat16(__bfloat162float(v[j]) + __bfloat162float(sh[j]));
+                        for (int j = 0; j < 8; ++j)
+                            u[j] = pack_bf16(bf_lo(v[j]) + bf_lo(sv[j]), bf_hi(v[j]) + bf_hi(sv[j]));
                         store16_bf16(a.up_out + fp * a.Cout + co0 + c, u);
                     }
                 }
                 if (a.head_w) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        const float f = __bfloat162float(v[j]);
+                        const float f = j & 1 ? bf_hi(v[j >> 1]) : bf_lo(v[j >> 1]);
                         h0 = fmaf(a.head_w[c + j], f, h0);
                         h1 = fmaf(a.head_w[a.Cout + c + j], f, h1);
                     }
@@ -393,25 +407,37 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_conv(const __grid_constant__ 
 constexpr int WG_THREADS = 192;
 constexpr int WG_KX = 16;                               // pixels per tile row (one MMA, K = 16)
 
-// Block: a group of taps [t0, t0 + tpc), output-channel block mb (128), input-channel block nb
-// (N), pixel-tile chunk.  A tile is 16 x KY pixels.  Shared memory per stage:
-//   A [M / 8 groups][KY][16][8]: g at the tile's pixels, 8 output channels per group;
-//   B [N / 8 groups][KY + 2 h][16 + 2 h][8]: the input at the tile's pixels plus a one-pixel
-//     halo (h = 1 for 3x3 taps), so that every tap (dy, dx) of a tile row is the same matrix at
-//     another start address, ((row + h + dy) (16 + 2 h) + h + dx) 16 bytes.
-// Canonical MN-major, no swizzle: core matrix = 8 pixels x 8 channels (128 B), K-direction core
-// matrices 128 B apart (LBO), channel-direction one group apart (SBO).  One MMA per tile row and
-// tap accumulates into that tap's N TMEM columns.  Only the A groups of existing output channels
-// are copied (a.ga of them); the rest of A is zeroed once and stays zero.
+// bytes of a stage: the copied operands, and no less than an A operand of M rows reaches
+__host__ __device__ inline uint32_t wg_stage_bytes(int M, int ga, int N, int ky, int h) {
+    const uint32_t ag = (uint32_t)(WG_KX * ky) * 64;
+    const uint32_t both = (uint32_t)ga * ag + (uint32_t)(N * (WG_KX + 2 * h) * (ky + 2 * h)) * 2;
+    const uint32_t reach = (uint32_t)(M / 32) * ag;
+    return ((both > reach ? both : reach) + 1023u) & ~1023u;
+}
+
+// Block: a group of taps [t0, t0 + tpc), output-channel block mb (of M), input-channel block nb (N),
+// pixel-tile chunk.  A tile is 16 x KY pixels.  Shared memory per stage, in blocks of 32 channels (the
+// input's 16 where it has only 16) whose pixels are rows of 64 (32) bytes, swizzled:
+//   A [channel block][KY][16]: g at the tile's pixels;
+//   B [channel block][KY + 2 h][16 + 2 h]: the input at the tile's pixels plus a one-pixel halo (h = 1
+//     for 3x3 taps), so that every tap (dy, dx) of a tile row is the same matrix at another start
+//     address, (row + h + dy) (16 + 2 h) + h + dx pixels on (the swizzle is a function of the address).
+// MN-major: 8 pixels x one channel block are a swizzle atom, the K-direction atoms follow each other
+// (SBO), channel blocks are one block apart (LBO).  One MMA per tile row and tap accumulates into that
+// tap's N TMEM columns.  With fewer output channels than M the A operand runs on into the stage's B:
+// those accumulator rows are not read.  (As [8-channel group][pixel] tiles without a swizzle the copies
+// had 16-byte rows, of which the TMA unit moves one per 2.4 cycles: 75 -> 42 us for 128 x 128 x 9 over
+// 131 k pixels, 101 -> 54 us for 256 x 256 x 9 over 33 k.)
 __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__ CUtensorMap gmap,
                                                          const __grid_constant__ CUtensorMap xmap, TcWgradArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int S = a.stages, N = a.N, KY = a.ky, h = a.T == 9 ? 1 : 0;
     const int HX = WG_KX + 2 * h, HY = KY + 2 * h;
-    const uint32_t AG = (uint32_t)(WG_KX * KY * 16), BG = (uint32_t)(HX * HY * 16);
-    const int MG = a.M / 8;   // groups of the A operand
-    const uint32_t ABYTES = (uint32_t)MG * AG;
-    const uint32_t STAGE = (ABYTES + (uint32_t)(N / 8) * BG + 127u) & ~127u;
+    const uint32_t AROW = 64, BROW = (uint32_t)a.cbx * 2;   // bytes of a pixel's channel block
+    const uint32_t AG = (uint32_t)(WG_KX * KY) * AROW, BG = (uint32_t)(HX * HY) * BROW;
+    const int NBX = N / a.cbx;
+    const uint32_t ABYTES = (uint32_t)a.ga * AG;
+    const uint32_t STAGE = wg_stage_bytes(a.M, a.ga, N, KY, h);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)S * STAGE);   // full[S], empty[S], acc
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * S + 1);
     volatile int *fail = reinterpret_cast<volatile int *>(tslot + 1);
@@ -437,16 +463,6 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     const int64_t kt1 = kt0 + a.per_chunk < a.ktiles ? kt0 + a.per_chunk : a.ktiles;
     const int nk = (int)(kt1 > kt0 ? kt1 - kt0 : 0);
 
-    // A rows past the copied groups: zero, written once through the generic proxy and made
-    // visible to the tensor core's (async proxy) reads
-    if (a.ga < MG) {
-        const uint32_t zbytes = (uint32_t)(MG - a.ga) * AG;
-        for (int s = 0; s < S; ++s) {
-            uint4 *z = reinterpret_cast<uint4 *>(smem + (size_t)s * STAGE + (size_t)a.ga * AG);
-            for (uint32_t i = tid; i < zbytes / 16; i += WG_THREADS) z[i] = make_uint4(0, 0, 0, 0);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full(s), 1);
@@ -482,16 +498,19 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
                 const int b = (int)(q / a.tiles_y);
                 const int x0 = tx * WG_KX, y0 = ty * KY;
                 const uint32_t st = sbase + (uint32_t)s * STAGE;
-                mbar_expect_tx(full(s), (uint32_t)a.ga * AG + (uint32_t)(N / 8) * BG);
-                tma_load_5d(st, &gmap, 0, x0, y0, b, 16 * mb, full(s));
-                tma_load_5d(st + ABYTES, &xmap, 0, x0 - h, y0 - h, b, nb * (N / 8), full(s));
+                mbar_expect_tx(full(s), ABYTES + (uint32_t)NBX * BG);
+                tma_load_5d(st, &gmap, 0, x0, y0, b, (a.M / 32) * mb, full(s));
+                tma_load_5d(st + ABYTES, &xmap, 0, x0 - h, y0 - h, b, nb * NBX, full(s));
             }
         }
     } else if (warp == 5) {
         // ---- MMA issuer: one MMA (K = 16) per tile row and tap ----
         const uint32_t idesc = instr_desc_mn(a.M, N);
         const bool one = elect_lane();
-        const uint64_t ad0 = smem_desc(0, 128u, AG), bd0 = smem_desc(0, 128u, BG);
+        const uint64_t ad0 = smem_desc_sw<32>(0, AG, 8 * AROW);
+        const uint64_t bd0 = a.cbx == 32 ? smem_desc_sw<32>(0, BG, 8 * BROW) : smem_desc_sw<16>(0, BG, 8 * BROW);
+        const uint32_t bunit = BROW / 16;   // a pixel in descriptor units
+        const uint64_t brow = (uint64_t)((uint32_t)HX * bunit);   // a row of the input tile
         bool ok = true;
         for (int i = 0; i < nk && !*fail; ++i) {
             const uint32_t s = (uint32_t)i % (uint32_t)S;
@@ -500,17 +519,27 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t st = sbase + s * STAGE;
             const uint64_t ad = ad0 + (st >> 4), bd = bd0 + ((st + ABYTES) >> 4);
-            if (one) {
-                for (int j = 0; j < ntap; ++j) {
-                    const int t = t0 + j, dy = h ? t / 3 - 1 : 0, dx = h ? t % 3 - 1 : 0;
-                    const uint64_t bt = bd + (uint64_t)((h + dy) * HX + h + dx);
-                    const uint32_t d = tmem + (uint32_t)(j * N);
-                    for (int k4 = 0; k4 < KY; k4 += 4)   // KY is 4 or 8
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            umma(d, ad + (uint64_t)((k4 + q) * 16), bt + (uint64_t)((k4 + q) * HX), idesc,
-                                 (i > 0 || k4 + q > 0) ? 1u : 0u);
+            // loops and descriptors outside the elected lane's branch: inside it they would not be
+            // computed in uniform registers (44 cycles per MMA against 27)
+            for (int j = 0; j < ntap; ++j) {
+                const int t = t0 + j, dy = h ? t / 3 - 1 : 0, dx = h ? t % 3 - 1 : 0;
+                uint64_t bt = bd + (uint64_t)((uint32_t)((h + dy) * HX + h + dx) * bunit), at = ad;
+                const uint32_t d = tmem + (uint32_t)(j * N);
+                for (int k4 = 0; k4 < KY; k4 += 4) {   // KY is 4 or 8
+                    const uint64_t b1 = bt + brow, b2 = b1 + brow, b3 = b2 + brow;
+                    const uint32_t first = i > 0 || k4 > 0 ? 1u : 0u;
+                    if (one) {
+                        umma(d, at, bt, idesc, first);
+                        umma(d, at + WG_KX * 4, b1, idesc, 1u);
+                        umma(d, at + 2 * WG_KX * 4, b2, idesc, 1u);
+                        umma(d, at + 3 * WG_KX * 4, b3, idesc, 1u);
+                    }
+                    __syncwarp();
+                    bt = b3 + brow;
+                    at += 4 * WG_KX * 4;
                 }
+            }
+            if (one) {
                 umma_commit(empty(s));   // the stage is free once these MMAs have read it
             }
             __syncwarp();
@@ -592,22 +621,29 @@ PFN_cuTensorMapEncodeTiled_v12000 tc_encoder() {
     return fn;
 }
 
-template <int N, int T>
+// The epilogue warps bound these kernels, so shared memory is budgeted for the four blocks of 192 threads
+// that an SM's registers hold.
+constexpr uint32_t SMEM_PER_BLOCK = 55 * 1024;
+
+// the weights of one output-channel block of N stay in shared memory
+bool tc_resident(const TcConvArgs &a, int N) { return a.nblocks == 1 && a.Cin * a.T * 2 * N <= 48 * 1024; }
+
+template <int N, int T, int CB>
 cudaError_t tc_launch(const CUtensorMap &map, TcConvArgs a, cudaStream_t st) {
+    using IN = InTile<T, CB>;
     static int configured_dev = -1;
     static int nsm = 0, occ_threads = 0;
-    const uint32_t wbytes = (uint32_t)T * 32 * N;
-    const int nkb = a.Cin / 16;
-    const uint32_t wall = (uint32_t)nkb * wbytes;
-    a.resident = (a.nblocks == 1 && wall <= 48u * 1024u) ? 1 : 0;
+    const uint32_t wbytes = (uint32_t)T * 2 * CB * N;
+    const uint32_t wall = (uint32_t)(a.Cin / CB) * wbytes;
+    a.resident = tc_resident(a, N) ? 1 : 0;
     size_t smem;
     if (a.resident) {
-        int S = (int)((96u * 1024u - wall) / HALO_BYTES);
+        int S = ((int)SMEM_PER_BLOCK - (int)wall) / (int)IN::PITCH;
         a.stages = S < 2 ? 2 : (S > 8 ? 8 : S);
-        smem = wall + (size_t)a.stages * HALO_BYTES;
+        smem = wall + (size_t)a.stages * IN::PITCH;
     } else {
-        const uint32_t stage = HALO_BYTES + wbytes;
-        int S = (int)((72u * 1024u) / stage);
+        const uint32_t stage = IN::PITCH + wbytes;
+        int S = (int)(SMEM_PER_BLOCK / stage);
         a.stages = S < 2 ? 2 : (S > 4 ? 4 : S);
         smem = (size_t)a.stages * stage;
     }
@@ -623,13 +659,13 @@ cudaError_t tc_launch(const CUtensorMap &map, TcConvArgs a, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_tc_conv<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        e = cudaFuncSetAttribute(k_tc_conv<N, T, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         // registers and threads per SM from the kernel's attributes
         cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, k_tc_conv<N, T>);
+        e = cudaFuncGetAttributes(&fa, k_tc_conv<N, T, CB>);
         if (e != cudaSuccess) return e;
         const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
         occ_threads = 65536 / (regs_warp * (TC_THREADS / 32));
@@ -642,22 +678,23 @@ cudaError_t tc_launch(const CUtensorMap &map, TcConvArgs a, cudaStream_t st) {
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int64_t grid = (int64_t)nsm * per_sm;
     if (grid > a.ntiles) grid = a.ntiles;
-    k_tc_conv<N, T><<<(unsigned)grid, TC_THREADS, smem, st>>>(map, a);
+    k_tc_conv<N, T, CB><<<(unsigned)grid, TC_THREADS, smem, st>>>(map, a);
     return cudaGetLastError();
 }
 
-bool encode_nhwc_groups(CUtensorMap &map, const __nv_bfloat16 *p, int B, int H, int W, int C, int bx, int by,
-                        int groups_box) {
+// [B][H][W][C] viewed as (channel in block, x, y, image, channel block) with blocks of cb = 32 or 16
+// channels, swizzled over a block's bytes; blocks_box of them per copy
+bool encode_nhwc_blocks(CUtensorMap &map, const __nv_bfloat16 *p, int B, int H, int W, int C, int cb, int bx, int by,
+                        int blocks_box) {
     auto enc = tc_encoder();
     if (!enc) return false;
-    // [B][H][W][C] viewed as (channel in group, x, y, image, 8-channel group)
-    cuuint64_t dims[5] = {8, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B, (cuuint64_t)(C / 8)};
-    cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2, 16};
-    cuuint32_t box[5] = {8, (cuuint32_t)bx, (cuuint32_t)by, 1, (cuuint32_t)groups_box};
+    cuuint64_t dims[5] = {(cuuint64_t)cb, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B, (cuuint64_t)(C / cb)};
+    cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2, (cuuint64_t)cb * 2};
+    cuuint32_t box[5] = {(cuuint32_t)cb, (cuuint32_t)bx, (cuuint32_t)by, 1, (cuuint32_t)blocks_box};
     cuuint32_t es[5] = {1, 1, 1, 1, 1};
     return enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void *)p, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+               CU_TENSOR_MAP_INTERLEAVE_NONE, cb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
@@ -665,7 +702,7 @@ bool encode_nhwc_groups(CUtensorMap &map, const __nv_bfloat16 *p, int B, int H, 
 int tc_block_n(int Cout) { return Cout < 128 ? Cout : 128; }
 
 cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
-    if (a.Cin % 16 || a.Cout % 8 || a.Cin < 16 || (a.T != 1 && a.T != 9) || a.B < 1 || a.H < 1 || a.W < 1)
+    if ((a.Cin != 16 && a.Cin % 32) || a.Cout % 32 || a.Cin < 16 || a.Cout < 32 || (a.T != 1 && a.T != 9) || a.B < 1 || a.H < 1 || a.W < 1)
         return cudaErrorInvalidValue;
     a.N = a.Cin <= 256 ? a.Cin : 256;
     if (a.Cin % a.N) return cudaErrorInvalidValue;
@@ -674,21 +711,22 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
     // M = 64 for at most 64 output channels: an MMA reads half as much of A (24 cycles against 40 at
     // N = 32; 222 -> 180 us for 32 x 32 x 9 over 2.1 M pixels)
     a.M = a.Cout <= 64 ? 64 : 128;
-    a.ga = a.Cout < a.M ? a.Cout / 8 : a.M / 8;
+    a.ga = (a.Cout < a.M ? a.Cout : a.M) / 32;
+    a.cbx = a.Cin % 32 == 0 ? 32 : 16;
     // taps per block: as many N-column accumulators as the 512 TMEM columns hold, in groups of
     // balanced size
-    const int maxt = 512 / a.N;
+    // (N <= 32: of half the columns, for two blocks per SM, whose issuing warps overlap: 174 -> 133 us
+    // for 32 x 32 x 9 over 2.1 M pixels, although each block loads every tile)
+    const int maxt = a.N <= 32 ? 256 / a.N : 512 / a.N;
     a.ngroups = (a.T + maxt - 1) / maxt;
     a.tpc = (a.T + a.ngroups - 1) / a.ngroups;
     const int h = a.T == 9 ? 1 : 0;
     // tile height: 8 pixel rows when three stages of it fit in shared memory, else 4
-    auto stage_bytes = [&](int ky) {
-        const uint32_t ab = (uint32_t)(a.M / 8) * WG_KX * ky * 16, bb = (uint32_t)(a.N / 8) * (WG_KX + 2 * h) * (ky + 2 * h) * 16;
-        return (ab + bb + 127u) & ~127u;
-    };
+    auto stage_bytes = [&](int ky) { return wg_stage_bytes(a.M, a.ga, a.N, ky, h); };
     a.ky = stage_bytes(8) * 3 <= 196u * 1024u ? 8 : 4;
     const uint32_t stage = stage_bytes(a.ky);
-    int S = (int)((196u * 1024u) / stage);
+    const bool two = a.tpc * a.N <= 256 && stage * 3 <= 100u * 1024u;   // room for two blocks per SM
+    int S = (int)((two ? 100u * 1024u : 196u * 1024u) / stage);
     a.stages = S > 6 ? 6 : S;
     if (a.stages < 2) return cudaErrorInvalidConfiguration;
     a.tiles_x = (a.W + WG_KX - 1) / WG_KX;
@@ -709,7 +747,7 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
     // block); every chunk's partial sums must fit the buffer
     const int64_t per_chunk_blocks = (int64_t)a.ngroups * a.nbm * a.nbn;
     const int64_t count = (int64_t)a.Cout * a.T * a.Cin;
-    const int resident = a.tpc * a.N <= 256 && stage * a.stages <= 100u * 1024u ? 2 : 1;
+    const int resident = two ? 2 : 1;
     // (rounded down: one block more than the SMs hold is a second round for all)
     int64_t chunks = (int64_t)resident * nsm / per_chunk_blocks;
     if (chunks < 1) chunks = 1;
@@ -720,8 +758,8 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
     a.chunks = (int)((a.ktiles + a.per_chunk - 1) / a.per_chunk);
     const size_t smem = (size_t)a.stages * stage + 8 * (2 * a.stages + 1) + 16;
     CUtensorMap gmap, xmap;
-    if (!encode_nhwc_groups(gmap, a.g, a.B, a.H, a.W, a.Cout, WG_KX, a.ky, a.ga) ||
-        !encode_nhwc_groups(xmap, a.in, a.B, a.H, a.W, a.Cin, WG_KX + 2 * h, a.ky + 2 * h, a.N / 8))
+    if (!encode_nhwc_blocks(gmap, a.g, a.B, a.H, a.W, a.Cout, 32, WG_KX, a.ky, a.ga) ||
+        !encode_nhwc_blocks(xmap, a.in, a.B, a.H, a.W, a.Cin, a.cbx, WG_KX + 2 * h, a.ky + 2 * h, a.N / a.cbx))
         return cudaErrorInvalidValue;
     const int64_t grid = (int64_t)a.chunks * per_chunk_blocks;
     k_tc_wgrad<<<(unsigned)grid, WG_THREADS, smem, st>>>(gmap, xmap, a);
@@ -746,23 +784,33 @@ cudaError_t tc_conv(const __nv_bfloat16 *in, TcConvArgs a, cudaStream_t st) {
     if (a.head_w && a.Cout != 32) return cudaErrorInvalidValue;
     auto enc = tc_encoder();
     if (!enc) return cudaErrorNotSupported;
-    // activation tensor [B][H][W][Cin] BF16, box of 8 channels x 10 x 18 pixels x 1 image
-    CUtensorMap map;
-    cuuint64_t dims[4] = {(cuuint64_t)a.Cin, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
-    cuuint64_t strides[3] = {(cuuint64_t)a.Cin * 2, (cuuint64_t)a.W * a.Cin * 2, (cuuint64_t)a.H * a.W * a.Cin * 2};
-    cuuint32_t box[4] = {8, HALO_X, HALO_Y, 1};
-    cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)in, dims, strides, box, es,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     a.nblocks = a.Cout / N;
     a.tiles_x = (a.W + TILE_X - 1) / TILE_X;
     a.tiles_y = (a.H + TILE_Y - 1) / TILE_Y;
     a.ntiles = (int64_t)a.B * a.tiles_y * a.tiles_x * a.nblocks;
-    if (N == 32) return a.T == 9 ? tc_launch<32, 9>(map, a, st) : tc_launch<32, 1>(map, a, st);
-    if (N == 64) return a.T == 9 ? tc_launch<64, 9>(map, a, st) : tc_launch<64, 1>(map, a, st);
-    return a.T == 9 ? tc_launch<128, 9>(map, a, st) : tc_launch<128, 1>(map, a, st);
+    if (a.ntiles > INT32_MAX) return cudaErrorInvalidValue;
+    // 32 channels per stage where the weights are resident or small; else 16, so that a stage with its
+    // weight slab stays small enough for two or three blocks per SM
+    const int cb = a.Cin % 32 == 0 && (tc_resident(a, N) || a.T == 1) ? 32 : 16;
+    // activation tensor [B][H][W][Cin] BF16, box of cb channels x the staged pixels of 1 image
+    CUtensorMap map;
+    const int halo = a.T == 9 ? 2 : 0;
+    cuuint64_t dims[4] = {(cuuint64_t)a.Cin, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
+    cuuint64_t strides[3] = {(cuuint64_t)a.Cin * 2, (cuuint64_t)a.W * a.Cin * 2, (cuuint64_t)a.H * a.W * a.Cin * 2};
+    cuuint32_t box[4] = {(cuuint32_t)cb, (cuuint32_t)(TILE_X + halo), (cuuint32_t)(TILE_Y + halo), 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)in, dims, strides, box, es,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, cb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+#define GABP_CONV(NN) \
+    if (N == NN && a.T == 9) return cb == 32 ? tc_launch<NN, 9, 32>(map, a, st) : tc_launch<NN, 9, 16>(map, a, st); \
+    if (N == NN) return cb == 32 ? tc_launch<NN, 1, 32>(map, a, st) : tc_launch<NN, 1, 16>(map, a, st);
+    GABP_CONV(32)
+    GABP_CONV(64)
+    GABP_CONV(128)
+#undef GABP_CONV
+    return cudaErrorInvalidValue;
 }
 
 
