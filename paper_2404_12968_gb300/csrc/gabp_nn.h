@@ -54,15 +54,24 @@ struct TcConvArgs {
     int64_t ntiles;
 };
 int tc_block_n(int Cout);
-// packed[nb][kb][t][h][n][e] = w[nb * N + n][t][16 kb + 8 h + e], N = tc_block_n(Cout)
-cudaError_t tc_pack_weights(const __nv_bfloat16 *w, int Cout, int T, int Cin, __nv_bfloat16 *out, cudaStream_t st);
+// The layers whose weights tc_pack_weights packs (in one launch: one per layer and direction, with the
+// flipped copies, were 40 of about 3 us each): off[l] = a layer's offset in w and out.
+// Forward: packed[nb][kb][t][h][n][e] = w[nb * N + n][t][16 kb + 8 h + e], N = tc_block_n(Cout); flip: the
+// same of the weights of the input gradient's convolution (flipped in space, Cin and Cout exchanged).
+struct TcPackLayers {
+    int n;
+    int64_t off[16];
+    int cout[16], taps[16], cin[16];
+    int block0[16];   // set by tc_pack_weights
+};
+cudaError_t tc_pack_weights(const __nv_bfloat16 *w, TcPackLayers layers, bool flip, __nv_bfloat16 *out, cudaStream_t st);
 cudaError_t tc_conv(const __nv_bfloat16 *in, TcConvArgs a, cudaStream_t st);
 int64_t wgrad_chunks(const WgradArgs &a);
 cudaError_t conv_wgrad(WgradArgs a, float *dw, cudaStream_t st);
 // Weight gradient on the tcgen05 tensor cores (gabp_nn_tc.cu): dw[co][t][ci] = sum over the
 // pixels p of g[p][co] in[p + d_t][ci] (zero outside the image), as partial sums over pixel
-// chunks in part (at most part_cap floats) reduced into dw in chunk order.  Cin 16 or a multiple
-// of 32 (at most 256 per block of N), Cout a multiple of 32 (blocks of 64 or 128).
+// chunks in part (at most part_cap floats) reduced into dw in chunk order; db[co] = sum of g[p][co].
+// Cin 16 or a multiple of 32 (at most 256 per block of N), Cout a multiple of 32 (blocks of 64 or 128).
 struct TcWgradArgs {
     const __nv_bfloat16 *g;     // [B][H][W][Cout]
     const __nv_bfloat16 *in;    // [B][H][W][Cin]
@@ -74,9 +83,9 @@ struct TcWgradArgs {
     int M, N, nbn, nbm, chunks, stages, ky, ga, cbx, tpc, ngroups;
     int64_t ktiles, tiles_x, tiles_y, per_chunk;
 };
-cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st);
-// out[i] = sum over c < chunks of part[c * count + i], in chunk order
-cudaError_t reduce_chunks(const float *part, int chunks, int64_t count, float *out, cudaStream_t st);
+cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st);
+// dw[i] and db[c]: sums in chunk order of count weight partials per chunk, then cout bias partials
+cudaError_t reduce_wgrad(const float *part, int chunks, int64_t count, int cout, float *dw, float *db, cudaStream_t st);
 // db[c] = sum over the P pixels of g[p][c]: chunk partials in part (at most part_cap floats),
 // reduced in chunk order; C at most 256
 cudaError_t bias_grad(const __nv_bfloat16 *g, int64_t P, int C, float *db, float *part, int64_t part_cap,

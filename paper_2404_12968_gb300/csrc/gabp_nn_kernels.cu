@@ -306,6 +306,20 @@ __device__ __forceinline__ void store8(__nv_bfloat16 *p, const float (&v)[8]) {
     *reinterpret_cast<uint4 *>(p) = q;
 }
 
+// the weight and the bias gradient of a layer: sums of the chunk partials in chunk order (count
+// weight sums per chunk, then cout bias sums per chunk)
+__global__ void k_reduce_wgrad(const float *part, int chunks, int64_t count, int cout, float *dw, float *db) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= count + cout) return;
+    const bool w = i < count;
+    const float *p = w ? part + i : part + (int64_t)chunks * count + (i - count);
+    const int64_t step = w ? count : cout;
+    float s = 0.f;
+    for (int c = 0; c < chunks; ++c) s += p[c * step];
+    if (w) dw[i] = s;
+    else db[i - count] = s;
+}
+
 // bias gradient, first stage: part[b][c] = sum of g[p][c] over the pixels of chunk b.  A thread
 // takes 8 channels (one 16-byte load) of every R-th pixel, R = 2048 / C; the block adds its R row
 // sums per channel in a fixed order.  C a multiple of 8.
@@ -571,8 +585,8 @@ cudaError_t conv_wgrad(WgradArgs a, float *dw, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t reduce_chunks(const float *part, int chunks, int64_t count, float *out, cudaStream_t st) {
-    k_reduce_chunks<<<nb(count), 256, 0, st>>>(part, chunks, count, out);
+cudaError_t reduce_wgrad(const float *part, int chunks, int64_t count, int cout, float *dw, float *db, cudaStream_t st) {
+    k_reduce_wgrad<<<nb(count + cout), 256, 0, st>>>(part, chunks, count, cout, dw, db);
     return cudaGetLastError();
 }
 

@@ -462,11 +462,12 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     const int64_t kt0 = (int64_t)chunk * a.per_chunk;
     const int64_t kt1 = kt0 + a.per_chunk < a.ktiles ? kt0 + a.per_chunk : a.ktiles;
     const int nk = (int)(kt1 > kt0 ? kt1 - kt0 : 0);
+    const bool bias = tg == 0 && nb == 0;   // this block also sums g over its pixels
 
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full(s), 1);
-            mbar_init(empty(s), 1);
+            mbar_init(empty(s), bias ? 5 : 1);   // the MMAs, and the four warps that sum the bias gradient
         }
         mbar_init(accb, 1);
         *fail = 0;
@@ -549,6 +550,33 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     } else {
         // ---- epilogue: warps 0-3.  M = 128: TMEM lane 32 w + lane = output channel 128 mb + 32 w +
         // lane; M = 64: the accumulator's rows 16 w .. 16 w + 15 are the first 16 lanes of warp w ----
+        // The bias gradient first, from the staged g while the MMAs run: thread = 8 channels (16 bytes
+        // of a pixel's row) of every R-th pixel.  (A kernel of its own read g once more: 290 us of a
+        // training step of 8 512^2 grids, which took 3.13 ms; with this and one packing launch 2.74.)
+        const int C8 = 4 * a.ga, R = 128 / C8, ch = tid % C8, pr = tid / C8;   // 4, 8 or 16 groups of channels
+        float bs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (bias)
+            for (int i = 0; i < nk; ++i) {
+                const int s = i % S;
+                const bool got = mbar_wait(full(s), (uint32_t)(i / S) & 1);
+                if (__any_sync(0xffffffffu, !got)) {
+                    *fail = 1;
+                    break;
+                }
+                const unsigned char *A = smem + (size_t)s * STAGE + (size_t)(ch >> 2) * AG;
+                for (int q = pr; q < WG_KX * KY; q += R) {
+                    // the 64-byte swizzle: address bits 4, 5 exclusive-or bits 7, 8
+                    const uint4 v = *reinterpret_cast<const uint4 *>(A + q * 64 + (((ch & 3) ^ ((q >> 1) & 3)) << 4));
+                    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        bs[2 * e] += bf_lo(w4[e]);
+                        bs[2 * e + 1] += bf_hi(w4[e]);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty(s));
+            }
         const bool ok = mbar_wait(accb, 0);
         if (!ok) *fail = 1;
         // warp-uniform decision: tcgen05.ld is a whole-warp instruction
@@ -578,6 +606,19 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
                 for (int c = 0; c < N; ++c) dst[c] = 0.f;
             }
         }
+        if (bias) {   // the R pixel groups' sums in order; every MMA has read the stages
+            float *sc = reinterpret_cast<float *>(smem);
+            asm volatile("bar.sync 1, 128;" ::: "memory");   // and every warp of the sums
+#pragma unroll
+            for (int e = 0; e < 8; ++e) sc[pr * 32 * a.ga + 8 * ch + e] = bs[e];
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            const int c0 = a.M * mb + tid;
+            if (tid < 32 * a.ga && c0 < a.Cout) {
+                float t = 0.f;
+                for (int q = 0; q < R; ++q) t += sc[q * 32 * a.ga + tid];
+                a.part[(int64_t)a.chunks * a.Cout * a.T * a.Cin + (int64_t)chunk * a.Cout + c0] = t;
+            }
+        }
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -589,23 +630,26 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     }
 }
 
-// packed[nb][kb][t][h][n][e] = w[nb * N + n][t][16 kb + 8 h + e]
-__global__ void k_tc_pack(const __nv_bfloat16 *w, int Cout, int T, int Cin, int N, __nv_bfloat16 *out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t total = (int64_t)Cout * T * Cin;
-    if (i >= total) return;
-    const int e = (int)(i & 7);
-    int64_t r = i >> 3;
-    const int n = (int)(r % N);
+// Packed weights of every layer in one launch, layer l at the same offset as in w.  Forward:
+// packed[nb][kb][t][h][n][e] = w[nb * N + n][t][16 kb + 8 h + e].  FLIP, the convolution of the input
+// gradient: the same of the weights flipped in space with Cin and Cout exchanged.
+template <bool FLIP> __global__ void k_tc_pack(const __nv_bfloat16 *w, TcPackLayers p, __nv_bfloat16 *out) {
+    int l = 0;
+    while (l + 1 < p.n && (int)blockIdx.x >= p.block0[l + 1]) ++l;
+    const int T = p.taps[l], Cin = p.cin[l], Cout = p.cout[l];
+    const int i = ((int)blockIdx.x - p.block0[l]) * 256 + (int)threadIdx.x;
+    if (i >= Cout * T * Cin) return;
+    const int K = FLIP ? Cout : Cin, R = FLIP ? Cin : Cout, N = R < 128 ? R : 128;   // contraction, rows, rows per block
+    int r = i >> 3;
+    const int n = r % N;
     r /= N;
-    const int h = (int)(r & 1);
+    const int h = r & 1;
     r >>= 1;
-    const int t = (int)(r % T);
+    const int t = r % T;
     r /= T;
-    const int nkb = Cin / 16;
-    const int kb = (int)(r % nkb);
-    const int nb = (int)(r / nkb);
-    out[i] = w[((int64_t)(nb * N + n) * T + t) * Cin + 16 * kb + 8 * h + e];
+    const int kb = r % (K / 16), nb = r / (K / 16);
+    const int row = nb * N + n, k = 16 * kb + 8 * h + (i & 7);
+    out[p.off[l] + i] = w[p.off[l] + (FLIP ? ((int64_t)k * T + (T - 1 - t)) * Cin + row : ((int64_t)row * T + t) * Cin + k)];
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tc_encoder() {
@@ -701,7 +745,7 @@ bool encode_nhwc_blocks(CUtensorMap &map, const __nv_bfloat16 *p, int B, int H, 
 
 int tc_block_n(int Cout) { return Cout < 128 ? Cout : 128; }
 
-cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
+cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st) {
     if ((a.Cin != 16 && a.Cin % 32) || a.Cout % 32 || a.Cin < 16 || a.Cout < 32 || (a.T != 1 && a.T != 9) || a.B < 1 || a.H < 1 || a.W < 1)
         return cudaErrorInvalidValue;
     a.N = a.Cin <= 256 ? a.Cin : 256;
@@ -752,7 +796,7 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
     int64_t chunks = (int64_t)resident * nsm / per_chunk_blocks;
     if (chunks < 1) chunks = 1;
     if (chunks > a.ktiles) chunks = a.ktiles;
-    if (chunks * count > a.part_cap) chunks = a.part_cap / count;
+    if (chunks * (count + a.Cout) > a.part_cap) chunks = a.part_cap / (count + a.Cout);
     if (chunks < 1) return cudaErrorInvalidValue;
     a.per_chunk = (a.ktiles + chunks - 1) / chunks;
     a.chunks = (int)((a.ktiles + a.per_chunk - 1) / a.per_chunk);
@@ -765,12 +809,17 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, cudaStream_t st) {
     k_tc_wgrad<<<(unsigned)grid, WG_THREADS, smem, st>>>(gmap, xmap, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return reduce_chunks(a.part, a.chunks, count, dw, st);
+    return reduce_wgrad(a.part, a.chunks, count, a.Cout, dw, db, st);
 }
 
-cudaError_t tc_pack_weights(const __nv_bfloat16 *w, int Cout, int T, int Cin, __nv_bfloat16 *out, cudaStream_t st) {
-    const int64_t total = (int64_t)Cout * T * Cin;
-    k_tc_pack<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(w, Cout, T, Cin, tc_block_n(Cout), out);
+cudaError_t tc_pack_weights(const __nv_bfloat16 *w, TcPackLayers p, bool flip, __nv_bfloat16 *out, cudaStream_t st) {
+    int blocks = 0;
+    for (int l = 0; l < p.n; ++l) {
+        p.block0[l] = blocks;
+        blocks += (p.cout[l] * p.taps[l] * p.cin[l] + 255) / 256;
+    }
+    if (flip) k_tc_pack<true><<<blocks, 256, 0, st>>>(w, p, out);
+    else k_tc_pack<false><<<blocks, 256, 0, st>>>(w, p, out);
     return cudaGetLastError();
 }
 

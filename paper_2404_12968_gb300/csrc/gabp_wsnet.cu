@@ -54,9 +54,9 @@ struct gabp_wsnet {
     __nv_bfloat16 *w16 = nullptr;    // BF16 copy (the flat vector, converted)
     __nv_bfloat16 *wt = nullptr;     // flipped/transposed weights scratch (largest layer)
     __nv_bfloat16 *wpk = nullptr;    // weights packed for the tensor-core forward (same offsets)
-    __nv_bfloat16 *wtpk = nullptr;   // flipped/transposed weights packed for the tensor-core backward (largest layer)
+    __nv_bfloat16 *wtpk = nullptr;   // flipped/transposed weights packed for the tensor-core backward (same offsets)
     float *zbias = nullptr;          // 256 zeros: the backward-data convolution has no bias
-    bool packed = false;             // wpk matches w16
+    bool packed = false, packed_bwd = false;   // wpk, wtpk match w16
     int *derr = nullptr;             // device flag of the tensor-core kernels (a bounded wait ran out)
     int kernels = GABP_WSNET_TCGEN05;
     const __nv_bfloat16 *xin = nullptr;   // caller's input, read in place by the tensor-core forward
@@ -192,6 +192,18 @@ int conv_fwd(gabp_wsnet *net, int l, const Buf &in, const Buf *skip, Buf &out, i
     return GABP_OK;
 }
 
+// layers l0 .. NLAYER - 1 for the weight packing
+gabp::nn::TcPackLayers pack_layers(const gabp_wsnet *net, int l0) {
+    gabp::nn::TcPackLayers p{};
+    for (int l = l0; l < NLAYER; ++l, ++p.n) {
+        p.off[p.n] = net->woff[l];
+        p.cout[p.n] = SPECS[l].cout;
+        p.taps[p.n] = SPECS[l].taps;
+        p.cin[p.n] = SPECS[l].cin;
+    }
+    return p;
+}
+
 // Forward on the tcgen05 tensor-core convolutions, with the pooling, the upsampling additions
 // and the head fused into the convolutions' epilogues.  Buffers that only the backward pass
 // reads (r2, r1, r0, d0) are written when gradients are wanted.
@@ -199,10 +211,7 @@ int forward_tc(gabp_wsnet *net) {
     const int B = net->B, H = net->H, W = net->W;
     cudaStream_t st = net->stream;
     if (!net->packed) {
-        for (int l = 0; l < NLAYER; ++l)
-            WK(gabp::nn::tc_pack_weights(net->w16 + net->woff[l], SPECS[l].cout, SPECS[l].taps, SPECS[l].cin,
-                                         net->wpk + net->woff[l], st),
-               "pack weights");
+        WK(gabp::nn::tc_pack_weights(net->w16, pack_layers(net, 0), false, net->wpk, st), "pack weights");
         net->packed = true;
     }
     const bool keep = net->grads;
@@ -323,19 +332,16 @@ int conv_bwd(gabp_wsnet *net, int l, const Buf &g, const Buf &in, Buf *din, int 
         ta.Cin = s.cin;
         ta.Cout = s.cout;
         ta.T = s.taps;
-        WK(gabp::nn::tc_wgrad(ta, net->g + net->woff[l], st), "tensor-core weight gradient");
+        WK(gabp::nn::tc_wgrad(ta, net->g + net->woff[l], net->g + net->boff[l], st), "tensor-core weight gradient");
     } else {
         WK(gabp::nn::conv_wgrad(wa, net->g + net->woff[l], st), "conv wgrad");
+        WK(gabp::nn::bias_grad(g.p, (int64_t)B * h * w, s.cout, net->g + net->boff[l], net->part, net->part_n, st), "bias grad");
     }
-    WK(gabp::nn::bias_grad(g.p, (int64_t)B * h * w, s.cout, net->g + net->boff[l], net->part, net->part_n, st),
-       "bias grad");
     if (din && net->kernels == GABP_WSNET_TCGEN05) {
         // gradient w.r.t. the input: the forward convolution of g with the flipped, transposed
         // weights (Cin and Cout exchanged), on the tcgen05 tensor cores like the forward pass
-        WK(gabp::nn::flip_transpose(net->w16 + net->woff[l], s.cout, s.taps, s.cin, net->wt, st), "flip");
-        WK(gabp::nn::tc_pack_weights(net->wt, s.cin, s.taps, s.cout, net->wtpk, st), "pack flipped weights");
         gabp::nn::TcConvArgs a{};
-        a.wpk = net->wtpk;
+        a.wpk = net->wtpk + net->woff[l];
         a.bias = net->zbias;
         a.out = din->p;
         a.mask = relu ? relu->p : nullptr;
@@ -375,6 +381,10 @@ int backward(gabp_wsnet *net) {
     cudaStream_t st = net->stream;
     int rc;
     Buf &ga = net->ga, &gb = net->gb;
+    if (net->kernels == GABP_WSNET_TCGEN05 && !net->packed_bwd) {   // (layer 0 has no input gradient)
+        WK(gabp::nn::tc_pack_weights(net->w16, pack_layers(net, 1), true, net->wtpk, st), "pack flipped weights");
+        net->packed_bwd = true;
+    }
     // head and the ReLU before it
     WK(gabp::nn::head_relu_bwd(net->dout, net->d0.p, P0, net->w + net->head_off, gb.p, net->part, net->part_n,
                                net->g + net->head_off, st),
@@ -508,7 +518,7 @@ int gabp_wsnet_create(gabp_wsnet **out, uint64_t seed, int device) {
     if (e == cudaSuccess) e = cudaMalloc((void **)&net->w16, sizeof(__nv_bfloat16) * off);
     if (e == cudaSuccess) e = cudaMalloc((void **)&net->wt, sizeof(__nv_bfloat16) * maxw);
     if (e == cudaSuccess) e = cudaMalloc((void **)&net->wpk, sizeof(__nv_bfloat16) * off);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&net->wtpk, sizeof(__nv_bfloat16) * maxw);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&net->wtpk, sizeof(__nv_bfloat16) * off);
     if (e == cudaSuccess) e = cudaMalloc((void **)&net->zbias, sizeof(float) * 256);
     if (e == cudaSuccess) e = cudaMemset(net->zbias, 0, sizeof(float) * 256);
     if (e == cudaSuccess) e = cudaMalloc((void **)&net->derr, sizeof(int));
@@ -540,7 +550,7 @@ int gabp_wsnet_set_params(gabp_wsnet *net, const float *params) {
     if (!net || !params) return GABP_ERR_ARG;
     WK(cudaMemcpy(net->w, params, sizeof(float) * net->nparam, cudaMemcpyDefault), "copy params");
     WK(gabp::nn::to_bf16(net->w, net->w16, net->nparam, net->stream), "to bf16");
-    net->packed = false;
+    net->packed = net->packed_bwd = false;
     WK(cudaStreamSynchronize(net->stream), "sync");
     return GABP_OK;
 }
@@ -613,7 +623,7 @@ int gabp_wsnet_train_step(gabp_wsnet *net, const void *const *xs, const float *c
     WK(gabp::nn::adam(net->w, net->m, net->v, net->g, net->nparam, lr, 0.9f, 0.999f, 1e-8f, net->step, net->w16,
                       net->stream),
        "adam");
-    net->packed = false;
+    net->packed = net->packed_bwd = false;
     WK(cudaStreamSynchronize(net->stream), "sync");
     return GABP_OK;
 }
