@@ -70,7 +70,7 @@ int64_t wgrad_chunks(const WgradArgs &a);
 cudaError_t conv_wgrad(WgradArgs a, float *dw, cudaStream_t st);
 // Weight gradient on the tcgen05 tensor cores (gabp_nn_tc.cu): dw[co][t][ci] = sum over the
 // pixels p of g[p][co] in[p + d_t][ci] (zero outside the image), as partial sums over pixel
-// chunks in part (at most part_cap floats) reduced into dw in chunk order; db[co] = sum of g[p][co].
+// chunks in part (at most part_cap floats) reduced into dw in a fixed order; db[co] = sum of g[p][co].
 // Cin 16 or a multiple of 32 (at most 256 per block of N), Cout a multiple of 32 (blocks of 64 or 128).
 struct TcWgradArgs {
     const __nv_bfloat16 *g;     // [B][H][W][Cout]
@@ -80,11 +80,12 @@ struct TcWgradArgs {
     int *err;                   // device flag, set if a bounded wait ran out
     int B, H, W, Cin, Cout, T;
     // set by tc_wgrad
-    int M, N, nbn, nbm, chunks, stages, ky, ga, cbx, tpc, ngroups;
+    int M, N, nbn, nbm, chunks, stages, ky, ga, cbx, tpc, ngroups, stage, xbytes;
     int64_t ktiles, tiles_x, tiles_y, per_chunk;
 };
 cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st);
-// dw[i] and db[c]: sums in chunk order of count weight partials per chunk, then cout bias partials
+// dw[i] and db[c]: sums over the chunks, in a fixed order, of count weight partials per chunk, then
+// cout bias partials per chunk
 cudaError_t reduce_wgrad(const float *part, int chunks, int64_t count, int cout, float *dw, float *db, cudaStream_t st);
 // db[c] = sum over the P pixels of g[p][c]: chunk partials in part (at most part_cap floats),
 // reduced in chunk order; C at most 256

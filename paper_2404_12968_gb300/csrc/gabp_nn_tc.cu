@@ -414,6 +414,10 @@ __host__ __device__ inline uint32_t wg_stage_bytes(int M, int ga, int N, int ky,
     const uint32_t reach = (uint32_t)(M / 32) * ag;
     return ((both > reach ? both : reach) + 1023u) & ~1023u;
 }
+// the same with taps stacked: the input (and a pixel past it, which the fourth tap reaches), then g
+__host__ __device__ inline uint32_t wg_stacked_x_bytes(int cin, int ky) {
+    return ((uint32_t)((WG_KX + 2) * (ky + 2) + 1) * (uint32_t)cin * 2 + 1023u) & ~1023u;
+}
 
 // Block: a group of taps [t0, t0 + tpc), output-channel block mb (of M), input-channel block nb (N),
 // pixel-tile chunk.  A tile is 16 x KY pixels.  Shared memory per stage, in blocks of 32 channels (the
@@ -428,6 +432,15 @@ __host__ __device__ inline uint32_t wg_stage_bytes(int M, int ga, int N, int ky,
 // those accumulator rows are not read.  (As [8-channel group][pixel] tiles without a swizzle the copies
 // had 16-byte rows, of which the TMA unit moves one per 2.4 cycles: 75 -> 42 us for 128 x 128 x 9 over
 // 131 k pixels, 101 -> 54 us for 256 x 256 x 9 over 33 k.)
+//
+// STACK (3x3 taps of 16 or 32 input channels, at most 64 output channels): the operands exchange roles,
+// and A is the input with the taps of a row as its channel blocks, one pixel apart: M = 4 blocks
+// (dx = -1, 0, 1 and one that is not read) x Cin, N = Cout.  An MMA is bound by reading its operands
+// from shared memory (M = 64, N = 32: 24 cycles; this one: 64) and does the work of three; all nine
+// taps take 3 Cout TMEM columns, so no tile is loaded twice.  32 x 32 x 9 over 2.1 M pixels: 88 us (51 of
+// them by the operand reads alone; memory: 40), and a training step's four layers of this kind 432 ->
+// 259 us.  (Keeping g as A, M = 64, and three taps in N = 96: 313.)
+template <bool STACK>
 __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__ CUtensorMap gmap,
                                                          const __grid_constant__ CUtensorMap xmap, TcWgradArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -435,9 +448,10 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     const int HX = WG_KX + 2 * h, HY = KY + 2 * h;
     const uint32_t AROW = 64, BROW = (uint32_t)a.cbx * 2;   // bytes of a pixel's channel block
     const uint32_t AG = (uint32_t)(WG_KX * KY) * AROW, BG = (uint32_t)(HX * HY) * BROW;
-    const int NBX = N / a.cbx;
+    const int NBX = STACK ? 1 : N / a.cbx;
     const uint32_t ABYTES = (uint32_t)a.ga * AG;
-    const uint32_t STAGE = wg_stage_bytes(a.M, a.ga, N, KY, h);
+    const uint32_t GOFF = STACK ? (uint32_t)a.xbytes : 0, XOFF = STACK ? 0 : ABYTES;   // g and the input in a stage
+    const uint32_t STAGE = (uint32_t)a.stage;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)S * STAGE);   // full[S], empty[S], acc
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * S + 1);
     volatile int *fail = reinterpret_cast<volatile int *>(tslot + 1);
@@ -446,7 +460,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
     auto full = [&](int s) { return saddr(&bars[s]); };
     auto empty = [&](int s) { return saddr(&bars[S + s]); };
     const uint32_t accb = saddr(&bars[2 * S]);
-    const uint32_t need = (uint32_t)(a.tpc * N);
+    const uint32_t need = (uint32_t)((STACK ? 3 : a.tpc) * N);
     const uint32_t tcols = need <= 32 ? 32u : (need <= 64 ? 64u : (need <= 128 ? 128u : (need <= 256 ? 256u : 512u)));
 
     // block -> (chunk, tap group, mb, nb)
@@ -500,16 +514,17 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
                 const int x0 = tx * WG_KX, y0 = ty * KY;
                 const uint32_t st = sbase + (uint32_t)s * STAGE;
                 mbar_expect_tx(full(s), ABYTES + (uint32_t)NBX * BG);
-                tma_load_5d(st, &gmap, 0, x0, y0, b, (a.M / 32) * mb, full(s));
-                tma_load_5d(st + ABYTES, &xmap, 0, x0 - h, y0 - h, b, nb * NBX, full(s));
+                tma_load_5d(st + GOFF, &gmap, 0, x0, y0, b, (a.M / 32) * mb, full(s));
+                tma_load_5d(st + XOFF, &xmap, 0, x0 - h, y0 - h, b, nb * NBX, full(s));
             }
         }
     } else if (warp == 5) {
         // ---- MMA issuer: one MMA (K = 16) per tile row and tap ----
         const uint32_t idesc = instr_desc_mn(a.M, N);
         const bool one = elect_lane();
+        const uint32_t xg = STACK ? BROW : BG;   // between the input's blocks: one pixel, one channel block
         const uint64_t ad0 = smem_desc_sw<32>(0, AG, 8 * AROW);
-        const uint64_t bd0 = a.cbx == 32 ? smem_desc_sw<32>(0, BG, 8 * BROW) : smem_desc_sw<16>(0, BG, 8 * BROW);
+        const uint64_t bd0 = a.cbx == 32 ? smem_desc_sw<32>(0, xg, 8 * BROW) : smem_desc_sw<16>(0, xg, 8 * BROW);
         const uint32_t bunit = BROW / 16;   // a pixel in descriptor units
         const uint64_t brow = (uint64_t)((uint32_t)HX * bunit);   // a row of the input tile
         bool ok = true;
@@ -519,10 +534,10 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
             if (__any_sync(0xffffffffu, !ok)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t st = sbase + s * STAGE;
-            const uint64_t ad = ad0 + (st >> 4), bd = bd0 + ((st + ABYTES) >> 4);
+            const uint64_t ad = ad0 + ((st + GOFF) >> 4), bd = bd0 + ((st + XOFF) >> 4);
             // loops and descriptors outside the elected lane's branch: inside it they would not be
             // computed in uniform registers (44 cycles per MMA against 27)
-            for (int j = 0; j < ntap; ++j) {
+            for (int j = 0; !STACK && j < ntap; ++j) {
                 const int t = t0 + j, dy = h ? t / 3 - 1 : 0, dx = h ? t % 3 - 1 : 0;
                 uint64_t bt = bd + (uint64_t)((uint32_t)((h + dy) * HX + h + dx) * bunit), at = ad;
                 const uint32_t d = tmem + (uint32_t)(j * N);
@@ -540,6 +555,18 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
                     at += 4 * WG_KX * 4;
                 }
             }
+            // (consecutive MMAs into different accumulators)
+            if (STACK)
+                for (int k = 0; k < KY; ++k) {
+                    const uint64_t x0 = bd + (uint64_t)k * brow, x1 = x0 + brow, x2 = x1 + brow, g = ad + (uint64_t)(k * WG_KX * 4);
+                    const uint32_t acc = i > 0 || k > 0 ? 1u : 0u;
+                    if (one) {
+                        umma(tmem, x0, g, idesc, acc);
+                        umma(tmem + (uint32_t)N, x1, g, idesc, acc);
+                        umma(tmem + (uint32_t)(2 * N), x2, g, idesc, acc);
+                    }
+                    __syncwarp();
+                }
             if (one) {
                 umma_commit(empty(s));   // the stage is free once these MMAs have read it
             }
@@ -563,7 +590,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
                     *fail = 1;
                     break;
                 }
-                const unsigned char *A = smem + (size_t)s * STAGE + (size_t)(ch >> 2) * AG;
+                const unsigned char *A = smem + (size_t)s * STAGE + GOFF + (size_t)(ch >> 2) * AG;
                 for (int q = pr; q < WG_KX * KY; q += R) {
                     // the 64-byte swizzle: address bits 4, 5 exclusive-or bits 7, 8
                     const uint4 v = *reinterpret_cast<const uint4 *>(A + q * 64 + (((ch & 3) ^ ((q >> 1) & 3)) << 4));
@@ -581,8 +608,25 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
         if (!ok) *fail = 1;
         // warp-uniform decision: tcgen05.ld is a whole-warp instruction
         const bool go = __all_sync(0xffffffffu, ok && !*fail);
+        if (STACK && go) {
+            // accumulator row = (tap of the row: this warp, input channel), column = output channel
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const bool mine = warp < 3 && lane < a.Cin;
+#pragma unroll 1
+            for (int j = 0; j < 3; ++j)
+#pragma unroll 1
+                for (int c = 0; c < N; c += 16) {
+                    uint32_t v[16] = {};
+                    if (nk > 0) tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(j * N + c), v);
+                    float *dst = a.part + (((int64_t)chunk * a.Cout + c) * 9 + 3 * j + warp) * a.Cin + lane;
+                    if (mine) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) dst[(int64_t)e * 9 * a.Cin] = __uint_as_float(v[e]);
+                    }
+                }
+        }
         const int co = a.M == 128 ? 128 * mb + 32 * warp + lane : (lane < 16 ? 16 * warp + lane : a.Cout);
-        if (go && nk > 0) {
+        if (!STACK && go && nk > 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
             for (int j = 0; j < ntap; ++j) {
@@ -600,7 +644,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
                     }
                 }
             }
-        } else if (go && co < a.Cout) {   // an empty chunk: zero partial sums
+        } else if (!STACK && go && co < a.Cout) {   // an empty chunk: zero partial sums
             for (int j = 0; j < ntap; ++j) {
                 float *dst = a.part + (((int64_t)chunk * a.Cout + co) * a.T + t0 + j) * a.Cin + nb * N;
                 for (int c = 0; c < N; ++c) dst[c] = 0.f;
@@ -612,7 +656,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_tc_wgrad(const __grid_constant__
 #pragma unroll
             for (int e = 0; e < 8; ++e) sc[pr * 32 * a.ga + 8 * ch + e] = bs[e];
             asm volatile("bar.sync 1, 128;" ::: "memory");
-            const int c0 = a.M * mb + tid;
+            const int c0 = STACK ? tid : a.M * mb + tid;
             if (tid < 32 * a.ga && c0 < a.Cout) {
                 float t = 0.f;
                 for (int q = 0; q < R; ++q) t += sc[q * 32 * a.ga + tid];
@@ -748,28 +792,34 @@ int tc_block_n(int Cout) { return Cout < 128 ? Cout : 128; }
 cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st) {
     if ((a.Cin != 16 && a.Cin % 32) || a.Cout % 32 || a.Cin < 16 || a.Cout < 32 || (a.T != 1 && a.T != 9) || a.B < 1 || a.H < 1 || a.W < 1)
         return cudaErrorInvalidValue;
-    a.N = a.Cin <= 256 ? a.Cin : 256;
-    if (a.Cin % a.N) return cudaErrorInvalidValue;
-    a.nbn = a.Cin / a.N;
-    a.nbm = (a.Cout + 127) / 128;
+    // the narrow layers (64 x 64 would fill M = 128 with two taps, no fewer operand bytes per tap)
+    const bool stack = a.T == 9 && a.Cin <= 32 && a.Cout <= 64;
+    a.N = stack ? a.Cout : (a.Cin <= 256 ? a.Cin : 256);
+    if (!stack && a.Cin % a.N) return cudaErrorInvalidValue;
+    a.nbn = stack ? 1 : a.Cin / a.N;
+    a.nbm = stack ? 1 : (a.Cout + 127) / 128;
     // M = 64 for at most 64 output channels: an MMA reads half as much of A (24 cycles against 40 at
     // N = 32; 222 -> 180 us for 32 x 32 x 9 over 2.1 M pixels)
-    a.M = a.Cout <= 64 ? 64 : 128;
-    a.ga = (a.Cout < a.M ? a.Cout : a.M) / 32;
+    a.M = stack ? 4 * a.Cin : (a.Cout <= 64 ? 64 : 128);
+    a.ga = stack ? a.Cout / 32 : (a.Cout < a.M ? a.Cout : a.M) / 32;
     a.cbx = a.Cin % 32 == 0 ? 32 : 16;
     // taps per block: as many N-column accumulators as the 512 TMEM columns hold, in groups of
     // balanced size
-    // (N <= 32: of half the columns, for two blocks per SM, whose issuing warps overlap: 174 -> 133 us
-    // for 32 x 32 x 9 over 2.1 M pixels, although each block loads every tile)
-    const int maxt = a.N <= 32 ? 256 / a.N : 512 / a.N;
+    const int maxt = stack ? 9 : 512 / a.N;
     a.ngroups = (a.T + maxt - 1) / maxt;
     a.tpc = (a.T + a.ngroups - 1) / a.ngroups;
     const int h = a.T == 9 ? 1 : 0;
     // tile height: 8 pixel rows when three stages of it fit in shared memory, else 4
-    auto stage_bytes = [&](int ky) { return wg_stage_bytes(a.M, a.ga, a.N, ky, h); };
+    auto stage_bytes = [&](int ky) {
+        return stack ? wg_stacked_x_bytes(a.Cin, ky) + (uint32_t)(a.ga * WG_KX * ky * 64) : wg_stage_bytes(a.M, a.ga, a.N, ky, h);
+    };
     a.ky = stage_bytes(8) * 3 <= 196u * 1024u ? 8 : 4;
     const uint32_t stage = stage_bytes(a.ky);
-    const bool two = a.tpc * a.N <= 256 && stage * 3 <= 100u * 1024u;   // room for two blocks per SM
+    a.stage = (int)stage;
+    a.xbytes = stack ? (int)wg_stacked_x_bytes(a.Cin, a.ky) : 0;
+    // (32 input channels with taps stacked: one block per SM.  Two are 12 % faster, but the sums of twice
+    // as many chunks round otherwise)
+    const bool two = (stack ? a.Cin == 16 : a.tpc * a.N <= 256) && stage * 3 <= 100u * 1024u;   // room for two blocks per SM
     int S = (int)((two ? 100u * 1024u : 196u * 1024u) / stage);
     a.stages = S > 6 ? 6 : S;
     if (a.stages < 2) return cudaErrorInvalidConfiguration;
@@ -781,7 +831,9 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_tc_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        e = cudaFuncSetAttribute(k_tc_wgrad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(k_tc_wgrad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
@@ -803,10 +855,11 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st) {
     const size_t smem = (size_t)a.stages * stage + 8 * (2 * a.stages + 1) + 16;
     CUtensorMap gmap, xmap;
     if (!encode_nhwc_blocks(gmap, a.g, a.B, a.H, a.W, a.Cout, 32, WG_KX, a.ky, a.ga) ||
-        !encode_nhwc_blocks(xmap, a.in, a.B, a.H, a.W, a.Cin, a.cbx, WG_KX + 2 * h, a.ky + 2 * h, a.N / a.cbx))
+        !encode_nhwc_blocks(xmap, a.in, a.B, a.H, a.W, a.Cin, a.cbx, WG_KX + 2 * h, a.ky + 2 * h, stack ? 1 : a.N / a.cbx))
         return cudaErrorInvalidValue;
     const int64_t grid = (int64_t)a.chunks * per_chunk_blocks;
-    k_tc_wgrad<<<(unsigned)grid, WG_THREADS, smem, st>>>(gmap, xmap, a);
+    if (stack) k_tc_wgrad<true><<<(unsigned)grid, WG_THREADS, smem, st>>>(gmap, xmap, a);
+    else k_tc_wgrad<false><<<(unsigned)grid, WG_THREADS, smem, st>>>(gmap, xmap, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return reduce_wgrad(a.part, a.chunks, count, a.Cout, dw, db, st);
