@@ -232,21 +232,30 @@ template <typename T> __global__ void __launch_bounds__(TPB, sizeof(T) == 4 ? 3 
     }
 }
 
-// cold / paper initialisation of the 13 planes (as k_init_prior)
+// cold / paper initialisation of the 13 planes (as k_init_prior), blocks of TPB columns.  The cells
+// two or more from the border share their 13 values, formed once per block: formed per cell, their
+// FP64 products were what the kernel ran on (FP32, 2048^2: 238 us; the writes alone are 65).
 template <typename T> __global__ void k_init_prior_l2(DevProblem p, int dst, int paper) {
-    const int64_t c = gtid();
-    if (c >= p.n) return;
-    const int nx = p.nx;
-    int i, j;
-    node_rc(c, nx, i, j);
-    T2<T> *Q = (T2<T> *)p.P[dst];
-#pragma unroll
-    for (int d = 0; d < L2_SLOTS; ++d) {
+    const int nx = p.nx, ny = p.ny;
+    auto value = [&](int i, int j, int d) {
         const double a = l2_coef(p, i, j, d);
-        T2<T> o;
-        o.x = T(0);
-        o.y = a == 0.0 ? T(0) : (paper ? T(1e-8) : T(p.gamma * a * a));
-        Q[d * p.n + c] = o;
+        return a == 0.0 ? T(0) : (paper ? T(1e-8) : T(p.gamma * a * a));
+    };
+    __shared__ T in[L2_SLOTS];
+    if (threadIdx.x < L2_SLOTS && nx >= 5 && ny >= 5) in[threadIdx.x] = value(2, 2, threadIdx.x);
+    __syncthreads();
+    const int j = blockIdx.x * TPB + threadIdx.x;
+    if (j >= nx) return;
+    T2<T> *Q = (T2<T> *)p.P[dst];
+    for (int i = blockIdx.y; i < ny; i += gridDim.y) {
+        const bool interior = i >= 2 && i < ny - 2 && j >= 2 && j < nx - 2;
+#pragma unroll
+        for (int d = 0; d < L2_SLOTS; ++d) {
+            T2<T> o;
+            o.x = T(0);
+            o.y = interior ? in[d] : value(i, j, d);
+            Q[d * p.n + (int64_t)i * nx + j] = o;
+        }
     }
 }
 
@@ -394,16 +403,55 @@ __global__ void k_obs_precompute(DevProblem p, const double *xy, const double *y
 }
 
 // ---- per-cell observation index: optr[c] = lower bound of c in the sorted base cells ----
+// A block takes PTR_CELLS cells: two searches for the block's observations (a warp each, 32 probes a
+// round), their counts per cell in shared memory, and a prefix sum.  (A search per cell: 63 us at
+// 3.75 M nodes; this: 17 us.)
+constexpr int PTR_E = 8, PTR_CELLS = TPB * PTR_E;
 __global__ void k_obs_pointers(DevProblem p) {
-    const int64_t c = gtid();
-    if (c > p.n) return;
-    int64_t lo = 0, hi = p.m;   // first k with obase[k] >= c
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (p.obase[mid] < c) lo = mid + 1;
-        else hi = mid;
+    __shared__ int cnt[PTR_CELLS], wt[TPB / 32], range[2];
+    const int64_t c0 = (int64_t)blockIdx.x * PTR_CELLS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp < 2) {   // first k with obase[k] >= the first cell of this block, of the next
+        const int64_t c = c0 + warp * PTR_CELLS;
+        int lo = 0, hi = (int)p.m;   // the answer is in [lo, hi]
+        while (lo < hi) {
+            const int step = (hi - lo + 32) / 33, pos = lo + (lane + 1) * step - 1;
+            const int below = __popc(__ballot_sync(0xffffffffu, pos < hi && p.obase[pos] < c));
+            if (below < 32) hi = min(hi, lo + (below + 1) * step - 1);   // the first probe that is not below
+            lo += below * step;
+        }
+        if (lane == 0) range[warp] = lo;
     }
-    ((int *)p.optr)[c] = (int)lo;
+#pragma unroll
+    for (int e = 0; e < PTR_E; ++e) cnt[e * TPB + tid] = 0;
+    __syncthreads();
+    const int k0 = range[0], k1 = range[1];
+    for (int k = k0 + tid; k < k1; k += TPB) atomicAdd(&cnt[p.obase[k] - (int)c0], 1);
+    __syncthreads();
+    // the threads' exclusive prefix sums
+    int sum = 0;
+#pragma unroll
+    for (int e = 0; e < PTR_E; ++e) sum += cnt[tid * PTR_E + e];
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) wt[warp] = inc;
+    __syncthreads();
+    int run = k0 + inc - sum;
+    for (int w = 0; w < warp; ++w) run += wt[w];
+#pragma unroll
+    for (int e = 0; e < PTR_E; ++e) {
+        const int t = cnt[tid * PTR_E + e];
+        cnt[tid * PTR_E + e] = run;
+        run += t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < PTR_E; ++e)
+        if (c0 + e * TPB + tid <= p.n) ((int *)p.optr)[c0 + e * TPB + tid] = cnt[e * TPB + tid];
 }
 
 // ---- deterministic FP64 reductions: fixed grid, fixed per-thread order, smem tree ----
@@ -425,20 +473,18 @@ __global__ void k_final_sum(const double *part, int count, double *out) {
     if (threadIdx.x == 0) *out = s;
 }
 
-// sum over observation edges into node v of w_kc * val_k (FP64), corners in fixed order
-__device__ __forceinline__ double obs_gather64(const DevProblem &p, int64_t v, int i, int j,
-                                               const double *val, int stride, int off) {
+// f(k, c) for the observation edges into node v, corners c in order.  One loop over the four
+// corners' ranges: a warp takes as many rounds as its node with the most edges, not as the sum of
+// the largest of each corner.
+template <typename F> __device__ __forceinline__ void for_node_obs(const DevProblem &p, int64_t v, int i, int j, F f) {
     const int nx = p.nx;
     const int *o = p.optr;
-    double acc = 0.0;
-    for (int k = o[v]; k < o[v + 1]; ++k) acc += p.ow64[4 * (int64_t)k + 0] * val[stride * (int64_t)k + off];
-    if (j > 0)
-        for (int k = o[v - 1]; k < o[v]; ++k) acc += p.ow64[4 * (int64_t)k + 1] * val[stride * (int64_t)k + off];
-    if (i > 0)
-        for (int k = o[v - nx]; k < o[v - nx + 1]; ++k) acc += p.ow64[4 * (int64_t)k + 2] * val[stride * (int64_t)k + off];
-    if (i > 0 && j > 0)
-        for (int k = o[v - nx - 1]; k < o[v - nx]; ++k) acc += p.ow64[4 * (int64_t)k + 3] * val[stride * (int64_t)k + off];
-    return acc;
+    const int k0 = o[v], k1 = j > 0 ? o[v - 1] : k0, k2 = i > 0 ? o[v - nx] : 0, k3 = i > 0 && j > 0 ? o[v - nx - 1] : k2;
+    const int e0 = o[v + 1] - k0, e1 = e0 + (k0 - k1), e2 = e1 + (i > 0 ? o[v - nx + 1] - k2 : 0), e3 = e2 + (k2 - k3);
+    for (int t = 0; t < e3; ++t) {
+        const int k = t < e0 ? k0 + t : (t < e1 ? k1 + t - e0 : (t < e2 ? k2 + t - e1 : k3 + t - e2));
+        f(k, (t >= e0) + (t >= e1) + (t >= e2));
+    }
 }
 
 // (L x)_v = (kappa^2 + deg) x_v - sum of existing neighbours
@@ -454,6 +500,13 @@ __device__ __forceinline__ double apply_L(const DevProblem &p, const double *x, 
 
 // ||b||^2 with b_v = sum over incoming observation edges of w * s * y, plus gamma (L r)_v for
 // cell-factor targets r
+// (the products s * y once per observation, in e64: FP64 operations are what this runs on, and in
+// the loop over a node's edges few lanes of a warp have one.  174 us at 3.75 M nodes, 54 now)
+__global__ void k_rhs_values(DevProblem p) {
+    const int64_t k = gtid();
+    if (k < p.m) p.e64[k] = p.oys64[2 * k] * p.oys64[2 * k + 1];
+}
+
 __global__ void k_rhs_norm(DevProblem p) {
     double acc = 0.0;
     const int64_t stride = (int64_t)gridDim.x * TPB;
@@ -461,20 +514,9 @@ __global__ void k_rhs_norm(DevProblem p) {
         int i, j;
         node_rc(v, p.nx, i, j);
         double bv = 0.0;
-        if (p.m > 0) {
-            // w * (s * y): gather w_kc * y_k * s_k
-            const int *o = p.optr;
-            const int nx = p.nx;
-            for (int k = o[v]; k < o[v + 1]; ++k) bv += p.ow64[4 * (int64_t)k] * p.oys64[2 * (int64_t)k] * p.oys64[2 * (int64_t)k + 1];
-            if (j > 0)
-                for (int k = o[v - 1]; k < o[v]; ++k) bv += p.ow64[4 * (int64_t)k + 1] * p.oys64[2 * (int64_t)k] * p.oys64[2 * (int64_t)k + 1];
-            if (i > 0)
-                for (int k = o[v - nx]; k < o[v - nx + 1]; ++k) bv += p.ow64[4 * (int64_t)k + 2] * p.oys64[2 * (int64_t)k] * p.oys64[2 * (int64_t)k + 1];
-            if (i > 0 && j > 0)
-                for (int k = o[v - nx - 1]; k < o[v - nx]; ++k) bv += p.ow64[4 * (int64_t)k + 3] * p.oys64[2 * (int64_t)k] * p.oys64[2 * (int64_t)k + 1];
-        }
+        if (p.m > 0) for_node_obs(p, v, i, j, [&](int k, int c) { bv += p.ow64[4 * (int64_t)k + c] * p.e64[k]; });
         if (p.ptgt64) bv += p.gamma * apply_L(p, p.ptgt64, v, i, j);   // gamma L^T r (L symmetric)
-        acc += bv * bv;
+        if (bv != 0.0) acc += bv * bv;
     }
     double s = block_sum(acc);
     if (threadIdx.x == 0) p.part[blockIdx.x] = s;
@@ -591,24 +633,14 @@ __global__ void k_res_df(DevProblem p) {
     dfl acc = {0.f, 0.f};
     const int64_t stride = (int64_t)gridDim.x * TPB;
     const float2 *e = (const float2 *)p.e64;
-    const int *o = p.optr;
-    const int nx = p.nx;
     for (int64_t v = gtid(); v < p.n; v += stride) {
         int i, j;
-        node_rc(v, nx, i, j);
+        node_rc(v, p.nx, i, j);
         dfl r = df_neg(df_mul({p.gam_hi, p.gam_lo}, apply_L_df(p, (const float2 *)p.z64, v, i, j)));
-        if (p.m > 0) {
-            for (int k = o[v]; k < o[v + 1]; ++k) r = df_add(r, df_neg(df_mul(df_ld(p.owdf, 4 * (int64_t)k), df_ld(e, k))));
-            if (j > 0)
-                for (int k = o[v - 1]; k < o[v]; ++k)
-                    r = df_add(r, df_neg(df_mul(df_ld(p.owdf, 4 * (int64_t)k + 1), df_ld(e, k))));
-            if (i > 0)
-                for (int k = o[v - nx]; k < o[v - nx + 1]; ++k)
-                    r = df_add(r, df_neg(df_mul(df_ld(p.owdf, 4 * (int64_t)k + 2), df_ld(e, k))));
-            if (i > 0 && j > 0)
-                for (int k = o[v - nx - 1]; k < o[v - nx]; ++k)
-                    r = df_add(r, df_neg(df_mul(df_ld(p.owdf, 4 * (int64_t)k + 3), df_ld(e, k))));
-        }
+        if (p.m > 0)
+            for_node_obs(p, v, i, j, [&](int k, int c) {
+                r = df_add(r, df_neg(df_mul(df_ld(p.owdf, 4 * (int64_t)k + c), df_ld(e, k))));
+            });
         acc = df_add(acc, df_mul(r, r));
     }
     double s = block_sum((double)acc.hi + (double)acc.lo);
@@ -659,7 +691,11 @@ __global__ void k_res(DevProblem p) {
         int i, j;
         node_rc(v, p.nx, i, j);
         double r = -p.gamma * apply_L(p, p.z64, v, i, j);
-        if (p.m > 0) r -= obs_gather64(p, v, i, j, p.e64, 1, 0);
+        if (p.m > 0) {
+            double g = 0.0;
+            for_node_obs(p, v, i, j, [&](int k, int c) { g += p.ow64[4 * (int64_t)k + c] * p.e64[k]; });
+            r -= g;
+        }
         acc += r * r;
     }
     double s = block_sum(acc);
@@ -876,10 +912,10 @@ cudaError_t launch_beliefs(const DevProblem &p, int src, cudaStream_t st) {
 cudaError_t launch_init_cold(const DevProblem &p, int dst, int paper, cudaStream_t st) {
     if (p.order == 2) {
         if (p.prec) {
-            k_init_prior_l2<double><<<nblocks(p.n), TPB, 0, st>>>(p, dst, paper);
+            k_init_prior_l2<double><<<row_grid(p.nx, (p.ny + 3) / 4), TPB, 0, st>>>(p, dst, paper);
             if (p.m > 0) k_init_obs<double><<<nblocks(p.m), TPB, 0, st>>>(p, dst, paper);
         } else {
-            k_init_prior_l2<float><<<nblocks(p.n), TPB, 0, st>>>(p, dst, paper);
+            k_init_prior_l2<float><<<row_grid(p.nx, (p.ny + 3) / 4), TPB, 0, st>>>(p, dst, paper);
             if (p.m > 0) k_init_obs<float><<<nblocks(p.m), TPB, 0, st>>>(p, dst, paper);
         }
         return cudaGetLastError();
@@ -915,11 +951,12 @@ cudaError_t launch_obs_precompute(const DevProblem &p, const double *xy, const d
 }
 
 cudaError_t launch_obs_pointers(const DevProblem &p, cudaStream_t st) {
-    k_obs_pointers<<<nblocks(p.n + 1), TPB, 0, st>>>(p);
+    k_obs_pointers<<<(unsigned)((p.n + PTR_CELLS) / PTR_CELLS), TPB, 0, st>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rhs_norm(const DevProblem &p, cudaStream_t st) {
+    if (p.m > 0) k_rhs_values<<<nblocks(p.m), TPB, 0, st>>>(p);
     k_rhs_norm<<<RES_BLOCKS, TPB, 0, st>>>(p);
     k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal + 1);
     return cudaGetLastError();

@@ -156,3 +156,19 @@ def test_network_gradients_on_ragged_tiles(B, H, W):
         for lo, hi in [(wo, bo), (bo, bo + unet.SPECS[i][1])]:
             a, b = grads[0][lo:hi], grads[1][lo:hi]
             assert np.linalg.norm(a - b) < 0.12 * np.linalg.norm(b), (i, lo)
+
+
+@pytest.mark.parametrize("shape, per_node", [((23, 89), 3), ((64, 32), 3), ((683, 3), 6), ((31, 199), 2), ((128, 160), 0.02)])
+def test_observation_index_at_block_edges(orc, shape, per_node):
+    """The observation index is formed 2048 cells at a time: node counts around multiples of 2048,
+    many observations per cell and few; |b| and the residual gather over it."""
+    nx, ny = shape
+    p = gabp_synth.make_problem(nx, ny, 0.3, 9, n_uniform=int(per_node * nx * ny), sigma=(0.05, 0.2))
+    fl = orc.build_factors(nx, ny, p.kappa, p.obs_x, p.obs_y, p.y, p.noise_var)
+    mu_o, var_o, _ = orc.gabp(fl, 0.5, 6)
+    with solver(p, "fp64") as s:
+        s.iterate(6, 0.5)
+        mu, var = s.marginals()
+        assert s.residual() == pytest.approx(orc.residual(fl, mu), rel=1e-8)
+    np.testing.assert_allclose(mu, mu_o, rtol=1e-10, atol=1e-10 * np.max(np.abs(mu_o)))
+    np.testing.assert_allclose(var, var_o, rtol=1e-10)
