@@ -1302,14 +1302,18 @@ int batch_residuals(gabp_batch *b) {
         if (b->g_res) cudaGraphExecDestroy(b->g_res);
         b->g_res = nullptr;
         cudaGraph_t g = nullptr;
+        double *out = nullptr;   // the pinned scalars, written by the last kernel
+        BK(cudaHostGetDevicePointer((void **)&out, b->h_scal, 0), "pinned scalars");
         BK(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
-        cudaError_t le = cudaSuccess;
-        for (int i = 0; i < count && le == cudaSuccess; ++i) {
-            le = gabp::launch_residual(b->inst[i]->p, b->cur, b->cap);
-            if (le == cudaSuccess)
-                le = cudaMemcpyAsync(b->h_scal + 2 * i, b->inst[i]->p.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                     b->cap);
+        int64_t max_n = 0, sum_n = 0, max_m = 0, sum_m = 0;
+        for (const gabp_ctx *c : b->inst) {
+            max_n = std::max(max_n, c->p.n);
+            max_m = std::max(max_m, c->p.m);
+            sum_n += c->p.n;
+            sum_m += c->p.m;
         }
+        cudaError_t le =
+            gabp::launch_residual_batch(b->d_table, count, max_n, sum_n, max_m, sum_m, b->cur, out, b->cap);
         if (le == cudaSuccess)
             le = cudaMemcpyAsync(b->h_scal + 2 * count, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->cap);
         cudaError_t ee = cudaStreamEndCapture(b->cap, &g);

@@ -126,6 +126,10 @@ cudaError_t launch_obs_sort(int64_t m, int nx, int ny, const double *xy, const d
                             int *obase, double *sxy, double *sy, double *svar, void *scratch, cudaStream_t st);
 // residual of the messages in buffer src; leaves ||r||^2 in scal[0] (beliefs recomputed)
 cudaError_t launch_residual(const DevProblem &p, int src, cudaStream_t st);
+// residuals of the members of a batch (their problems at t on the device; the largest and the summed
+// node and observation counts): (|r|^2, |b|^2) per member to out
+cudaError_t launch_residual_batch(const DevProblem *t, int count, int64_t max_n, int64_t sum_n, int64_t max_m,
+                                  int64_t sum_m, int src, double *out, cudaStream_t st);
 // ---- the alpha = 4 prior (order 2: cell factors = rows of L^2, 13 planes; gabp_split.cu) ----
 // one synchronous iteration (beliefs, cell factors, observation factors); initialisation as
 // launch_init_cold (which dispatches on p.order, as do launch_beliefs, launch_residual and

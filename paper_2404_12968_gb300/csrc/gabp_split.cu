@@ -473,6 +473,19 @@ __global__ void k_final_sum(const double *part, int count, double *out) {
     if (threadIdx.x == 0) *out = s;
 }
 
+// the same of every member of a batch; out: (|r|^2, |b|^2) per member
+__global__ void k_final_sum_batch(const DevProblem *t, double *out) {
+    const DevProblem &p = t[blockIdx.x];
+    double acc = 0.0;
+    for (int q = threadIdx.x; q < RES_BLOCKS; q += TPB) acc += p.part[q];
+    const double s = block_sum(acc);
+    if (threadIdx.x == 0) {
+        p.scal[0] = s;
+        out[2 * blockIdx.x] = s;
+        out[2 * blockIdx.x + 1] = p.scal[1];
+    }
+}
+
 // f(k, c) for the observation edges into node v, corners c in order.  One loop over the four
 // corners' ranges: a warp takes as many rounds as its node with the most edges, not as the sum of
 // the largest of each corner.
@@ -581,28 +594,42 @@ __device__ __forceinline__ dfl df_belief_mean(const BeliefStore<float> &b) {
     return df_fast2sum(q1, q2);
 }
 
+// The problem of a block in the FP32 residual's kernels: the kernel parameter, or member blockIdx.y
+// of a batch's table (whose grid is sized for the average member: the loops stride).
+struct OneProblem {
+    DevProblem p;
+    __device__ __forceinline__ const DevProblem &operator()() const { return p; }
+};
+struct BatchTable {
+    const DevProblem *t;
+    __device__ __forceinline__ const DevProblem &operator()() const { return t[blockIdx.y]; }
+};
+__device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * blockDim.x; }
+
 // the same mean straight from the messages of buffer src (the belief kept in registers, not
 // stored): the FP32 residual's first pass
-__global__ void k_mu_direct_df(DevProblem p, int src) {
-    const int64_t v = gtid();
-    if (v >= p.n) return;
-    int i, j;
-    node_rc(v, p.nx, i, j);
-    df_st((float2 *)p.mu64, v, df_belief_mean(node_belief<float>(p, v, i, j, src)));
+template <typename S> __global__ void k_mu_direct_df(const S s, int src) {
+    const DevProblem &p = s();
+    for (int64_t v = gtid(); v < p.n; v += gstride()) {
+        int i, j;
+        node_rc(v, p.nx, i, j);
+        df_st((float2 *)p.mu64, v, df_belief_mean(node_belief<float>(p, v, i, j, src)));
+    }
 }
 
 // e_k = s_k (h_k . mu - y_k)
-__global__ void k_obs_err_df(DevProblem p) {
-    const int64_t k = gtid();
-    if (k >= p.m) return;
-    const int64_t b = p.obase[k];
+template <typename S> __global__ void k_obs_err_df(const S s) {
+    const DevProblem &p = s();
     const float2 *mu = (const float2 *)p.mu64;
-    const int64_t nodes[4] = {b, b + 1, b + p.nx, b + p.nx + 1};
-    dfl hm = df_mul(df_ld(p.owdf, 4 * k), df_ld(mu, nodes[0]));
+    for (int64_t k = gtid(); k < p.m; k += gstride()) {
+        const int64_t b = p.obase[k];
+        const int64_t nodes[4] = {b, b + 1, b + p.nx, b + p.nx + 1};
+        dfl hm = df_mul(df_ld(p.owdf, 4 * k), df_ld(mu, nodes[0]));
 #pragma unroll
-    for (int c = 1; c < 4; ++c) hm = df_add(hm, df_mul(df_ld(p.owdf, 4 * k + c), df_ld(mu, nodes[c])));
-    const dfl e = df_mul(df_ld(p.oysdf, 2 * k + 1), df_add(hm, df_neg(df_ld(p.oysdf, 2 * k))));
-    df_st((float2 *)p.e64, k, e);
+        for (int c = 1; c < 4; ++c) hm = df_add(hm, df_mul(df_ld(p.owdf, 4 * k + c), df_ld(mu, nodes[c])));
+        const dfl e = df_mul(df_ld(p.oysdf, 2 * k + 1), df_add(hm, df_neg(df_ld(p.oysdf, 2 * k))));
+        df_st((float2 *)p.e64, k, e);
+    }
 }
 
 // (L x)_v with the zero-Neumann stencil: (kappa^2 + deg) x_v - sum of the existing neighbours
@@ -617,19 +644,21 @@ __device__ __forceinline__ dfl apply_L_df(const DevProblem &p, const float2 *x, 
     return s;
 }
 
-__global__ void k_Lmu_df(DevProblem p) {
-    const int64_t v = gtid();
-    if (v >= p.n) return;
-    int i, j;
-    node_rc(v, p.nx, i, j);
-    dfl z = apply_L_df(p, (const float2 *)p.mu64, v, i, j);
-    if (p.ptgtdf) z = df_add(z, df_neg(df_ld(p.ptgtdf, v)));   // l_v . mu - r_v
-    df_st((float2 *)p.z64, v, z);
+template <typename S> __global__ void k_Lmu_df(const S s) {
+    const DevProblem &p = s();
+    for (int64_t v = gtid(); v < p.n; v += gstride()) {
+        int i, j;
+        node_rc(v, p.nx, i, j);
+        dfl z = apply_L_df(p, (const float2 *)p.mu64, v, i, j);
+        if (p.ptgtdf) z = df_add(z, df_neg(df_ld(p.ptgtdf, v)));   // l_v . mu - r_v
+        df_st((float2 *)p.z64, v, z);
+    }
 }
 
 // partial sums of r_v^2, r = b - A mu = -gamma L (L mu) - H^T (s (H mu - y)); per-thread sums in
 // double-float, then the same fixed-order FP64 block reduction as the FP64 path
-__global__ void k_res_df(DevProblem p) {
+template <typename S> __global__ void k_res_df(const S s) {
+    const DevProblem &p = s();
     dfl acc = {0.f, 0.f};
     const int64_t stride = (int64_t)gridDim.x * TPB;
     const float2 *e = (const float2 *)p.e64;
@@ -643,8 +672,8 @@ __global__ void k_res_df(DevProblem p) {
             });
         acc = df_add(acc, df_mul(r, r));
     }
-    double s = block_sum((double)acc.hi + (double)acc.lo);
-    if (threadIdx.x == 0) p.part[blockIdx.x] = s;
+    const double sum = block_sum((double)acc.hi + (double)acc.lo);
+    if (threadIdx.x == 0) p.part[blockIdx.x] = sum;
 }
 
 template <typename T> __global__ void k_mu(DevProblem p) {
@@ -996,9 +1025,10 @@ cudaError_t launch_df_precompute(const DevProblem &p, cudaStream_t st) {
 cudaError_t launch_residual_mu(const DevProblem &p, cudaStream_t st) {
     if (p.order == 2) return cudaErrorInvalidValue;   // order-2 contexts: launch_residual only
     if (p.prec == 0) {
-        if (p.m > 0) k_obs_err_df<<<nblocks(p.m), TPB, 0, st>>>(p);
-        k_Lmu_df<<<nblocks(p.n), TPB, 0, st>>>(p);
-        k_res_df<<<RES_BLOCKS, TPB, 0, st>>>(p);
+        const OneProblem s{p};
+        if (p.m > 0) k_obs_err_df<<<nblocks(p.m), TPB, 0, st>>>(s);
+        k_Lmu_df<<<nblocks(p.n), TPB, 0, st>>>(s);
+        k_res_df<<<RES_BLOCKS, TPB, 0, st>>>(s);
     } else {
         if (p.m > 0) k_obs_err<<<nblocks(p.m), TPB, 0, st>>>(p);
         k_Lmu<<<nblocks(p.n), TPB, 0, st>>>(p);
@@ -1011,12 +1041,8 @@ cudaError_t launch_residual_mu(const DevProblem &p, cudaStream_t st) {
 cudaError_t launch_residual(const DevProblem &p, int src, cudaStream_t st) {
     if (p.order == 1 && p.prec == 0) {
         // FP32 messages: the residual in double-float arithmetic (FP32 pipes, ~48-bit significands)
-        k_mu_direct_df<<<nblocks(p.n), TPB, 0, st>>>(p, src);
-        if (p.m > 0) k_obs_err_df<<<nblocks(p.m), TPB, 0, st>>>(p);
-        k_Lmu_df<<<nblocks(p.n), TPB, 0, st>>>(p);
-        k_res_df<<<RES_BLOCKS, TPB, 0, st>>>(p);
-        k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal);
-        return cudaGetLastError();
+        k_mu_direct_df<<<nblocks(p.n), TPB, 0, st>>>(OneProblem{p}, src);
+        return launch_residual_mu(p, st);
     }
     cudaError_t e = launch_beliefs(p, src, st);
     if (e != cudaSuccess) return e;
@@ -1039,6 +1065,30 @@ cudaError_t launch_residual(const DevProblem &p, int src, cudaStream_t st) {
     k_Lmu<<<nblocks(p.n), TPB, 0, st>>>(p);
     k_res<<<RES_BLOCKS, TPB, 0, st>>>(p);
     k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal);
+    return cudaGetLastError();
+}
+
+// The residuals of a batch's members (FP32, alpha = 2; t: their problems on the device) in five
+// launches, (|r|^2, |b|^2) per member to out (device-accessible).  A chain of launches per member,
+// in one graph, took 580 us for 16 grids of 128^2 to 1024^2, this 286.  The grid gives every member
+// up to four times the blocks of the average one, so that no mix of sizes launches many more empty
+// blocks than full ones.
+cudaError_t launch_residual_batch(const DevProblem *t, int count, int64_t max_n, int64_t sum_n, int64_t max_m,
+                                  int64_t sum_m, int src, double *out, cudaStream_t st) {
+    auto width = [&](int64_t most, int64_t sum) {
+        const unsigned fair = 4 * nblocks((sum + count - 1) / count);
+        return std::min(nblocks(most), std::max(fair, 64u));
+    };
+    constexpr int ROWS = 32768;   // members per launch (grid.y is at most 65535)
+    for (int i = 0; i < count; i += ROWS) {
+        const unsigned rows = (unsigned)std::min(ROWS, count - i);
+        const BatchTable s{t + i};
+        k_mu_direct_df<<<dim3(width(max_n, sum_n), rows), TPB, 0, st>>>(s, src);
+        if (max_m > 0) k_obs_err_df<<<dim3(width(max_m, sum_m), rows), TPB, 0, st>>>(s);
+        k_Lmu_df<<<dim3(width(max_n, sum_n), rows), TPB, 0, st>>>(s);
+        k_res_df<<<dim3(RES_BLOCKS, rows), TPB, 0, st>>>(s);
+        k_final_sum_batch<<<rows, TPB, 0, st>>>(t + i, out + 2 * i);
+    }
     return cudaGetLastError();
 }
 

@@ -172,3 +172,18 @@ def test_observation_index_at_block_edges(orc, shape, per_node):
         assert s.residual() == pytest.approx(orc.residual(fl, mu), rel=1e-8)
     np.testing.assert_allclose(mu, mu_o, rtol=1e-10, atol=1e-10 * np.max(np.abs(mu_o)))
     np.testing.assert_allclose(var, var_o, rtol=1e-10)
+
+
+def test_batch_residuals_of_very_uneven_members():
+    """One grid of 352 blocks among grids of one: the batch's residual kernels give a member four times
+    the average member's blocks (68), so the large one strides.  The same sums as a single context."""
+    from paper_2404_12968_gb300 import Batch
+    probs = [_problem(300, 300)] + [_problem(8 + i, 8, seed=i) for i in range(20)] + [gabp_synth.make_problem(9, 8, 0.1, 4)]
+    with Batch(probs, tile_y=14) as b:
+        for iters in (8, 7):   # both message buffers
+            b.iterate(iters, 0.3)
+            res = b.residuals()
+        for i, p in enumerate(probs):
+            with solver(p, "fp32") as s:
+                s.iterate(15, 0.3)
+                assert s.residual() == res[i], i
