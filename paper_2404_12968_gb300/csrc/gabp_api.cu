@@ -195,8 +195,12 @@ int sync_scalars(gabp_ctx *c, int first, const char *what) {
 }
 
 // Graph of `len` (even) iterations starting from buffer 0.
+bool graph_ready(const gabp_ctx *c, int len, double beta) {
+    return c->gexec && c->g_len == len && c->g_beta == beta && c->g_kernel == c->kernel;
+}
+
 int ensure_graph(gabp_ctx *c, int len, double beta) {
-    if (c->gexec && c->g_len == len && c->g_beta == beta && c->g_kernel == c->kernel) return GABP_OK;
+    if (graph_ready(c, len, beta)) return GABP_OK;
     drop_graph(c);
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
@@ -229,6 +233,13 @@ int run_iterations(gabp_ctx *c, int64_t count, double beta) {
         ++c->iters;
     }
     if (count >= G) {
+        if (!graph_ready(c, G, beta)) {
+            // the first G iterations launched one by one: the GPU works on them while the host captures
+            // and instantiates the graph (80 us, as long as 16 iterations of a 361 x 181 grid take)
+            for (int t = 0; t < G; ++t) CK(launch_iteration(c, t & 1, beta, c->stream), "iteration launch");
+            count -= G;
+            c->iters += G;
+        }
         int rc = ensure_graph(c, G, beta);
         if (rc != GABP_OK) return rc;
         while (count >= G) {
