@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import gabp_synth
-from gpu_common import ensure_built, solver
+from gpu_common import decode_messages, ensure_built, solver, sorted_obs_order
 
 pytestmark = pytest.mark.gpu
 
@@ -187,3 +187,19 @@ def test_batch_residuals_of_very_uneven_members():
             with solver(p, "fp32") as s:
                 s.iterate(15, 0.3)
                 assert s.residual() == res[i], i
+
+
+@pytest.mark.parametrize("m", [1, 31, 33, 1024, 1025, 4097, 16383, 16384, 16385])
+@pytest.mark.parametrize("shape", [(2, 3), (19, 13), (201, 330)])
+def test_observation_sort_in_one_block(orc, m, shape):
+    """Up to 16384 observations one block sorts them, beyond that the passes over many: the stable
+    order by base cell, for cell counts of one, two and three 8-bit digits, with many ties."""
+    nx, ny = shape
+    rng = np.random.default_rng(m + nx)
+    x, y = rng.uniform(0, nx - 1, m), rng.uniform(0, ny - 1, m)
+    x[m // 3:m // 2], y[m // 3:m // 2] = 0.5, ny - 1.0
+    p = gabp_synth.Problem(nx, ny, 0.3, x, y, rng.normal(size=m), rng.uniform(0.01, 0.2, m))
+    order, base, w = sorted_obs_order(orc, p)
+    with solver(p, "fp64") as s:
+        _, obs = decode_messages(s.get_messages(), p, "fp64")
+    np.testing.assert_allclose(obs[:, :, 1], (w ** 2 / p.noise_var[:, None])[order], rtol=1e-12, atol=0)
