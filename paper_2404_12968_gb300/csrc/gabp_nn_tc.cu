@@ -168,14 +168,27 @@ __device__ __forceinline__ uint32_t relu_bf16(uint32_t v) {   // max(., 0); roun
 __device__ __forceinline__ uint32_t positive_mask(uint32_t v) {   // all ones in the halves above zero
     return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&v), __nv_bfloat162(__float2bfloat16(0.f), __float2bfloat16(0.f)));
 }
+// 16 channels of a pixel (32 bytes, aligned) in one 256-bit access: a whole sector per lane (two
+// 128-bit stores made two partial writes of each: 85 -> 72 us for 32 x 32 x 9 over 2.1 M pixels,
+// 112 -> 98 us with the loads too for 64 x 32 x 1 with upsampling, 0.5 M to 2.1 M)
 __device__ __forceinline__ void store16_bf16(__nv_bfloat16 *dst, const uint32_t (&v)[8]) {
-    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
-    reinterpret_cast<uint4 *>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                 "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+__device__ __forceinline__ void load16_bf16(const __nv_bfloat16 *src, uint32_t (&v)[8]) {
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "l"(src));
+}
+__device__ __forceinline__ void prefetch_l2(const __nv_bfloat16 *p, uint32_t bytes) {   // multiples of 16
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 template <int N, int T, int CB>
 __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant__ CUtensorMap in_map, TcConvArgs a) {
     using IN = InTile<T, CB>;
+    constexpr bool UP = T == 1;   // the epilogues: 1x1 convolutions may upsample, 3x3 ones may pool or have the head
     constexpr uint32_t WBYTES = (uint32_t)T * 2 * CB * N;      // weight slab of one channel block
     extern __shared__ __align__(1024) unsigned char smem[];
     const int S = a.stages;
@@ -245,6 +258,16 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
             for (int64_t tile = blockIdx.x; tile < ntiles && !*fail; tile += gridDim.x) {
                 int b, y0, x0, nb;
                 tile_coords(tile, b, y0, x0, nb);
+                if (a.nblocks == 1 && (a.mask || a.up_out)) {   // what this tile's epilogue reads, towards L2
+                    const int w = min(TILE_X, a.W - x0), h = min(TILE_Y, a.H - y0);
+                    if (a.mask)
+                        for (int y = y0; y < y0 + h; ++y)
+                            prefetch_l2(a.mask + (((int64_t)b * a.H + y) * a.W + x0) * a.Cout, (uint32_t)(w * a.Cout) * 2);
+                    if (a.up_out)
+                        for (int y = 2 * y0; y < 2 * (y0 + h); ++y)
+                            prefetch_l2(a.up_skip + (((int64_t)b * (2 * a.H) + y) * (2 * a.W) + 2 * x0) * a.Cout,
+                                        (uint32_t)(2 * w * a.Cout) * 2);
+                }
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = (int)(it % S);
                     const uint32_t use = (uint32_t)(it / S);
@@ -317,14 +340,23 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
             const bool valid = gy < a.H && gx < a.W;
             const int co0 = nb * N;
             const int64_t pix = ((int64_t)b * a.H + gy) * a.W + gx;
+            auto fine = [&](int q) {   // pixel q of the 2 x 2 above this one on the twice as fine grid
+                return (((int64_t)b * (2 * a.H) + 2 * gy + (q >> 1)) * (2 * a.W) + 2 * gx + (q & 1)) * a.Cout;
+            };
             float h0 = 0.f, h1 = 0.f;
-            if (a.head_w) {
+            if (!UP && a.head_w) {
                 h0 = a.head_b[0];
                 h1 = a.head_b[1];
             }
 #pragma unroll 1
             for (int c = 0; c < N; c += 16) {
                 uint32_t r[16], v[8];   // 16 channels: FP32 sums, BF16 pairs
+                // the mask and the skip tensor first: all their loads in flight at once
+                uint32_t mk[8], sv[4][8];
+                if (a.mask && valid) load16_bf16(a.mask + pix * a.Cout + co0 + c, mk);
+                if (UP && a.up_out && valid)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) load16_bf16(a.up_skip + fine(q) + co0 + c, sv[q]);
                 tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * N + c), r);
                 const float4 *bias4 = reinterpret_cast<const float4 *>(a.bias + co0 + c);
 #pragma unroll
@@ -336,15 +368,11 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
                 if (a.relu)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[j] = relu_bf16(v[j]);
-                if (a.mask && valid) {   // the ReLU's backward: zero where its output was not positive
-                    const uint4 *ms = reinterpret_cast<const uint4 *>(a.mask + pix * a.Cout + co0 + c);
-                    const uint4 m0 = ms[0], m1 = ms[1];
-                    const uint32_t mk[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                if (a.mask && valid)   // the ReLU's backward: zero where its output was not positive
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[j] &= positive_mask(mk[j]);
-                }
                 if (a.out && valid) store16_bf16(a.out + pix * a.Cout + co0 + c, v);
-                if (a.pool_out) {
+                if (!UP && a.pool_out) {
                     // 2x2 sum, scaled: (y, x), (y, x+1), (y+1, x), (y+1, x+1) are lanes +0, +1, +8, +9
                     uint32_t pv[8];
 #pragma unroll
@@ -359,23 +387,18 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
                         store16_bf16(a.pool_out + q * a.Cout + co0 + c, pv);
                     }
                 }
-                if (a.up_out && valid) {
+                if (UP && a.up_out && valid) {
                     // nearest upsampling to (2H, 2W) plus the skip tensor there
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const int fy = 2 * gy + (q >> 1), fx = 2 * gx + (q & 1);
-                        const int64_t fp = ((int64_t)b * (2 * a.H) + fy) * (2 * a.W) + fx;
-                        const uint4 *sk = reinterpret_cast<const uint4 *>(a.up_skip + fp * a.Cout + co0 + c);
-                        const uint4 s0 = sk[0], s1 = sk[1];
-                        const uint32_t sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
                         uint32_t u[8];
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            u[j] = pack_bf16(bf_lo(v[j]) + bf_lo(sv[j]), bf_hi(v[j]) + bf_hi(sv[j]));
-                        store16_bf16(a.up_out + fp * a.Cout + co0 + c, u);
+                            u[j] = pack_bf16(bf_lo(v[j]) + bf_lo(sv[q][j]), bf_hi(v[j]) + bf_hi(sv[q][j]));
+                        store16_bf16(a.up_out + fine(q) + co0 + c, u);
                     }
                 }
-                if (a.head_w) {
+                if (!UP && a.head_w) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const float f = j & 1 ? bf_hi(v[j >> 1]) : bf_lo(v[j >> 1]);
@@ -384,7 +407,7 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
                     }
                 }
             }
-            if (a.head_w && valid) {
+            if (!UP && a.head_w && valid) {
                 a.head_out[2 * pix] = h0;
                 a.head_out[2 * pix + 1] = h1;
             }
@@ -882,8 +905,8 @@ cudaError_t tc_conv(const __nv_bfloat16 *in, TcConvArgs a, cudaStream_t st) {
         a.H < 1 || a.B < 1)
         return cudaErrorInvalidValue;
     if (a.pool_out && (a.H % 2 || a.W % 2)) return cudaErrorInvalidValue;
-    if (a.up_out && !a.up_skip) return cudaErrorInvalidValue;
-    if (a.head_w && a.Cout != 32) return cudaErrorInvalidValue;
+    if (a.up_out && (!a.up_skip || a.T != 1)) return cudaErrorInvalidValue;
+    if ((a.head_w && (a.Cout != 32 || a.T != 9)) || (a.pool_out && a.T != 9)) return cudaErrorInvalidValue;
     auto enc = tc_encoder();
     if (!enc) return cudaErrorNotSupported;
     a.nblocks = a.Cout / N;
