@@ -181,10 +181,6 @@ __device__ __forceinline__ void load16_bf16(const __nv_bfloat16 *src, uint32_t (
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                  : "l"(src));
 }
-__device__ __forceinline__ void prefetch_l2(const __nv_bfloat16 *p, uint32_t bytes) {   // multiples of 16
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 template <int N, int T, int CB>
 __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant__ CUtensorMap in_map, TcConvArgs a) {
     using IN = InTile<T, CB>;
@@ -258,16 +254,6 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
             for (int64_t tile = blockIdx.x; tile < ntiles && !*fail; tile += gridDim.x) {
                 int b, y0, x0, nb;
                 tile_coords(tile, b, y0, x0, nb);
-                if (a.nblocks == 1 && (a.mask || a.up_out)) {   // what this tile's epilogue reads, towards L2
-                    const int w = min(TILE_X, a.W - x0), h = min(TILE_Y, a.H - y0);
-                    if (a.mask)
-                        for (int y = y0; y < y0 + h; ++y)
-                            prefetch_l2(a.mask + (((int64_t)b * a.H + y) * a.W + x0) * a.Cout, (uint32_t)(w * a.Cout) * 2);
-                    if (a.up_out)
-                        for (int y = 2 * y0; y < 2 * (y0 + h); ++y)
-                            prefetch_l2(a.up_skip + (((int64_t)b * (2 * a.H) + y) * (2 * a.W) + 2 * x0) * a.Cout,
-                                        (uint32_t)(2 * w * a.Cout) * 2);
-                }
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = (int)(it % S);
                     const uint32_t use = (uint32_t)(it / S);
@@ -330,10 +316,6 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
         int lt = 0;
         for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++lt) {
             const int acc = lt & 1;
-            const bool ok = mbar_wait(accf(acc), ((uint32_t)lt >> 1) & 1);
-            if (!ok) *fail = 1;
-            if (__any_sync(0xffffffffu, !ok) || *fail) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             int b, y0, x0, nb;
             tile_coords(tile, b, y0, x0, nb);
             const int gy = y0 + yy, gx = x0 + xx;
@@ -343,6 +325,20 @@ __global__ void __launch_bounds__(TC_THREADS, 4) k_tc_conv(const __grid_constant
             auto fine = [&](int q) {   // pixel q of the 2 x 2 above this one on the twice as fine grid
                 return (((int64_t)b * (2 * a.H) + 2 * gy + (q >> 1)) * (2 * a.W) + 2 * gx + (q & 1)) * a.Cout;
             };
+            // what the epilogue reads, towards L2 while the accumulator is made (a tile earlier, by the
+            // producer, 80 MB in flight ran each other out of L2: the skip tensor was read twice)
+            if (UP && a.up_out && valid)
+#pragma unroll
+                for (int q = 0; q < 4; q += N == 32 ? 2 : 1)
+#pragma unroll
+                    for (int c = 0; c < N; c += 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.up_skip + fine(q) + co0 + c));
+            if (a.mask && valid)
+#pragma unroll
+                for (int c = 0; c < N; c += 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.mask + pix * a.Cout + co0 + c));
+            const bool ok = mbar_wait(accf(acc), ((uint32_t)lt >> 1) & 1);
+            if (!ok) *fail = 1;
+            if (__any_sync(0xffffffffu, !ok) || *fail) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             float h0 = 0.f, h1 = 0.f;
             if (!UP && a.head_w) {
                 h0 = a.head_b[0];
