@@ -455,6 +455,9 @@ __global__ void k_obs_pointers(DevProblem p) {
 }
 
 // ---- deterministic FP64 reductions: fixed grid, fixed per-thread order, smem tree ----
+// The kernels on this grid of RES_BLOCKS = 1024 blocks are bounded to the registers of 7 blocks per SM,
+// 1064 on 152 SMs: at 6 (39 registers, 912 blocks) a ninth of the blocks ran in a second round of their
+// own (2048^2: k_res_df 59 -> 54 us, k_rhs_norm 52 -> 44, k_res 89 -> 83).
 __device__ __forceinline__ double block_sum(double x) {
     __shared__ double sh[TPB];
     sh[threadIdx.x] = x;
@@ -514,13 +517,13 @@ __device__ __forceinline__ double apply_L(const DevProblem &p, const double *x, 
 // ||b||^2 with b_v = sum over incoming observation edges of w * s * y, plus gamma (L r)_v for
 // cell-factor targets r
 // (the products s * y once per observation, in e64: FP64 operations are what this runs on, and in
-// the loop over a node's edges few lanes of a warp have one.  174 us at 3.75 M nodes, 54 now)
+// the loop over a node's edges few lanes of a warp have one.  174 us at 3.75 M nodes, 46 now)
 __global__ void k_rhs_values(DevProblem p) {
     const int64_t k = gtid();
     if (k < p.m) p.e64[k] = p.oys64[2 * k] * p.oys64[2 * k + 1];
 }
 
-__global__ void k_rhs_norm(DevProblem p) {
+__global__ void __launch_bounds__(TPB, 7) k_rhs_norm(DevProblem p) {
     double acc = 0.0;
     const int64_t stride = (int64_t)gridDim.x * TPB;
     for (int64_t v = gtid(); v < p.n; v += stride) {
@@ -644,7 +647,7 @@ __device__ __forceinline__ dfl apply_L_df(const DevProblem &p, const float2 *x, 
     return s;
 }
 
-template <typename S> __global__ void k_Lmu_df(const S s) {
+template <typename S> __global__ void __launch_bounds__(TPB, 8) k_Lmu_df(const S s) {
     const DevProblem &p = s();
     for (int64_t v = gtid(); v < p.n; v += gstride()) {
         int i, j;
@@ -657,7 +660,7 @@ template <typename S> __global__ void k_Lmu_df(const S s) {
 
 // partial sums of r_v^2, r = b - A mu = -gamma L (L mu) - H^T (s (H mu - y)); per-thread sums in
 // double-float, then the same fixed-order FP64 block reduction as the FP64 path
-template <typename S> __global__ void k_res_df(const S s) {
+template <typename S> __global__ void __launch_bounds__(TPB, 7) k_res_df(const S s) {
     const DevProblem &p = s();
     dfl acc = {0.f, 0.f};
     const int64_t stride = (int64_t)gridDim.x * TPB;
@@ -713,7 +716,7 @@ __global__ void k_Lmu(DevProblem p) {
 }
 
 // r = b - A mu = -gamma L (L mu) - H^T S (H mu - y); accumulate ||r||^2
-__global__ void k_res(DevProblem p) {
+__global__ void __launch_bounds__(TPB, 7) k_res(DevProblem p) {
     double acc = 0.0;
     const int64_t stride = (int64_t)gridDim.x * TPB;
     for (int64_t v = gtid(); v < p.n; v += stride) {
