@@ -489,19 +489,43 @@ __global__ void k_final_sum_batch(const DevProblem *t, double *out) {
     }
 }
 
-// f(k, c) for the observation edges into node v, corners c in order.  One loop over the four
-// corners' ranges: a warp takes as many rounds as its node with the most edges, not as the sum of
-// the largest of each corner.
-template <typename F> __device__ __forceinline__ void for_node_obs(const DevProblem &p, int64_t v, int i, int j, F f) {
+// The observation edges into node v, corners c in order: add(load(k, c)) for each.  One loop over the
+// four corners' ranges: a warp takes as many rounds as its node with the most edges, not as the sum of
+// the largest of each corner.  GROUP edges' loads are in flight before the first of them is added.
+template <int GROUP, typename L, typename A>
+__device__ __forceinline__ void for_node_obs(const DevProblem &p, int64_t v, int i, int j, L load, A add) {
     const int nx = p.nx;
     const int *o = p.optr;
     const int k0 = o[v], k1 = j > 0 ? o[v - 1] : k0, k2 = i > 0 ? o[v - nx] : 0, k3 = i > 0 && j > 0 ? o[v - nx - 1] : k2;
     const int e0 = o[v + 1] - k0, e1 = e0 + (k0 - k1), e2 = e1 + (i > 0 ? o[v - nx + 1] - k2 : 0), e3 = e2 + (k2 - k3);
-    for (int t = 0; t < e3; ++t) {
-        const int k = t < e0 ? k0 + t : (t < e1 ? k1 + t - e0 : (t < e2 ? k2 + t - e1 : k3 + t - e2));
-        f(k, (t >= e0) + (t >= e1) + (t >= e2));
+    for (int t = 0; t < e3; t += GROUP) {
+        decltype(load(0, 0)) x[GROUP];
+#pragma unroll
+        for (int q = 0; q < GROUP; ++q) {
+            const int u = t + q;
+            const int k = u < e0 ? k0 + u : (u < e1 ? k1 + u - e0 : (u < e2 ? k2 + u - e1 : k3 + u - e2));
+            if (u < e3) x[q] = load(k, (u >= e0) + (u >= e1) + (u >= e2));
+        }
+#pragma unroll
+        for (int q = 0; q < GROUP; ++q)
+            if (t + q < e3) add(x[q]);
     }
 }
+
+// Which form of a kernel that gathers over for_node_obs a problem takes.  Where nodes have many edges
+// the time is the loop's, a latency per edge with one edge at a time, so they are taken in groups of
+// four, in 64 registers (in 32 a group spills).  Where most nodes have none, the grid's 1024 blocks in
+// one wave count for more: one edge at a time, in 32 registers.  The line is two observations per node.
+// k_rhs_norm / k_res (FP64) / k_res_df in us, one by one and in groups: 2048^2 with 0.04 per node 40 / 80 /
+// 52 and 55 / 95 / 53, 512^2 with 1.9 21 / 20 / 17 and 20 / 21 / 18, 1024^2 with 4.8 110 / 113 / 103 and
+// 99 / 104 / 84, 32^2 with 1367 2250 / 2205 / 2228 and 1098 / 1096 / 1140 (a loop per corner: 1756 / 1181 /
+// 1938).  The FP64 kernels also take the groups on grids whose threads all fit the chip in 64 registers:
+// nothing is lost there (64^2 with 0.07 per node 8.0 / 7.4 and 6.8 / 7.0) and clusters on few nodes are
+// met (2000 observations in one cell of 64 x 32: 576 / 586 and 356 / 356; a loop per corner 506 / 338).
+inline bool many_obs(int64_t n, int64_t m) { return m > 2 * n; }
+inline bool many_obs_f64(int64_t n, int64_t m) { return many_obs(n, m) || n <= 512 * (int64_t)TPB; }   // 4 blocks per SM
+template <bool MANY> constexpr int obs_group = MANY ? 4 : 1;
+template <bool MANY> constexpr int res_blocks_per_sm = MANY ? 4 : 7;
 
 // (L x)_v = (kappa^2 + deg) x_v - sum of existing neighbours
 __device__ __forceinline__ double apply_L(const DevProblem &p, const double *x, int64_t v, int i, int j) {
@@ -523,14 +547,17 @@ __global__ void k_rhs_values(DevProblem p) {
     if (k < p.m) p.e64[k] = p.oys64[2 * k] * p.oys64[2 * k + 1];
 }
 
-__global__ void __launch_bounds__(TPB, 7) k_rhs_norm(DevProblem p) {
+template <bool MANY> __global__ void __launch_bounds__(TPB, res_blocks_per_sm<MANY>) k_rhs_norm(DevProblem p) {
     double acc = 0.0;
     const int64_t stride = (int64_t)gridDim.x * TPB;
     for (int64_t v = gtid(); v < p.n; v += stride) {
         int i, j;
         node_rc(v, p.nx, i, j);
         double bv = 0.0;
-        if (p.m > 0) for_node_obs(p, v, i, j, [&](int k, int c) { bv += p.ow64[4 * (int64_t)k + c] * p.e64[k]; });
+        if (p.m > 0)
+            for_node_obs<obs_group<MANY>>(
+                p, v, i, j, [&](int k, int c) { return make_double2(p.ow64[4 * (int64_t)k + c], p.e64[k]); },
+                [&](double2 x) { bv += x.x * x.y; });
         if (p.ptgt64) bv += p.gamma * apply_L(p, p.ptgt64, v, i, j);   // gamma L^T r (L symmetric)
         if (bv != 0.0) acc += bv * bv;
     }
@@ -660,7 +687,7 @@ template <typename S> __global__ void __launch_bounds__(TPB, 8) k_Lmu_df(const S
 
 // partial sums of r_v^2, r = b - A mu = -gamma L (L mu) - H^T (s (H mu - y)); per-thread sums in
 // double-float, then the same fixed-order FP64 block reduction as the FP64 path
-template <typename S> __global__ void __launch_bounds__(TPB, 7) k_res_df(const S s) {
+template <bool MANY, typename S> __global__ void __launch_bounds__(TPB, res_blocks_per_sm<MANY>) k_res_df(const S s) {
     const DevProblem &p = s();
     dfl acc = {0.f, 0.f};
     const int64_t stride = (int64_t)gridDim.x * TPB;
@@ -670,9 +697,13 @@ template <typename S> __global__ void __launch_bounds__(TPB, 7) k_res_df(const S
         node_rc(v, p.nx, i, j);
         dfl r = df_neg(df_mul({p.gam_hi, p.gam_lo}, apply_L_df(p, (const float2 *)p.z64, v, i, j)));
         if (p.m > 0)
-            for_node_obs(p, v, i, j, [&](int k, int c) {
-                r = df_add(r, df_neg(df_mul(df_ld(p.owdf, 4 * (int64_t)k + c), df_ld(e, k))));
-            });
+            for_node_obs<obs_group<MANY>>(
+                p, v, i, j,
+                [&](int k, int c) {
+                    const float2 w = p.owdf[4 * (int64_t)k + c], y = e[k];
+                    return make_float4(w.x, w.y, y.x, y.y);
+                },
+                [&](float4 x) { r = df_add(r, df_neg(df_mul({x.x, x.y}, {x.z, x.w}))); });
         acc = df_add(acc, df_mul(r, r));
     }
     const double sum = block_sum((double)acc.hi + (double)acc.lo);
@@ -716,7 +747,7 @@ __global__ void k_Lmu(DevProblem p) {
 }
 
 // r = b - A mu = -gamma L (L mu) - H^T S (H mu - y); accumulate ||r||^2
-__global__ void __launch_bounds__(TPB, 7) k_res(DevProblem p) {
+template <bool MANY> __global__ void __launch_bounds__(TPB, res_blocks_per_sm<MANY>) k_res(DevProblem p) {
     double acc = 0.0;
     const int64_t stride = (int64_t)gridDim.x * TPB;
     for (int64_t v = gtid(); v < p.n; v += stride) {
@@ -725,7 +756,9 @@ __global__ void __launch_bounds__(TPB, 7) k_res(DevProblem p) {
         double r = -p.gamma * apply_L(p, p.z64, v, i, j);
         if (p.m > 0) {
             double g = 0.0;
-            for_node_obs(p, v, i, j, [&](int k, int c) { g += p.ow64[4 * (int64_t)k + c] * p.e64[k]; });
+            for_node_obs<obs_group<MANY>>(
+                p, v, i, j, [&](int k, int c) { return make_double2(p.ow64[4 * (int64_t)k + c], p.e64[k]); },
+                [&](double2 x) { g += x.x * x.y; });
             r -= g;
         }
         acc += r * r;
@@ -989,7 +1022,8 @@ cudaError_t launch_obs_pointers(const DevProblem &p, cudaStream_t st) {
 
 cudaError_t launch_rhs_norm(const DevProblem &p, cudaStream_t st) {
     if (p.m > 0) k_rhs_values<<<nblocks(p.m), TPB, 0, st>>>(p);
-    k_rhs_norm<<<RES_BLOCKS, TPB, 0, st>>>(p);
+    if (many_obs_f64(p.n, p.m)) k_rhs_norm<true><<<RES_BLOCKS, TPB, 0, st>>>(p);
+    else k_rhs_norm<false><<<RES_BLOCKS, TPB, 0, st>>>(p);
     k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal + 1);
     return cudaGetLastError();
 }
@@ -1025,17 +1059,25 @@ cudaError_t launch_df_precompute(const DevProblem &p, cudaStream_t st) {
 
 // the residual of a mean already in p.mu64 (double-float pairs for FP32 contexts, FP64 values
 // for FP64 contexts): the kernels after the mean in launch_residual
+namespace {
+void launch_res(const DevProblem &p, cudaStream_t st) {
+    if (many_obs_f64(p.n, p.m)) k_res<true><<<RES_BLOCKS, TPB, 0, st>>>(p);
+    else k_res<false><<<RES_BLOCKS, TPB, 0, st>>>(p);
+}
+}  // namespace
+
 cudaError_t launch_residual_mu(const DevProblem &p, cudaStream_t st) {
     if (p.order == 2) return cudaErrorInvalidValue;   // order-2 contexts: launch_residual only
     if (p.prec == 0) {
         const OneProblem s{p};
         if (p.m > 0) k_obs_err_df<<<nblocks(p.m), TPB, 0, st>>>(s);
         k_Lmu_df<<<nblocks(p.n), TPB, 0, st>>>(s);
-        k_res_df<<<RES_BLOCKS, TPB, 0, st>>>(s);
+        if (many_obs(p.n, p.m)) k_res_df<true><<<RES_BLOCKS, TPB, 0, st>>>(s);
+        else k_res_df<false><<<RES_BLOCKS, TPB, 0, st>>>(s);
     } else {
         if (p.m > 0) k_obs_err<<<nblocks(p.m), TPB, 0, st>>>(p);
         k_Lmu<<<nblocks(p.n), TPB, 0, st>>>(p);
-        k_res<<<RES_BLOCKS, TPB, 0, st>>>(p);
+        launch_res(p, st);
     }
     k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal);
     return cudaGetLastError();
@@ -1058,7 +1100,7 @@ cudaError_t launch_residual(const DevProblem &p, int src, cudaStream_t st) {
         k_Lx<<<nblocks(p.n), TPB, 0, st>>>(p, p.mu64, p.z64);
         k_Lx<<<nblocks(p.n), TPB, 0, st>>>(p, p.z64, p.mu64);
         k_Lx<<<nblocks(p.n), TPB, 0, st>>>(p, p.mu64, p.z64);
-        k_res<<<RES_BLOCKS, TPB, 0, st>>>(p);
+        launch_res(p, st);
         k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal);
         return cudaGetLastError();
     }
@@ -1066,7 +1108,7 @@ cudaError_t launch_residual(const DevProblem &p, int src, cudaStream_t st) {
     else k_mu<float><<<nblocks(p.n), TPB, 0, st>>>(p);
     if (p.m > 0) k_obs_err<<<nblocks(p.m), TPB, 0, st>>>(p);
     k_Lmu<<<nblocks(p.n), TPB, 0, st>>>(p);
-    k_res<<<RES_BLOCKS, TPB, 0, st>>>(p);
+    launch_res(p, st);
     k_final_sum<<<1, TPB, 0, st>>>(p.part, RES_BLOCKS, p.scal);
     return cudaGetLastError();
 }
@@ -1089,7 +1131,8 @@ cudaError_t launch_residual_batch(const DevProblem *t, int count, int64_t max_n,
         k_mu_direct_df<<<dim3(width(max_n, sum_n), rows), TPB, 0, st>>>(s, src);
         if (max_m > 0) k_obs_err_df<<<dim3(width(max_m, sum_m), rows), TPB, 0, st>>>(s);
         k_Lmu_df<<<dim3(width(max_n, sum_n), rows), TPB, 0, st>>>(s);
-        k_res_df<<<dim3(RES_BLOCKS, rows), TPB, 0, st>>>(s);
+        if (many_obs(sum_n, sum_m)) k_res_df<true><<<dim3(RES_BLOCKS, rows), TPB, 0, st>>>(s);
+        else k_res_df<false><<<dim3(RES_BLOCKS, rows), TPB, 0, st>>>(s);
         k_final_sum_batch<<<rows, TPB, 0, st>>>(t + i, out + 2 * i);
     }
     return cudaGetLastError();

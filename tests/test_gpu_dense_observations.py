@@ -1,0 +1,81 @@
+"""GPU: grids with many observations per node (the coarse levels of a multigrid hierarchy, clusters):
+the same results as the oracle, and no longer in time than their edges take.  Times are ratios, taken
+in one process from the fastest of several calls."""
+import time
+
+import numpy as np
+import pytest
+
+import gabp_synth
+from gpu_common import ensure_built, solver
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    ensure_built()
+
+
+def _dense(nx, ny, m, seed=3):
+    """m observations spread over the grid, in pinned arrays."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(seed)
+    xy, y, nv = (torch.empty(s, dtype=torch.float64, pin_memory=True).numpy() for s in ((m, 2), (m,), (m,)))
+    xy[...] = rng.uniform(0, 1, (m, 2)) * np.array([nx - 1.0, ny - 1.0])
+    y[...] = rng.standard_normal(m)
+    nv[...] = 0.1
+    return dict(nx=nx, ny=ny, kappa=0.2, obs_xy=xy, y=y, noise_var=nv)
+
+
+def _fastest(call, n):
+    best = float("inf")
+    for _ in range(n):
+        t = time.perf_counter()
+        call()
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+def _steady():
+    """1000 FP64 iterations of a 64 x 64 grid: a time that follows the SM clock alone."""
+    with solver(gabp_synth.make_problem(64, 64, 0.3, 1, n_uniform=500), "fp64") as s:
+        s.iterate(1000, 0.5)
+        return _fastest(lambda: s.iterate(1000, 0.5), 5)
+
+
+def test_residual_of_many_observations_per_node_in_time():
+    """1172 observations per node, FP32: 0.44 of 1000 small FP64 iterations with one load of an edge in
+    flight, 0.36 in a loop per corner, 0.33 in groups of four.  The bound: a loop per corner and 5 %."""
+    from paper_2404_12968_gb300 import Solver
+    with Solver(precision="fp32", **_dense(16, 16, 300000)) as s:
+        s.residual()
+        assert _fastest(s.residual, 20) < 0.38 * _steady()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("shape, m", [((2, 2), 3), ((2, 2), 9), ((17, 9), 306), ((17, 9), 307), ((64, 32), 9000), ((301, 437), 1000),
+                                      ((301, 437), 263075)])
+def test_residual_at_the_lines_of_its_forms(orc, precision, shape, m):
+    """Edge counts that are and are not multiples of the groups, and both sides of the lines: two
+    observations per node, 512 * 256 nodes."""
+    nx, ny = shape
+    p = gabp_synth.make_problem(nx, ny, 0.3, 9, n_uniform=m, sigma=(0.05, 0.2))
+    fl = orc.build_factors(nx, ny, p.kappa, p.obs_x, p.obs_y, p.y, p.noise_var)
+    with solver(p, precision) as s:
+        s.iterate(4, 0.5)
+        mu, _ = s.marginals()
+        assert s.residual() == pytest.approx(orc.residual(fl, mu), rel=1e-8)
+
+
+def test_batch_residuals_of_dense_members():
+    """Members with more than two observations per node on average: the same sums as single contexts."""
+    from paper_2404_12968_gb300 import Batch
+    probs = [gabp_synth.make_problem(n, n + 3, 0.3, n, n_uniform=k * n * n) for n, k in ((40, 5), (33, 3), (90, 4))]
+    with Batch(probs, tile_y=14) as b:
+        b.iterate(6, 0.3)
+        res = b.residuals()
+    for p, r in zip(probs, res):
+        with solver(p, "fp32") as s:
+            s.iterate(6, 0.3)
+            assert s.residual() == r
