@@ -403,16 +403,23 @@ __global__ void k_obs_precompute(DevProblem p, const double *xy, const double *y
 }
 
 // ---- per-cell observation index: optr[c] = lower bound of c in the sorted base cells ----
-// A block takes PTR_CELLS cells: two searches for the block's observations (a warp each, 32 probes a
+// A block takes E cells per thread: two searches for the block's observations (a warp each, 32 probes a
 // round), their counts per cell in shared memory, and a prefix sum.  (A search per cell: 63 us at
-// 3.75 M nodes; this: 17 us.)
-constexpr int PTR_E = 8, PTR_CELLS = TPB * PTR_E;
-__global__ void k_obs_pointers(DevProblem p) {
-    __shared__ int cnt[PTR_CELLS], wt[TPB / 32], range[2];
-    const int64_t c0 = (int64_t)blockIdx.x * PTR_CELLS;
+// 3.75 M nodes; this, E = 8: 17 us.)  Blocks with more than PTR_MANY observations per cell search per
+// cell instead, in the block's range, a thread's cells side by side: counted, 1.4 M observations on
+// 64 x 32 nodes kept one SM busy for 400 us (now 14, the plain search 13).  The counts are the faster
+// ones up to about 50 per cell (E = 1, 49 per cell: 10.9 us both; 21: 9.6 against 11.4).  One cell per
+// thread (E = 1) up to 2^18 nodes, where larger blocks leave SMs idle (512^2 with 1.9 per node 9.9 and
+// 7.7 us, 256^2 with 21 21 and 9.6; 1024^2 with 4.8 14.4 and 19.5, 2500 x 1500 16.5 and 29).
+constexpr int PTR_MANY = 48;
+constexpr int64_t PTR_SMALL_NODES = (int64_t)1 << 18;
+template <int E> __global__ void k_obs_pointers(DevProblem p) {
+    constexpr int CELLS = TPB * E;
+    __shared__ int cnt[CELLS], wt[TPB / 32], range[2];
+    const int64_t c0 = (int64_t)blockIdx.x * CELLS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (warp < 2) {   // first k with obase[k] >= the first cell of this block, of the next
-        const int64_t c = c0 + warp * PTR_CELLS;
+        const int64_t c = c0 + warp * CELLS;
         int lo = 0, hi = (int)p.m;   // the answer is in [lo, hi]
         while (lo < hi) {
             const int step = (hi - lo + 32) / 33, pos = lo + (lane + 1) * step - 1;
@@ -423,15 +430,29 @@ __global__ void k_obs_pointers(DevProblem p) {
         if (lane == 0) range[warp] = lo;
     }
 #pragma unroll
-    for (int e = 0; e < PTR_E; ++e) cnt[e * TPB + tid] = 0;
+    for (int e = 0; e < E; ++e) cnt[e * TPB + tid] = 0;
     __syncthreads();
     const int k0 = range[0], k1 = range[1];
+    if (k1 - k0 > PTR_MANY * CELLS) {
+        const int len = k1 - k0, c = (int)c0 + tid;
+        int pos[E];   // of the block's observations, those before cell c + e TPB
+#pragma unroll
+        for (int e = 0; e < E; ++e) pos[e] = 0;
+        for (int step = 1 << (31 - __clz(len)); step > 0; step >>= 1)
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (pos[e] + step <= len && p.obase[k0 + pos[e] + step - 1] < c + e * TPB) pos[e] += step;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (c0 + e * TPB + tid <= p.n) ((int *)p.optr)[c0 + e * TPB + tid] = k0 + pos[e];
+        return;
+    }
     for (int k = k0 + tid; k < k1; k += TPB) atomicAdd(&cnt[p.obase[k] - (int)c0], 1);
     __syncthreads();
     // the threads' exclusive prefix sums
     int sum = 0;
 #pragma unroll
-    for (int e = 0; e < PTR_E; ++e) sum += cnt[tid * PTR_E + e];
+    for (int e = 0; e < E; ++e) sum += cnt[tid * E + e];
     int inc = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -443,14 +464,14 @@ __global__ void k_obs_pointers(DevProblem p) {
     int run = k0 + inc - sum;
     for (int w = 0; w < warp; ++w) run += wt[w];
 #pragma unroll
-    for (int e = 0; e < PTR_E; ++e) {
-        const int t = cnt[tid * PTR_E + e];
-        cnt[tid * PTR_E + e] = run;
+    for (int e = 0; e < E; ++e) {
+        const int t = cnt[tid * E + e];
+        cnt[tid * E + e] = run;
         run += t;
     }
     __syncthreads();
 #pragma unroll
-    for (int e = 0; e < PTR_E; ++e)
+    for (int e = 0; e < E; ++e)
         if (c0 + e * TPB + tid <= p.n) ((int *)p.optr)[c0 + e * TPB + tid] = cnt[e * TPB + tid];
 }
 
@@ -1016,7 +1037,8 @@ cudaError_t launch_obs_precompute(const DevProblem &p, const double *xy, const d
 }
 
 cudaError_t launch_obs_pointers(const DevProblem &p, cudaStream_t st) {
-    k_obs_pointers<<<(unsigned)((p.n + PTR_CELLS) / PTR_CELLS), TPB, 0, st>>>(p);
+    if (p.n <= PTR_SMALL_NODES) k_obs_pointers<1><<<(unsigned)((p.n + TPB) / TPB), TPB, 0, st>>>(p);
+    else k_obs_pointers<8><<<(unsigned)((p.n + 8 * TPB) / (8 * TPB)), TPB, 0, st>>>(p);
     return cudaGetLastError();
 }
 

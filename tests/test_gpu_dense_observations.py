@@ -79,3 +79,41 @@ def test_batch_residuals_of_dense_members():
         with solver(p, "fp32") as s:
             s.iterate(6, 0.3)
             assert s.residual() == r
+
+
+def test_creation_on_few_nodes_in_time():
+    """4 M observations on 64 x 32 nodes: creation takes 2.0 times that on 256 x 256 nodes; 2.5 with all
+    of them counted by one block of the observation index, 2.4 with a search per cell and a loop per
+    corner in the right-hand side.  The bound: between, 2.25."""
+    from paper_2404_12968_gb300 import Solver
+    best = []
+    for nx, ny in ((64, 32), (256, 256)):
+        kw = _dense(nx, ny, 4000000)
+        best.append(_fastest(lambda: Solver(precision="fp32", **kw).close(), 12))
+    assert best[0] < 2.25 * best[1]
+
+
+@pytest.mark.parametrize("shape, m, patch", [((32, 32), 49000, None), ((32, 32), 49400, None), ((64, 33), 13000, (0, 0, 1, 1)),
+                                             ((64, 33), 13000, (62, 31, 1, 1)), ((512, 512), 14000, (508, 508, 3, 3)),
+                                             ((513, 512), 100000, (100, 500, 40, 9)), ((601, 500), 100000, (0, 0, 599, 3)),
+                                             ((601, 500), 98000, (560, 480, 40, 19)), ((2, 2), 20000, None)])
+def test_observation_index_of_clusters(orc, shape, m, patch):
+    """Blocks of the observation index that search per cell (more than 48 observations per cell of 256 or
+    2048) beside blocks that count, at the first and the last cells, and both cells per thread (up to
+    512^2 nodes and above).  The residual gathers over the index."""
+    nx, ny = shape
+    rng = np.random.default_rng(m + nx)
+    x0, y0, w, h = patch or (0, 0, nx - 1, ny - 1)
+    x, y = x0 + w * rng.uniform(0, 1, m), y0 + h * rng.uniform(0, 1, m)
+    k = max(nx * ny // 50, 1)   # a few everywhere
+    x[:k], y[:k] = rng.uniform(0, nx - 1, k), rng.uniform(0, ny - 1, k)
+    p = gabp_synth.Problem(nx, ny, 0.3, x, y, rng.normal(size=m), rng.uniform(0.01, 0.2, m))
+    fl = orc.build_factors(nx, ny, p.kappa, p.obs_x, p.obs_y, p.y, p.noise_var)
+    with solver(p, "fp64") as s:
+        s.iterate(2, 0.5)
+        mu, _ = s.marginals()
+        assert s.residual() == pytest.approx(orc.residual(fl, mu), rel=1e-8)
+        split = solver(p, "fp64", kernel=2)
+        split.iterate(2, 0.5)
+        assert np.array_equal(split.get_messages(), s.get_messages())
+        split.close()
