@@ -117,3 +117,16 @@ def test_observation_index_of_clusters(orc, shape, m, patch):
         split.iterate(2, 0.5)
         assert np.array_equal(split.get_messages(), s.get_messages())
         split.close()
+
+
+def test_split_observation_factors_in_time():
+    """Split form, FP32, 1601^2 nodes: an iteration with 5 M observations takes 2.4 times one with 84 k;
+    2.6 and 3.0 with word-wide accesses of the observation factors, as the compiler orders them.  The
+    bound: 2.75."""
+    from paper_2404_12968_gb300 import GABP_KERNEL_SPLIT, Solver
+    best = []
+    for m in (5000000, 84000):
+        with Solver(precision="fp32", kernel=GABP_KERNEL_SPLIT, **_dense(1601, 1601, m)) as s:
+            s.iterate(40, 0.3)
+            best.append(_fastest(lambda: s.iterate(100, 0.3), 6))
+    assert best[0] < 2.75 * best[1]
