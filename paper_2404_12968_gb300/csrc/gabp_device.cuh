@@ -173,12 +173,30 @@ template <typename T> struct Belief {
 // base (x-1, row) with corner cl for indices [lo, mid) and base (x, row) with corner cr for
 // [mid, hi).  The two ranges are adjacent in the base-sorted observation array, so the terms
 // are added in increasing observation index; every iteration kernel uses this order (corners
-// 1, 0 from the node's row, then 3, 2 from the row below).
+// 1, 0 from the node's row, then 3, 2 from the row below).  Four terms' loads are in flight together; the
+// rest one by one, in a loop that is not unrolled: most nodes have a term or two, and code for more of
+// them costs those.  Sweep kernel, 63^2 nodes with 0.1, 3 and 10 observations each: 103, 295 and 660 us per
+// iteration; one loop as the compiler unrolls it 110, 301 and 655, by words 109, 294 and 667.
+constexpr int OBS_LOADS = 4;
 template <typename T>
 __device__ __forceinline__ void add_obs_pair(CompSum<T> &se, CompSum<T> &sl, const T *O, int lo, int mid,
                                              int hi, int cl, int cr) {
-    for (int k = lo; k < hi; ++k) {
-        const T2<T> q = *reinterpret_cast<const T2<T> *>(O + 8 * (int64_t)k + 2 * (k < mid ? cl : cr));
+    const T2<T> *Q = reinterpret_cast<const T2<T> *>(O) + 4u * (unsigned)lo;
+    int l = mid - lo, n = hi - lo;
+#pragma unroll 1
+    for (; n >= OBS_LOADS; n -= OBS_LOADS, l -= OBS_LOADS, Q += 4 * OBS_LOADS) {
+        T2<T> x[OBS_LOADS];
+#pragma unroll
+        for (int q = 0; q < OBS_LOADS; ++q) x[q] = Q[4 * q + (q < l ? cl : cr)];
+#pragma unroll
+        for (int q = 0; q < OBS_LOADS; ++q) {
+            se.add(x[q].x);
+            sl.add(x[q].y);
+        }
+    }
+#pragma unroll 1
+    for (; n > 0; --n, --l, Q += 4) {
+        const T2<T> q = Q[l > 0 ? cl : cr];
         se.add(q.x);
         sl.add(q.y);
     }
