@@ -543,18 +543,14 @@ __global__ void __launch_bounds__(WNT) k_fused_f64_wide(const __grid_constant__ 
 
 // SMs of the current device (looked up once per device)
 int sm_count() {
-    static int dev_cached = -1, nsm = 152;
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev != dev_cached) {
-        int v = 0;
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0) {
-            nsm = v;
-            dev_cached = dev;
-        } else {
-            cudaGetLastError();
-        }
-    }
-    return nsm;
+    static PerDevice<int> cache;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cache.get(dev, nsm, [&](int &v) { return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev); }) == cudaSuccess &&
+        nsm > 0)
+        return nsm;
+    cudaGetLastError();
+    return 152;
 }
 
 constexpr int F64_MAX_TY = 32;   // a warp holds the tile's row ranges
@@ -573,13 +569,16 @@ cudaError_t launch_f64(const DevProblem &p, int ty, int src, double beta, cudaSt
 template <typename T, int TX, int TY>
 cudaError_t launch_shape(const DevProblem &p, int src, double beta, cudaStream_t st) {
     using LY = FusedLayout<T, TX, TY>;
-    static bool configured = false;   // per instantiation; the attribute is per function
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k_fused<T, TX, TY>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice<bool> configured;   // per instantiation; the attribute is per function and device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    bool set = false;
+    e = configured.get(dev, set, [](bool &v) {
+        v = true;
+        return cudaFuncSetAttribute(k_fused<T, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes);
+    });
+    if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + TY - 1) / TY));
     k_fused<T, TX, TY><<<grid, FT, LY::bytes, st>>>(p, src, (T)beta);
     return cudaGetLastError();

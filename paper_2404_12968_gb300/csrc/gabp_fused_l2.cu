@@ -267,15 +267,14 @@ __global__ void __launch_bounds__(32 * TY, 24 / TY)
 
 // persistent grid of k_fused_l2<TY>: SMs x resident blocks (set up once per device)
 template <int TY> cudaError_t l2_persistent_grid(int &grid) {
-    static int grid_cache = 0;
-    static int configured_dev = -1;
+    static PerDevice<int> cache;
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
+    const cudaError_t ge = cudaGetDevice(&dev);
+    if (ge != cudaSuccess) return ge;
+    return cache.get(dev, grid, [&](int &blocks) {
         // shared memory is only the belief windows: leave the rest of the SM's storage to L1,
         // which holds the message planes between phase A and phase B
-        e = cudaFuncSetAttribute(k_fused_l2<TY>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+        cudaError_t e = cudaFuncSetAttribute(k_fused_l2<TY>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
         if (e != cudaSuccess) return e;
         int nsm = 0, per_sm = 0;
         e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -283,11 +282,9 @@ template <int TY> cudaError_t l2_persistent_grid(int &grid) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_l2<TY>, 32 * TY, 0);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        grid_cache = nsm * per_sm;
-        configured_dev = dev;
-    }
-    grid = grid_cache;
-    return cudaSuccess;
+        blocks = nsm * per_sm;
+        return cudaSuccess;
+    });
 }
 
 // Run length for nx x ny on 28 x TY tiles: among 1, 2, 4, 8 and 16 the one whose busiest block

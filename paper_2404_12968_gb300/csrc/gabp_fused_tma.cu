@@ -466,14 +466,13 @@ __global__ void __launch_bounds__(TileLayout<TY, S, RW>::TNT, DENSE ? 1 : TileLa
 // persistent grid of k_fused_tma<...>: SMs x resident blocks (set up once per device)
 template <int TY, int S, int RW, bool BATCH, bool DENSE = false> cudaError_t persistent_grid(int &grid) {
     using LY = TileLayout<TY, S, RW>;
-    static int grid_cache = 0;
-    static int configured_dev = -1;
+    static PerDevice<int> cache;
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_fused_tma<TY, S, RW, BATCH, DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)LY::bytes);
+    const cudaError_t ge = cudaGetDevice(&dev);
+    if (ge != cudaSuccess) return ge;
+    return cache.get(dev, grid, [&](int &blocks) {
+        cudaError_t e = cudaFuncSetAttribute(k_fused_tma<TY, S, RW, BATCH, DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)LY::bytes);
         if (e != cudaSuccess) return e;
         int nsm = 0, per_sm = 0;
         e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -481,11 +480,9 @@ template <int TY, int S, int RW, bool BATCH, bool DENSE = false> cudaError_t per
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_tma<TY, S, RW, BATCH, DENSE>, LY::TNT, LY::bytes);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        grid_cache = nsm * per_sm;
-        configured_dev = dev;
-    }
-    grid = grid_cache;
-    return cudaSuccess;
+        blocks = nsm * per_sm;
+        return cudaSuccess;
+    });
 }
 
 template <int TY, int S, int RW, bool DENSE = false>
@@ -519,7 +516,7 @@ cudaError_t launch_cfg(const DevProblem &p, const TmaMaps &maps, int src, double
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};   // every thread finds the same
     if (!fn) {
         void *ptr = nullptr;
         cudaDriverEntryPointQueryResult q;

@@ -7,6 +7,7 @@
 #include <string>
 
 #include "gabp_device.cuh"
+#include "gabp_per_device.h"
 
 namespace gabp {
 

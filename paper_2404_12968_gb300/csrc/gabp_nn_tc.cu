@@ -37,6 +37,7 @@
 #include <stdint.h>
 
 #include "gabp_nn.h"
+#include "gabp_per_device.h"
 
 namespace gabp {
 namespace nn {
@@ -716,7 +717,7 @@ template <bool FLIP> __global__ void k_tc_pack(const __nv_bfloat16 *w, TcPackLay
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tc_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};   // every thread finds the same
     if (!fn) {
         void *ptr = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -738,8 +739,10 @@ bool tc_resident(const TcConvArgs &a, int N) { return a.nblocks == 1 && a.Cin * 
 template <int N, int T, int CB>
 cudaError_t tc_launch(const CUtensorMap &map, TcConvArgs a, cudaStream_t st) {
     using IN = InTile<T, CB>;
-    static int configured_dev = -1;
-    static int nsm = 0, occ_threads = 0;
+    struct Limits {
+        int nsm, occ_threads;
+    };
+    static PerDevice<Limits> cache;
     const uint32_t wbytes = (uint32_t)T * 2 * CB * N;
     const uint32_t wall = (uint32_t)(a.Cin / CB) * wbytes;
     a.resident = tc_resident(a, N) ? 1 : 0;
@@ -765,25 +768,27 @@ cudaError_t tc_launch(const CUtensorMap &map, TcConvArgs a, cudaStream_t st) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_tc_conv<N, T, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    Limits lim{};
+    e = cache.get(dev, lim, [&](Limits &v) {
+        cudaError_t e = cudaFuncSetAttribute(k_tc_conv<N, T, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        e = cudaDeviceGetAttribute(&v.nsm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         // registers and threads per SM from the kernel's attributes
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, k_tc_conv<N, T, CB>);
         if (e != cudaSuccess) return e;
         const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
-        occ_threads = 65536 / (regs_warp * (TC_THREADS / 32));
-        if (occ_threads > 2048 / TC_THREADS) occ_threads = 2048 / TC_THREADS;
-        configured_dev = dev;
-    }
+        v.occ_threads = 65536 / (regs_warp * (TC_THREADS / 32));
+        if (v.occ_threads > 2048 / TC_THREADS) v.occ_threads = 2048 / TC_THREADS;
+        return cudaSuccess;
+    });
+    if (e != cudaSuccess) return e;
     int per_sm = (int)((228 * 1024) / (smem + 1024));
-    if (per_sm > occ_threads) per_sm = occ_threads;
+    if (per_sm > lim.occ_threads) per_sm = lim.occ_threads;
     if (per_sm > tmem_cap) per_sm = tmem_cap;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    int64_t grid = (int64_t)nsm * per_sm;
+    int64_t grid = (int64_t)lim.nsm * per_sm;
     if (grid > a.ntiles) grid = a.ntiles;
     k_tc_conv<N, T, CB><<<(unsigned)grid, TC_THREADS, smem, st>>>(map, a);
     return cudaGetLastError();
@@ -845,19 +850,18 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st) {
     a.tiles_x = (a.W + WG_KX - 1) / WG_KX;
     a.tiles_y = (a.H + a.ky - 1) / a.ky;
     a.ktiles = (int64_t)a.B * a.tiles_y * a.tiles_x;
-    static int configured_dev = -1, nsm = 0;
-    int dev = 0;
+    static PerDevice<int> sms;
+    int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_tc_wgrad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = sms.get(dev, nsm, [&](int &v) {
+        cudaError_t e = cudaFuncSetAttribute(k_tc_wgrad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(k_tc_wgrad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        configured_dev = dev;
-    }
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    });
+    if (e != cudaSuccess) return e;
     // blocks: about one per SM per resident slot over (chunk, tap group, output block, input
     // block); every chunk's partial sums must fit the buffer
     const int64_t per_chunk_blocks = (int64_t)a.ngroups * a.nbm * a.nbn;

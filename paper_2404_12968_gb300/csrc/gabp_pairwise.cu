@@ -266,15 +266,16 @@ namespace {
 template <typename T>
 cudaError_t pw_launch(const DevProblem &p, const void *Pd, const void *hv, const void *Pn, const void *src, void *dst, double c,
                       double eta, cudaStream_t st) {
-    static int configured_dev = -1;
+    static PerDevice<bool> configured;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(k_pw_iter<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PwSlots<T>));
-        if (e != cudaSuccess) return e;
-        configured_dev = dev;
-    }
+    bool set = false;
+    e = configured.get(dev, set, [](bool &v) {
+        v = true;
+        return cudaFuncSetAttribute(k_pw_iter<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PwSlots<T>));
+    });
+    if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((p.n + PwSlots<T>::NT - 1) / PwSlots<T>::NT);
     return launch_pdl(true, k_pw_iter<T>, dim3(blocks), PwSlots<T>::NT, sizeof(PwSlots<T>), st, p.nx, p.ny, p.n, (const T *)Pd, (const T *)hv,
                       (const T *)Pn, (const T2<T> *)src, (T2<T> *)dst, (T)c, (T)(1.0 / c), (T)eta);

@@ -369,23 +369,30 @@ __global__ void __launch_bounds__(SWEEP_WARPS * 32)
     }
 }
 
-template <int H> cudaError_t launch_h(const DevProblem &p, int src, double beta, cudaStream_t st) {
-    static int grid_cache = 0, configured_dev = -1;
+// blocks of a kernel of SWEEP_WARPS warps that the device holds at once
+template <auto KERNEL> cudaError_t resident_blocks(int &blocks) {
+    static PerDevice<int> cache;
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
+    const cudaError_t ge = cudaGetDevice(&dev);
+    if (ge != cudaSuccess) return ge;
+    return cache.get(dev, blocks, [&](int &v) {
         int nsm = 0, per_sm = 0;
-        e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<H>, SWEEP_WARPS * 32, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, SWEEP_WARPS * 32, 0);
         if (e != cudaSuccess) return e;
-        grid_cache = nsm * (per_sm > 0 ? per_sm : 1);
-        configured_dev = dev;
-    }
+        v = nsm * (per_sm > 0 ? per_sm : 1);
+        return cudaSuccess;
+    });
+}
+
+template <int H> cudaError_t launch_h(const DevProblem &p, int src, double beta, cudaStream_t st) {
+    int resident = 0;   // blocks
+    const cudaError_t e = resident_blocks<k_sweep<H>>(resident);
+    if (e != cudaSuccess) return e;
     const int nstrips = ((p.nx + SW - 1) / SW) * ((p.ny + H - 1) / H);
     const int blocks = (nstrips + SWEEP_WARPS - 1) / SWEEP_WARPS;
-    const int grid = blocks < grid_cache ? blocks : grid_cache;
+    const int grid = blocks < resident ? blocks : resident;
     k_sweep<H><<<grid, SWEEP_WARPS * 32, 0, st>>>(p, src, (float)beta);
     return cudaGetLastError();
 }
@@ -400,21 +407,11 @@ namespace {
 template <int H>
 cudaError_t launch_batch_h(const DevProblem *table, const int *strip_start, const int *active, int count,
                            int total_strips, int src, double beta, cudaStream_t st) {
-    static int grid_cache = 0, configured_dev = -1;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    int resident = 0;   // blocks
+    const cudaError_t e = resident_blocks<k_sweep_batch<H>>(resident);
     if (e != cudaSuccess) return e;
-    if (configured_dev != dev) {
-        int nsm = 0, per_sm = 0;
-        e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_batch<H>, SWEEP_WARPS * 32, 0);
-        if (e != cudaSuccess) return e;
-        grid_cache = nsm * (per_sm > 0 ? per_sm : 1);
-        configured_dev = dev;
-    }
     const int blocks = (total_strips + SWEEP_WARPS - 1) / SWEEP_WARPS;
-    const int grid = blocks < grid_cache ? blocks : grid_cache;
+    const int grid = blocks < resident ? blocks : resident;
     if (grid < 1) return cudaSuccess;
     k_sweep_batch<H><<<grid, SWEEP_WARPS * 32, 0, st>>>(table, strip_start, active, count, src, (float)beta);
     return cudaGetLastError();
