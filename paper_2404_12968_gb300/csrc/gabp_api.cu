@@ -194,6 +194,22 @@ int sync_scalars(gabp_ctx *c, int first, const char *what) {
     return GABP_OK;
 }
 
+// Where a call's iterations started.  A kernel that gave up has written nothing: point back at the
+// messages of that point, which a check after an odd number of iterations would leave.
+struct CallStart {
+    gabp_ctx *c;
+    int cur;
+    int64_t iters;
+    explicit CallStart(gabp_ctx *ctx) : c(ctx), cur(ctx->cur), iters(ctx->iters) {}
+    int back_if_gave_up(int rc) const {   // rc: of sync_scalars or of what ends with it
+        if (rc == GABP_ERR_TIMEOUT) {
+            c->cur = cur;
+            c->iters = iters;
+        }
+        return rc;
+    }
+};
+
 // Graph of `len` (even) iterations starting from buffer 0.
 bool graph_ready(const gabp_ctx *c, int len, double beta) {
     return c->gexec && c->g_len == len && c->g_beta == beta && c->g_kernel == c->kernel;
@@ -776,22 +792,16 @@ int gabp_iterate(gabp_ctx *c, int n_iters, double damping) {
     DeviceGuard g(c->dev);
     if (!g.ok) return fail(c, GABP_ERR_CUDA, "cudaSetDevice failed");
     c->err.clear();
+    const CallStart start(c);
     if (n_iters >= 0) {
-        const int cur0 = c->cur;
-        const int64_t iters0 = c->iters;
         int rc = run_iterations(c, n_iters, damping);
         if (rc) return rc;
-        rc = sync_scalars(c, NSCAL, "iterate sync");
-        if (rc) {   // a kernel gave up: point back at the messages the call started from
-            c->cur = cur0;
-            c->iters = iters0;
-        }
-        return rc;
+        return start.back_if_gave_up(sync_scalars(c, NSCAL, "iterate sync"));
     }
     double best = INFINITY, res = NAN;
     int64_t done = 0;
     for (;;) {
-        int rc = compute_residual(c, &res);
+        int rc = start.back_if_gave_up(compute_residual(c, &res));
         if (rc) return rc;
         if (!std::isfinite(res)) return fail(c, GABP_ERR_DIVERGED, "residual is not finite");
         if (res <= c->opt.tol) return GABP_OK;
@@ -825,10 +835,11 @@ int gabp_iterate_early_stop(gabp_ctx *c, int max_iters, double damping, double t
     c->err.clear();
     if (stopped_at) *stopped_at = 0;
     // iterations 1 and 2 of this call; the change of iteration 2 is the reference
+    const CallStart start(c);
     int rc = run_iterations(c, 2, damping);
     if (rc) return rc;
     double ref = 0.0, d = 0.0;
-    if ((rc = compute_msg_change(c, &ref))) return rc;
+    if ((rc = start.back_if_gave_up(compute_msg_change(c, &ref)))) return rc;
     if (!std::isfinite(ref)) return fail(c, GABP_ERR_DIVERGED, "message change is not finite");
     int64_t t = 2;
     for (;;) {
@@ -837,7 +848,7 @@ int gabp_iterate_early_stop(gabp_ctx *c, int max_iters, double damping, double t
         if (t + chunk > max_iters) chunk = max_iters - t;
         if ((rc = run_iterations(c, (int)chunk, damping))) return rc;   // checked with the message change
         t += chunk;
-        if ((rc = compute_msg_change(c, &d))) return rc;
+        if ((rc = start.back_if_gave_up(compute_msg_change(c, &d)))) return rc;
         if (!std::isfinite(d)) return fail(c, GABP_ERR_DIVERGED, "message change is not finite");
         if (d < tau * ref) {
             if (stopped_at) *stopped_at = t;
