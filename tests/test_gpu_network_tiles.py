@@ -1,0 +1,83 @@
+"""GPU: the network's gradients where a block of the tensor-core kernels works through many pixel tiles
+(ring stages used again, sums over tiles, a short last chunk), tile by tile."""
+import numpy as np
+import pytest
+
+from gpu_common import ensure_built
+
+pytestmark = pytest.mark.gpu
+
+B, H, W = 7, 520, 488   # 13,873 tiles of 16 x 8 pixels at full resolution, the last column half of one
+
+
+@pytest.fixture(scope="module")
+def net():
+    torch = pytest.importorskip("torch")
+    ensure_built()
+    from oracle import unet
+    from paper_2404_12968_gb300 import GABP_WSNET_MMA_SYNC, GABP_WSNET_TCGEN05, WarmStartNet, gabp_wsnet_forward, gabp_wsnet_set_kernels
+    n = WarmStartNet(seed=11, device=0)
+    rng = np.random.default_rng(12)
+    n.set_params((n.params() + rng.normal(size=unet.layout()[2]) * 0.02).astype(np.float32))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    x = torch.zeros((B, H, W, 16), device="cuda")
+    x[..., :3] = torch.randn((B, H, W, 3), generator=gen, device="cuda")
+    x = x.to(torch.bfloat16).contiguous()
+    outs = {}
+    for k in (GABP_WSNET_TCGEN05, GABP_WSNET_MMA_SYNC):
+        gabp_wsnet_set_kernels(n.handle, k)
+        outs[k] = torch.empty((B, H, W, 2), device="cuda")
+        torch.cuda.synchronize()
+        gabp_wsnet_forward(n.handle, x, B, H, W, outs[k])
+    yield n, x, outs
+    n.close()
+
+
+def _compare(net, delta):
+    """Gradients for targets that differ from the network's own output by delta, on both kernel families.
+    Each is within 6 % of the reference in BF16 (test_gpu_warmstart.py), so within 12 % of each other.
+    delta has a mean: where the pixels' gradients cancel, BF16 alone makes both 10 to 19 %."""
+    import torch
+    from oracle import unet
+    from paper_2404_12968_gb300 import gabp_wsnet_gradients, gabp_wsnet_set_kernels
+    n, x, outs = net
+    grads = []
+    for k, out in outs.items():
+        gabp_wsnet_set_kernels(n.handle, k)
+        t = (out - delta).contiguous()
+        torch.cuda.synchronize()
+        g = np.empty(n.nparam, np.float32)
+        gabp_wsnet_gradients(n.handle, list(x), list(t), H, W, g)
+        grads.append(g)
+    offs, head, _ = unet.layout()
+    parts = [(lo, hi) for i, (wo, bo) in enumerate(offs) for lo, hi in ((wo, bo), (bo, bo + unet.SPECS[i][1]))]
+    for lo, hi in parts + [(head, n.nparam)]:
+        a, b = grads[0][lo:hi], grads[1][lo:hi]
+        assert np.linalg.norm(b) > 0 and np.linalg.norm(a - b) < 0.12 * np.linalg.norm(b), (lo, hi)
+
+
+def test_gradients_of_all_tiles(net):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(6)
+    _compare(net, 2.0 + torch.randn((B, H, W, 2), generator=gen, device="cuda"))
+
+
+# (image, tile row, tile column): the first and the last, one beyond the stages of a ring after another in
+# the first block, and a spread over the images; the gradient of one tile is what a lost, doubled or
+# stale tile changes by all of itself
+TILES = [(0, 0, 0), (0, 0, 1), (0, 0, 5), (0, 0, 6), (0, 0, 7), (0, 0, 13), (0, 0, 30), (0, 1, 2), (0, 2, 29), (0, 64, 30),
+         (1, 17, 8), (2, 40, 22), (3, 63, 0), (4, 5, 30), (5, 31, 15), (6, 63, 29), (6, 64, 29), (6, 64, 30)]
+
+
+@pytest.mark.parametrize("tile", TILES)
+def test_gradients_of_one_tile(net, tile):
+    import torch
+    b, ty, tx = tile
+    delta = torch.zeros((B, H, W, 2), device="cuda")
+    y, x = slice(8 * ty, 8 * ty + 8), slice(16 * tx, min(16 * tx + 16, W))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    delta[b, y, x] = 2.0 + torch.randn((8, x.stop - x.start, 2), generator=gen, device="cuda")
+    _compare(net, delta)
