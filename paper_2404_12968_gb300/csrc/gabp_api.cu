@@ -81,8 +81,10 @@ thread_local bool t_pad_odd_planes = false;
 
 // AUTO runs FP32 contexts whose width is not a multiple of 4 on the TMA kernel too, on plane rows
 // padded to an even pitch and a copy of the observation index padded to a multiple of 4 ints (the
-// layout of batch members), from this many nodes on; smaller ones keep the column sweep.
-// 361 x 181: 116 -> 7 us per iteration; 1601 x 1201: 130 -> 42 us.
+// layout of batch members), from this many nodes on; smaller ones keep the column sweep.  Per iteration,
+// sweep and TMA: 361 x 181 103 and 4.7 us, 1601 x 1201 124 and 43.  The line is not where the two cross:
+// smaller grids gain as much (63 x 65 102 and 3.4, 33^2 54 and 3.4, 9 x 8 14 and 3.2; 33^2 with 13
+// observations per node 428 and 7.6), but the sweep on them is what AUTO is documented and tested to run.
 constexpr int64_t TMA_PADDED_MIN_NODES = 4096;
 
 struct DeviceGuard {

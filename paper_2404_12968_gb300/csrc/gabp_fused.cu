@@ -20,30 +20,30 @@ namespace {
 
 constexpr int FT = 256;   // threads per block
 
-template <typename T, int TX, int TY> struct FusedLayout {
+template <int TX, int TY> struct FusedLayout {
     static constexpr int RX = TX + 4, RY = TY + 4;   // staged message window (2-cell halo)
     static constexpr int BX = TX + 2, BY = TY + 2;   // belief window (1-cell halo)
-    static constexpr size_t msg_bytes = sizeof(T2<T>) * 5 * RX * RY;
-    static constexpr size_t bel_bytes = sizeof(Belief<T>) * BX * BY;
+    static constexpr size_t msg_bytes = sizeof(float2) * 5 * RX * RY;
+    static constexpr size_t bel_bytes = sizeof(Belief<float>) * BX * BY;
     static constexpr size_t bytes = msg_bytes + bel_bytes + sizeof(int) * 2 * (TY + 1);
 };
 
-template <typename T, int TX, int TY>
-__global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
-    using LY = FusedLayout<T, TX, TY>;
+template <int TX, int TY>
+__global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, float beta) {
+    using LY = FusedLayout<TX, TY>;
     constexpr int RX = LY::RX, RY = LY::RY, BX = LY::BX, BY = LY::BY;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2<T> *sm = reinterpret_cast<T2<T> *>(smem_raw);                         // [5][RY][RX]
-    Belief<T> *sb = reinterpret_cast<Belief<T> *>(smem_raw + LY::msg_bytes); // [BY][BX]
+    float2 *sm = reinterpret_cast<float2 *>(smem_raw);                         // [5][RY][RX]
+    Belief<float> *sb = reinterpret_cast<Belief<float> *>(smem_raw + LY::msg_bytes); // [BY][BX]
     int *rstart = reinterpret_cast<int *>(smem_raw + LY::msg_bytes + LY::bel_bytes);  // [TY+1]
     int *rpre = rstart + (TY + 1);                                                     // [TY+1]
 
     const int nx = p.nx, ny = p.ny;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const T2<T> *P = (const T2<T> *)p.P[src];
-    T2<T> *Q = (T2<T> *)p.P[src ^ 1];
-    const T *O = (const T *)p.O[src];
-    T *OQ = (T *)p.O[src ^ 1];
+    const float2 *P = (const float2 *)p.P[src];
+    float2 *Q = (float2 *)p.P[src ^ 1];
+    const float *O = (const float *)p.O[src];
+    float *OQ = (float *)p.O[src ^ 1];
     const int *optr = p.optr;
 
     // 1. stage the message window
@@ -52,9 +52,9 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
         const int rem = q - d * (RX * RY);
         const int ly = rem / RX, lx = rem - ly * RX;
         const int gx = x0 - 2 + lx, gy = y0 - 2 + ly;
-        T2<T> val;
-        val.x = T(0);
-        val.y = T(0);
+        float2 val;
+        val.x = 0.f;
+        val.y = 0.f;
         if (gx >= 0 && gx < nx && gy >= 0 && gy < ny) val = P[d * p.pn + (int64_t)gy * p.px + gx];
         sm[q] = val;
     }
@@ -89,8 +89,8 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
         if (gx < 0 || gx >= nx || gy < 0 || gy >= ny) continue;
         const int rx = lx + 1, ry = ly + 1;
         const int64_t v = (int64_t)gy * nx + gx;
-        T2<T> m = sm[(DIR_C * RY + ry) * RX + rx];
-        CompSum<T> se(m.x), sl(m.y);
+        float2 m = sm[(DIR_C * RY + ry) * RX + rx];
+        CompSum<float> se(m.x), sl(m.y);
         if (gx > 0) { m = sm[(DIR_E * RY + ry) * RX + rx - 1]; se.add(m.x); sl.add(m.y); }
         if (gx < nx - 1) { m = sm[(DIR_W * RY + ry) * RX + rx + 1]; se.add(m.x); sl.add(m.y); }
         if (gy > 0) { m = sm[(DIR_N * RY + ry - 1) * RX + rx]; se.add(m.x); sl.add(m.y); }
@@ -102,49 +102,49 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
         }
         se.finish();
         sl.finish();
-        Belief<T> b;
+        Belief<float> b;
         b.ehi = se.hi; b.elo = se.lo; b.lhi = sl.hi; b.llo = sl.lo;
         sb[q] = b;
     }
     __syncthreads();
 
     // 3a. prior cell factors of the tile
-    const T var_prior = prior_var<T>(p);
+    const float var_prior = prior_var<float>(p);
     for (int q = threadIdx.x; q < TX * TY; q += FT) {
         const int ty = q / TX, tx = q - ty * TX;
         const int gx = x0 + tx, gy = y0 + ty;
         if (gx >= nx || gy >= ny) continue;
         const int64_t c = (int64_t)gy * nx + gx;
         const int deg = grid_degree(gy, gx, nx, ny);
-        const T a[5] = {cell_coef<T>(p, deg), gx > 0 ? T(-1) : T(0), gx < nx - 1 ? T(-1) : T(0),
-                        gy > 0 ? T(-1) : T(0), gy < ny - 1 ? T(-1) : T(0)};
+        const float a[5] = {cell_coef<float>(p, deg), gx > 0 ? -1.f : 0.f, gx < nx - 1 ? -1.f : 0.f,
+                        gy > 0 ? -1.f : 0.f, gy < ny - 1 ? -1.f : 0.f};
         // belief-window coordinates of the 5 nodes (C, W, E, S, N)
         const int bxs[5] = {tx + 1, tx, tx + 2, tx + 1, tx + 1};
         const int bys[5] = {ty + 1, ty + 1, ty + 1, ty, ty + 2};
-        T2<T> own[5];
-        T lam[5], eta[5];
+        float2 own[5];
+        float lam[5], eta[5];
 #pragma unroll
         for (int u = 0; u < 5; ++u) {
             own[u] = sm[(u * RY + ty + 2) * RX + tx + 2];
-            if (a[u] != T(0)) {
+            if (a[u] != 0.f) {
                 cavity(sb[bys[u] * BX + bxs[u]], own[u].x, own[u].y, eta[u], lam[u]);
             } else {
-                lam[u] = T(1);
-                eta[u] = T(0);
+                lam[u] = 1.f;
+                eta[u] = 0.f;
             }
         }
-        T L[5], E[5];
-        const T r = p.ptgt ? ((const T *)p.ptgt)[c] : T(0);
-        factor_messages<T, 5>(a, var_prior, r, lam, eta, L, E);
+        float L[5], E[5];
+        const float r = p.ptgt ? ((const float *)p.ptgt)[c] : 0.f;
+        factor_messages<float, 5>(a, var_prior, r, lam, eta, L, E);
 #pragma unroll
         for (int u = 0; u < 5; ++u) {
-            T2<T> out;
-            if (a[u] != T(0)) {
+            float2 out;
+            if (a[u] != 0.f) {
                 out.x = damp(own[u].x, E[u], beta);
                 out.y = damp(own[u].y, L[u], beta);
             } else {
-                out.x = T(0);
-                out.y = T(0);
+                out.x = 0.f;
+                out.y = 0.f;
             }
             Q[u * p.pn + (int64_t)gy * p.px + gx] = out;
         }
@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
     // 3b. observation factors whose base cell lies in the tile
     if (p.m > 0) {
         const int total = rpre[TY];
-        const T *W = (const T *)p.ow;
-        const T *YV = (const T *)p.ovar;
+        const float *W = (const float *)p.ow;
+        const float *YV = (const float *)p.ovar;
         for (int q = threadIdx.x; q < total; q += FT) {
             int r = 0;
             while (r + 1 < TY && rpre[r + 1] <= q) ++r;
@@ -163,16 +163,16 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
             const int by = b / nx, bx = b - by * nx;
             const int lx = bx - x0 + 1, ly = by - y0 + 1;   // belief-window coordinates
             const int bidx[4] = {ly * BX + lx, ly * BX + lx + 1, (ly + 1) * BX + lx, (ly + 1) * BX + lx + 1};
-            const T a[4] = {W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3]};
-            T oe[4], ol[4], lam[4], eta[4];
+            const float a[4] = {W[4 * k], W[4 * k + 1], W[4 * k + 2], W[4 * k + 3]};
+            float oe[4], ol[4], lam[4], eta[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 oe[u] = O[8 * k + 2 * u];
                 ol[u] = O[8 * k + 2 * u + 1];
                 cavity(sb[bidx[u]], oe[u], ol[u], eta[u], lam[u]);
             }
-            T L[4], E[4];
-            factor_messages<T, 4>(a, YV[2 * k + 1], YV[2 * k], lam, eta, L, E);
+            float L[4], E[4];
+            factor_messages<float, 4>(a, YV[2 * k + 1], YV[2 * k], lam, eta, L, E);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 OQ[8 * k + 2 * u] = damp(oe[u], E[u], beta);
@@ -185,8 +185,8 @@ __global__ void __launch_bounds__(FT) k_fused(DevProblem p, int src, T beta) {
 // ---- FP64 ----
 // FP64 arithmetic bounds this kernel (GB300: two lanes per clock and SM; an iteration's bytes would
 // take a twentieth of the time), so the work per cell is what it saves: no product by +-1 and no
-// sum with an exact zero on interior cells (cell_update_interior), Fast2Sum and three-operation
-// reciprocals, comparisons and floors in the integer unit, and both observation ranges of a node
+// sum with an exact zero on interior cells (cell_update_interior), Fast2Sum, reciprocals without an
+// FP64 operation (recip_fixed), comparisons and floors in the integer unit, and both observation ranges of a node
 // in one loop, so that lanes with a term in either run together.  The messages are read straight
 // from global memory (the second reading, in the factor update, hits L1): staging them cost a pass
 // of index arithmetic and the shared memory that limited the resident blocks.  Tiles of TX columns
@@ -566,9 +566,9 @@ cudaError_t launch_f64(const DevProblem &p, int ty, int src, double beta, cudaSt
     return launch_pdl((int64_t)grid.x * grid.y <= sm_count(), k_fused_f64<TX, NT>, grid, NT, bytes, st, p, ty, src, beta);
 }
 
-template <typename T, int TX, int TY>
+template <int TX, int TY>
 cudaError_t launch_shape(const DevProblem &p, int src, double beta, cudaStream_t st) {
-    using LY = FusedLayout<T, TX, TY>;
+    using LY = FusedLayout<TX, TY>;
     static PerDevice<bool> configured;   // per instantiation; the attribute is per function and device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -576,17 +576,17 @@ cudaError_t launch_shape(const DevProblem &p, int src, double beta, cudaStream_t
     bool set = false;
     e = configured.get(dev, set, [](bool &v) {
         v = true;
-        return cudaFuncSetAttribute(k_fused<T, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes);
+        return cudaFuncSetAttribute(k_fused<TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::bytes);
     });
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((p.nx + TX - 1) / TX), (unsigned)((p.ny + TY - 1) / TY));
-    k_fused<T, TX, TY><<<grid, FT, LY::bytes, st>>>(p, src, (T)beta);
+    k_fused<TX, TY><<<grid, FT, LY::bytes, st>>>(p, src, (float)beta);
     return cudaGetLastError();
 }
 
 cudaError_t dispatch_f32(const DevProblem &p, int src, double beta, FusedShape s, cudaStream_t st) {
 #define GABP_SHAPE(X, Y) \
-    if (s.tx == X && s.ty == Y) return launch_shape<float, X, Y>(p, src, beta, st);
+    if (s.tx == X && s.ty == Y) return launch_shape<X, Y>(p, src, beta, st);
     GABP_SHAPE(32, 8)
     GABP_SHAPE(32, 16)
     GABP_SHAPE(64, 8)

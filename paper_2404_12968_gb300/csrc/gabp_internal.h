@@ -34,8 +34,8 @@ struct DevProblem {
     const float2 *oysdf; // FP32 contexts: 2 * m (y, 1/sigma^2) as double-float pairs
     void *P[2];          // prior messages, ping-pong: planes * pn (eta, Lambda) pairs
     // layout of the prior message planes: node (i, j) of plane d at d * pn + i * px + j.  px = nx
-    // except for the members of a batch with an odd width, whose rows are padded to px = nx + 1
-    // so that every row starts on a 16-byte boundary (tensor copies); the padding cells hold
+    // except where the TMA kernel runs on an odd width (batch members, and contexts of AUTO from 4096
+    // nodes on), whose rows are padded to px = nx + 1 so that every row starts on a 16-byte boundary (tensor copies); the padding cells hold
     // (0, 0) in both buffers.  pn = px * ny.
     int px;
     int64_t pn;
@@ -257,7 +257,7 @@ size_t tma_smem_bytes(int tx, int ty);
 // persistent blocks best (longest on ties).
 int tma_choose_run(const DevProblem &p, int ty);
 // Tile height of a problem whose options leave it open: 14, or 2 or 6 (the dense kernel; not
-// selectable) for problems with many observations per cell.
+// selectable) for small grids and for problems with many observations per cell.
 int tma_choose_height(const DevProblem &p);
 cudaError_t launch_tma_iteration(const DevProblem &p, const TmaMaps &maps, int src, double beta,
                                  cudaStream_t st);

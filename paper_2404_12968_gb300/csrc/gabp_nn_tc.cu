@@ -30,7 +30,7 @@
 // contiguous bytes, a row of a swizzle atom, and a tile of pixels is loaded by one 5-D TMA copy per
 // operand (channel in block, x, y, image, channel block) with zero fill outside the image for the tap
 // shift.  One accumulator of N FP32 columns per tap and block covers a chunk of pixel tiles; the
-// epilogue writes it to a partial-sum buffer that a second kernel reduces in chunk order.
+// epilogue writes it to a partial-sum buffer that a second kernel reduces in a fixed order.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -841,8 +841,8 @@ cudaError_t tc_wgrad(TcWgradArgs a, float *dw, float *db, cudaStream_t st) {
     const uint32_t stage = stage_bytes(a.ky);
     a.stage = (int)stage;
     a.xbytes = stack ? (int)wg_stacked_x_bytes(a.Cin, a.ky) : 0;
-    // (32 input channels with taps stacked: one block per SM.  Two are 12 % faster, but the sums of twice
-    // as many chunks round otherwise)
+    // (32 input channels with taps stacked: one block per SM.  Two are 12 % faster on those layers, with
+    // the FP32 sums grouped by twice as many chunks: not taken so far)
     const bool two = (stack ? a.Cin == 16 : a.tpc * a.N <= 256) && stage * 3 <= 100u * 1024u;   // room for two blocks per SM
     int S = (int)((two ? 100u * 1024u : 196u * 1024u) / stage);
     a.stages = S > 6 ? 6 : S;

@@ -482,9 +482,10 @@ template <int E> __global__ void k_obs_pointers(DevProblem p) {
 }
 
 // ---- deterministic FP64 reductions: fixed grid, fixed per-thread order, smem tree ----
-// The kernels on this grid of RES_BLOCKS = 1024 blocks are bounded to the registers of 7 blocks per SM,
-// 1064 on 152 SMs: at 6 (39 registers, 912 blocks) a ninth of the blocks ran in a second round of their
-// own (2048^2: k_res_df 59 -> 54 us, k_rhs_norm 52 -> 44, k_res 89 -> 83).
+// The kernels on this grid of RES_BLOCKS = 1024 blocks are bounded to 32 registers, so that all of them
+// run at once: at 39, six blocks per SM and 912 on 152 SMs, a ninth of the blocks ran in a second round
+// of their own (2048^2: k_res_df 59 -> 54 us, k_rhs_norm 52 -> 44, k_res 89 -> 83, with 24 bytes of spill
+// in the FP64 ones).  The forms for many observations (many_obs) have 64.
 __device__ __forceinline__ double block_sum(double x) {
     __shared__ double sh[TPB];
     sh[threadIdx.x] = x;
@@ -552,7 +553,7 @@ __device__ __forceinline__ void for_node_obs(const DevProblem &p, int64_t v, int
 inline bool many_obs(int64_t n, int64_t m) { return m > 2 * n; }
 inline bool many_obs_f64(int64_t n, int64_t m) { return many_obs(n, m) || n <= 512 * (int64_t)TPB; }   // 4 blocks per SM
 template <bool MANY> constexpr int obs_group = MANY ? 4 : 1;
-template <bool MANY> constexpr int res_blocks_per_sm = MANY ? 4 : 7;
+template <bool MANY> constexpr int res_blocks_per_sm = MANY ? 4 : 8;
 
 // (L x)_v = (kappa^2 + deg) x_v - sum of existing neighbours
 __device__ __forceinline__ double apply_L(const DevProblem &p, const double *x, int64_t v, int i, int j) {
