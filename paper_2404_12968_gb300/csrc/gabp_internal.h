@@ -35,8 +35,8 @@ struct DevProblem {
     void *P[2];          // prior messages, ping-pong: planes * pn (eta, Lambda) pairs
     // layout of the prior message planes: node (i, j) of plane d at d * pn + i * px + j.  px = nx
     // except where the TMA kernel runs on an odd width (batch members, and contexts of AUTO from 4096
-    // nodes on), whose rows are padded to px = nx + 1 so that every row starts on a 16-byte boundary (tensor copies); the padding cells hold
-    // (0, 0) in both buffers.  pn = px * ny.
+    // nodes on), whose rows are padded to px = nx + 1 so that every row starts on a 16-byte boundary
+    // (tensor copies); the padding cells hold (0, 0) in both buffers.  pn = px * ny.
     int px;
     int64_t pn;
     void *O[2];          // observation messages, ping-pong: per observation (eta, Lambda) of corners 0..3, interleaved
