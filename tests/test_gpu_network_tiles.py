@@ -7,7 +7,7 @@ from gpu_common import ensure_built
 
 pytestmark = pytest.mark.gpu
 
-B, H, W = 7, 520, 488   # 13,873 tiles of 16 x 8 pixels at full resolution, the last column half of one
+B, H, W = 7, 520, 488   # 14,105 tiles of 16 x 8 pixels at full resolution, the last column half of one
 
 
 @pytest.fixture(scope="module")
